@@ -111,6 +111,11 @@ enum { GRTX_TRAVERSAL_CHECKPOINT = 0, /* resume from checkpointed nodes + evicti
  * top of the paper's 512-2048); a ray with more hits is traced with k-buffer rounds
  * restarted from the root instead (same result, counted in fallbacks), and k must still be
  * one of the valid sizes.
+ * With GRTX_TRAVERSAL_CHECKPOINT the k-buffer bounds a round only once min(ckpt_capacity,
+ * evict_capacity) / 4 hits wait on the eviction list, and a ray drops whatever lies behind the
+ * depth at which the hits it holds already end it (their product of 1 - alpha below T_min).
+ * Calls without optional outputs walk the first round of a sphere-form scene for a tile of 32 rays
+ * at once, without checkpoints; the counters of grtx_stats are those of each ray's own rounds.
  * traversal: GRTX_TRAVERSAL_*, for either form: {sphere, proxy} x {checkpoint, restart} are the
  * paper's GRTX, GRTX-HW only (proxy + checkpoint), GRTX-SW only (sphere + restart) and the
  * baseline (proxy + restart) of Sec. V-B.

@@ -455,6 +455,10 @@ extern "C" GRTX_API int grtx_server_create(grtx_scene *const *scenes, int n_scen
     a.ckpt_cap = (int)C;
     a.evict_cap = (int)E;
     a.packet_stack = p->packet_stack > 0 ? std::min(p->packet_stack, kPacketStack) : kPacketStack;
+    set_window(a);
+    int64_t n_most = 0;
+    for (int i = 0; i < n_scenes; ++i) n_most = std::max<int64_t>(n_most, scenes[i]->n);
+    set_codes(a, FORM_SPHERE, false, n_most);
     int n_slots = v->blocks * 128;
     size_t ws = (size_t)blocks * per_block;
     v->lost_cap = (unsigned)blocks * (kBlock / 32);

@@ -213,6 +213,7 @@ int setup(grtx_scene *sc, const grtx_camera *cam, const grtx_params *p, TraceArg
                  : (p->traversal == GRTX_TRAVERSAL_SINGLE ? GRTX_DEFAULT_SINGLE_CAPACITY : GRTX_DEFAULT_CKPT_CAPACITY);
     a.evict_cap = p->evict_capacity > 0 ? p->evict_capacity : GRTX_DEFAULT_EVICT_CAPACITY;
     a.packet_stack = p->packet_stack > 0 ? std::min(p->packet_stack, kPacketStack) : kPacketStack;
+    set_window(a);
     return GRTX_OK;
 }
 
@@ -220,6 +221,7 @@ int run(grtx_scene *sc, TraceArgs &a, int k, bool instr, int pass, unsigned *que
 {
     int form = kernel_form(sc->form, wide, sc->bvh_quant != 0);
     bool single = a.traversal == GRTX_TRAVERSAL_SINGLE && pass == PASS_FWD;
+    set_codes(a, pass == PASS_BWD ? (int)FORM_SPHERE : form, instr, sc->n_valid);
     int bps = 0;
     int occ = single ? trace_single_occupancy(form, instr, &bps) : occupancy_k(k, form, instr, pass, &bps);
     if (occ != GRTX_OK || bps <= 0) return grtx_fail(GRTX_ERR_CUDA, "occupancy query failed");
@@ -449,6 +451,7 @@ extern "C" GRTX_API int grtx_trace_forward_batch(grtx_scene *sc, const grtx_came
     if (!set_list_offsets(a, 2 * C + E))
         return grtx_fail(GRTX_ERR_INVALID_ARG, "checkpoint/eviction capacities too large for the resident ray slots");
     a.discard = lists_discardable(a);
+    set_codes(a, FORM_SPHERE, false, sc->n_valid);
     ServeSeg *d = nullptr;      // the records, then the begins array
     st = grtx_malloc_async((void **)&d, (sizeof(ServeSeg) + sizeof(unsigned)) * n_cams, s);
     if (st) return st;

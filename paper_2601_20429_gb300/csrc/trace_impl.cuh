@@ -50,6 +50,9 @@ struct TraceArgs {
     float bg0, bg1, bg2;
     int ckpt_cap, evict_cap;
     int packet_stack;            // warp-stack entries a packet may use (1..kPacketStack)
+    int window;                  // first round of a checkpointed ray: hits kept past the k-buffer (see Cut)
+    float p_stop;                // product of (1 - alpha) below which a ray is known to terminate (see Cut)
+    int id_shift;                // bits below the leaf slot in a list entry of windowed rays: kCodeBits or 0
     // per-slot workspace, interleaved [entry][slot]; the kernels address every list entry as
     // ck0[offset] with a 32-bit offset (ck1 = ck0 + ck1_off, ev = ck0 + ev_off; the host checks
     // that the whole workspace has fewer than 2^31 entries)
@@ -311,6 +314,47 @@ struct KBuf {
     }
 };
 
+// How far a checkpointed ray still has to look. P is the product of (1 - alpha) over every hit
+// it has collected (blended, in the k-buffer or on the eviction list; each hit is collected
+// once) and far their farthest depth. Once P is below p_stop, just under T_min, the ray ends at
+// or before `far`: hits and nodes beyond it can never be blended, and are dropped, not
+// checkpointed. (p_stop = 0.98 T_min: P and the blended T round the same factors in different
+// orders, each product of n factors within n 2^-23 of the exact one, and a ray's lists hold
+// fewer than 2^17 hits.)
+constexpr int kCodeBits = 8;
+
+// -log2(q) of a hit's q = 1 - alpha in 8 bits, rounded down: exponents 2^-20 to 2^11 with 3 bits of
+// mantissa, 0 for anything below. Scenes of fewer than 2^24 leaf slots keep it below the slot in a
+// ray's list entries (slot << 8 | code, which orders as the slot does; see squeeze).
+__device__ __forceinline__ uint32_t opacity_code(float q)
+{
+    const int c = (int)((__float_as_uint(__log2f(q)) & 0x7fffffffu) >> 20) - (107 << 3);
+    return (uint32_t)min(max(c, 0), 255);
+}
+__device__ __forceinline__ float opacity_of_code(uint32_t c)
+{
+    return c ? __uint_as_float((c + (107u << 3)) << 20) : 0.f;
+}
+
+struct Cut {
+    float P, far;
+    __device__ __forceinline__ void clear()
+    {
+        P = 1.0f;
+        far = 0.0f;
+    }
+    __device__ __forceinline__ float top(const TraceArgs &a) const { return P < a.p_stop ? far : GRTX_INF; }
+    // Counts a hit of Gaussian record g (leaf slot gi) and returns the slot as the lists hold it.
+    __device__ __forceinline__ uint32_t add(const TraceArgs &a, const float4 *__restrict__ g, uint32_t gi, float t, float D2)
+    {
+        const float4 r3 = __ldg(g + 3);
+        const float q = 1.0f - fminf(r3.x * exp2f(r3.y * D2), a.alpha_max);
+        P *= q;
+        far = fmaxf(far, t);
+        return a.id_shift ? gi << kCodeBits | opacity_code(q) : gi;
+    }
+};
+
 __device__ __forceinline__ bool key_after(float t, uint32_t i, float Lt, uint32_t Li)
 {
     return t > Lt || (t == Lt && i > Li);
@@ -324,7 +368,8 @@ __device__ __forceinline__ bool key_after(float t, uint32_t i, float Lt, uint32_
 // is widened to 1 + 1e-5 + 4e-6 |o_l|, tested in squared form (no square root). Its t only
 // seeds stage 2, whose Newton step lands on the minimiser from any nearby start, so the
 // quotient is the fast approximate one.
-__device__ __forceinline__ bool sphere_candidate(float4 r0, float4 r1, float4 r2, float3 o, float3 d, float &t)
+__device__ __forceinline__ bool sphere_candidate(float4 r0, float4 r1, float4 r2, float3 o, float3 d, float &t,
+                                                 float &aa)
 {
     float vx = o.x - r0.w, vy = o.y - r1.w, vz = o.z - r2.w;
     float olx = fmaf(r0.x, vx, fmaf(r0.y, vy, r0.z * vz));
@@ -333,7 +378,7 @@ __device__ __forceinline__ bool sphere_candidate(float4 r0, float4 r1, float4 r2
     float dlx = fmaf(r0.x, d.x, fmaf(r0.y, d.y, r0.z * d.z));
     float dly = fmaf(r1.x, d.x, fmaf(r1.y, d.y, r1.z * d.z));
     float dlz = fmaf(r2.x, d.x, fmaf(r2.y, d.y, r2.z * d.z));
-    float aa = fmaf(dlx, dlx, fmaf(dly, dly, dlz * dlz));
+    aa = fmaf(dlx, dlx, fmaf(dly, dly, dlz * dlz));
     float bb = fmaf(olx, dlx, fmaf(oly, dly, olz * dlz));
     t = __fdividef(-bb, aa);
     float px = fmaf(t, dlx, olx), py = fmaf(t, dly, oly), pz = fmaf(t, dlz, olz);
@@ -341,6 +386,20 @@ __device__ __forceinline__ bool sphere_candidate(float4 r0, float4 r1, float4 r2
     float oo = fmaf(olx, olx, fmaf(oly, oly, olz * olz));
     float ex = D2 - (1.0f + 1e-5f);
     return ex <= 0.0f || ex * ex <= 1.6e-11f * oo;    // ex <= 4e-6 sqrt(oo)
+}
+__device__ __forceinline__ bool sphere_candidate(float4 r0, float4 r1, float4 r2, float3 o, float3 d, float &t)
+{
+    float aa;
+    return sphere_candidate(r0, r1, r2, o, d, t, aa);
+}
+
+// Whether the depth t of sphere_candidate may stand for an exact depth in (lo, hi]. Its error is the
+// rounding of o - mu taken through A, at most a few ulp of |t| and of the half chord 1 / |d_l| times
+// the Gaussian's aspect ratio: 1 % of both covers ratios up to 10^4.
+__device__ __forceinline__ bool in_range(float t, float aa, float lo, float hi)
+{
+    const float m = 0.01f * (fabsf(t) + rsqrtf(aa));
+    return !(t + m < lo) && !(t - m > hi);
 }
 
 // Error-free a + b = s + e (Knuth's two-sum).
@@ -899,7 +958,7 @@ __device__ __forceinline__ bool trace_round(const TraceArgs &a, const SceneRef &
                                             float inv_len, float tn, float tf,
                                             float Lt, uint32_t Li, bool ckpt, bool from_root,
                                             uint32_t src, int n_src, uint32_t dst, int &n_dst, uint32_t ev,
-                                            int &n_ev, KBuf<K> &kb, Counters &cnt)
+                                            int &n_ev, KBuf<K> &kb, Cut &cut, int window, Counters &cnt)
 {
     if constexpr (FORM == FORM_SPHERE4 || FORM == FORM_SPHERE4Q)
         return trace_round4<K, INSTR, FORM == FORM_SPHERE4Q>(a, sc, o, d, inv, tn, tf, Lt, Li, ckpt, from_root, src,
@@ -910,7 +969,8 @@ __device__ __forceinline__ bool trace_round(const TraceArgs &a, const SceneRef &
     // is visited without re-testing its entry depth, since its children meet the t_max test
     uint32_t stack[GRTX_STACK];
     int sp = 0, si = 0;
-    float tmax = kb.tmax;
+    const bool windowed = FORM != FORM_PROXY && ckpt && a.window > 0;
+    float tmax = windowed ? fminf(kb.n == K && n_ev >= window ? kb.tmax : GRTX_INF, cut.top(a)) : kb.tmax;
     uint32_t ref;
     float te;
     n_dst = 0;
@@ -927,7 +987,7 @@ __device__ __forceinline__ bool trace_round(const TraceArgs &a, const SceneRef &
     }
     for (;;) {
         if (te > tmax) {                              // fails the t_max test
-            if (ckpt) {
+            if (ckpt && !(windowed && te > cut.top(a))) {
                 if (n_dst >= a.ckpt_cap) return false;
                 L[dst + (uint32_t)n_dst * S] = make_uint2(ref, __float_as_uint(te));
                 ++n_dst;
@@ -953,10 +1013,11 @@ __device__ __forceinline__ bool trace_round(const TraceArgs &a, const SceneRef &
             }
             float t, D2, w[3];
             if (touch && sphere_test(sc.geom + 4 * (size_t)gi, o, d, t, D2, w)) {
-                if (D2 <= 1.0f && t > tn && t <= tf && key_after(t, gi, Lt, Li)) {
+                if (D2 <= 1.0f && t > tn && t <= tf && key_after(t, gi, Lt, Li) &&
+                    !(windowed && t > cut.top(a))) {
                     if (FORM != FORM_PROXY || !kb.contains(t, gi)) {
                         float ct = t;
-                        uint32_t ci = gi;
+                        uint32_t ci = windowed ? cut.add(a, sc.geom + 4 * (size_t)gi, gi, t, D2) : gi << a.id_shift;
                         if (kb.insert(ct, ci) && ckpt) {       // any-hit: rejected -> eviction list
                             if (n_ev >= a.evict_cap) return false;
                             L[ev + (uint32_t)n_ev * S] = make_uint2(__float_as_uint(ct), ci);
@@ -964,6 +1025,7 @@ __device__ __forceinline__ bool trace_round(const TraceArgs &a, const SceneRef &
                             if (INSTR) cnt.evictions++;
                         }
                         tmax = kb.tmax;                        // farthest kept key
+                        if (windowed) tmax = fminf(n_ev >= window ? tmax : GRTX_INF, cut.top(a));
                     }
                 }
             }
@@ -993,7 +1055,7 @@ __device__ __forceinline__ bool trace_round(const TraceArgs &a, const SceneRef &
                 ref = near0 ? c0 : c1;
                 te = near0 ? e0 : e1;
                 if (far_t > tmax) {
-                    if (ckpt) {
+                    if (ckpt && !(windowed && far_t > cut.top(a))) {
                         if (n_dst >= a.ckpt_cap) return false;
                         L[dst + (uint32_t)n_dst * S] = make_uint2(far_ref, __float_as_uint(far_t));
                         ++n_dst;
@@ -1044,12 +1106,13 @@ __device__ __forceinline__ bool trace_round(const TraceArgs &a, const SceneRef &
 // round from the root on its own, as after any capacity overflow in trace_ray.
 // ------------------------------------------------------------------------------------------
 constexpr int kPacketStack = GRTX_PACKET_STACK;
+constexpr int kWarpShared = 84;
 
 template <int K, int FORM, bool INSTR>
 __device__ __forceinline__ bool packet_round(const TraceArgs &a, const SceneRef &sc, bool valid, uint4 *pst, float3 o,
                                              float3 d, float3 inv, float inv_len, float tn, float tf, float Lt,
                                              uint32_t Li, bool ckpt, uint32_t dst, int &n_dst,
-                                             uint32_t ev, int &n_ev, KBuf<K> &kb, Counters &cnt,
+                                             uint32_t ev, int &n_ev, KBuf<K> &kb, Cut &cut, Counters &cnt,
                                              bool &lane_ok)
 {
     if constexpr (FORM == FORM_SPHERE4 || FORM == FORM_SPHERE4Q)
@@ -1059,7 +1122,9 @@ __device__ __forceinline__ bool packet_round(const TraceArgs &a, const SceneRef 
     const uint32_t S = (uint32_t)a.n_slots;
     uint2 *__restrict__ const L = a.ck0;      // lists: dst and ev are entry offsets into L
     const int lane = threadIdx.x & 31;
+    const bool windowed = FORM != FORM_PROXY && ckpt && a.window > 0;
     float tmax = kb.tmax;
+    bool cutting = !windowed;                           // (warp-uniform) some lane has a finite t_max
     n_dst = 0;
     n_ev = 0;
     lane_ok = true;
@@ -1071,7 +1136,8 @@ __device__ __forceinline__ bool packet_round(const TraceArgs &a, const SceneRef 
     bool have_te = true;
     for (;;) {
         bool in = (m >> lane) & 1u;
-        if (!have_te && in) {                           // a popped node: entry from the parent's box
+        if (!have_te && !cutting) te = tn;              // no lane would fail the t_max test
+        if (!have_te && cutting && in) {                // a popped node: entry from the parent's box
             const float4 *pn = sc.nodes + 4 * (size_t)parent;
             float x;
             if (slot == 0u) {
@@ -1084,7 +1150,7 @@ __device__ __forceinline__ bool packet_round(const TraceArgs &a, const SceneRef 
             if (FORM == FORM_PROXY) te = fmaf(-(slot == 0u ? __ldg(pn + 3).z : __ldg(pn + 3).w), inv_len, te);
         }
         bool go = in && lane_ok && !(te > tmax);
-        if (in && lane_ok && te > tmax && ckpt) {       // fails the t_max test: checkpoint it
+        if (in && lane_ok && te > tmax && ckpt && !(windowed && te > cut.top(a))) {   // fails the t_max test: checkpoint it
             if (n_dst >= a.ckpt_cap) {
                 lane_ok = false;
             } else {
@@ -1116,9 +1182,10 @@ __device__ __forceinline__ bool packet_round(const TraceArgs &a, const SceneRef 
                     }
                     float t, D2, w[3];
                     if (touch && sphere_test(sc.geom + 4 * (size_t)gi, o, d, t, D2, w) && D2 <= 1.0f && t > tn &&
-                        t <= tf && key_after(t, gi, Lt, Li) && (FORM != FORM_PROXY || !kb.contains(t, gi))) {
+                        t <= tf && key_after(t, gi, Lt, Li) && (FORM != FORM_PROXY || !kb.contains(t, gi)) &&
+                        !(windowed && t > cut.top(a))) {
                         float ct = t;
-                        uint32_t ci = gi;
+                        uint32_t ci = windowed ? cut.add(a, sc.geom + 4 * (size_t)gi, gi, t, D2) : gi << a.id_shift;
                         if (kb.insert(ct, ci) && ckpt) {
                             if (n_ev >= a.evict_cap) {
                                 lane_ok = false;
@@ -1129,8 +1196,10 @@ __device__ __forceinline__ bool packet_round(const TraceArgs &a, const SceneRef 
                             }
                         }
                         tmax = kb.tmax;
+                        if (windowed) tmax = fminf(n_ev >= a.window ? tmax : GRTX_INF, cut.top(a));
                     }
                 }
+                if (!cutting) cutting = __any_sync(full, tmax < GRTX_INF);
             } else {
                 const float4 *nd = sc.nodes + 4 * (size_t)ref;
                 float4 n0 = __ldg(nd), n1 = __ldg(nd + 1), n2 = __ldg(nd + 2), n3 = __ldg(nd + 3);
@@ -1195,6 +1264,252 @@ __device__ __forceinline__ bool packet_round(const TraceArgs &a, const SceneRef 
         }
     }
     return true;
+}
+
+// ------------------------------------------------------------------------------------------
+// The first round of a warp's rays over sphere leaves, walked for the tile instead of for each
+// ray. The warp bounds its rays by the box of their origins and the box of their directions, and
+// each lane takes one pending node and tests the node's two child boxes against that bundle, so
+// that one step expands up to 32 nodes. Leaves are gathered and tested in groups of 32: first
+// every ray filters all 32 (one broadcast record load each), which gives each lane a mask of its
+// candidates; then each lane takes its own candidates one after another through the exact test.
+// The k-buffer, eviction list and Cut of each ray are those of trace_round; there are no
+// checkpoints (a ray whose eviction list is too small leaves the walk and takes trace_round).
+//
+// Why: a packet that tests one node at a time for 32 rays is a chain of about 340 node steps, 150
+// pops and 130 leaf steps a tile on the 1M surface frame, and its exact tests run with a quarter
+// of the lanes. The walk takes 27 steps, 145 filters and 51 exact tests with 23 lanes each:
+// 3.3 G instead of 7.8 G warp instructions a frame. 1920x1080, k = 16: 9.8 ms with packets and
+// per-ray later rounds, 6.8 ms with packets bounded by opacity (Cut), 3.9 ms with the walk. What
+// bounds it now: instruction issue (69 % of the slots) and the L1 pipe (70 %: each lane gathers
+// its own records and SH coefficients).
+// Groups of 8 or 16 rays with a stack each took 7.9 and 4.7 ms against 4.0 for one of 32.
+// ------------------------------------------------------------------------------------------
+// The stack keeps kWalkReserve entries for walking one node at a time: past kWalkStack -
+// kWalkReserve pending nodes a step takes the top one only, as a depth-first walk does.
+constexpr int kWalkStack = 192, kWalkReserve = 48, kWalkLeaves = 128;
+
+struct __align__(16) WalkShared {
+    uint32_t stack[kWalkStack];  // pending nodes
+    uint32_t leaf[kWalkLeaves];  // gathered leaves
+    float c[12];                 // per axis: origin max, 1 / direction max, origin min, 1 / direction min
+};
+
+__device__ __forceinline__ float warp_min(float v)
+{
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, off));
+    return v;
+}
+__device__ __forceinline__ float warp_max(float v)
+{
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
+    return v;
+}
+
+// One axis of the bundle test. A ray of the bundle is inside [lo, hi] on this axis at depth t only
+// if lo <= o_max + t d_max and hi >= o_min + t d_min; each condition bounds t from below or from
+// above, by the sign of its direction bound (c[1], c[3] hold the reciprocals).
+__device__ __forceinline__ void bundle_axis(const float *c, float lo, float hi, float &e, float &x)
+{
+    const float ra = c[1], rb = c[3];
+    const float ta = (lo - c[0]) * ra, tb = (hi - c[2]) * rb;
+    if (ra > 0.f) e = fmaxf(e, ta); else x = fminf(x, ta);
+    if (rb > 0.f) x = fminf(x, tb); else e = fmaxf(e, tb);
+}
+
+// Shortens a ray's eviction list (n entries, row stride S) in the walk. Where the k-buffer and the
+// entries up to the list's mean depth m already hold the opacity at which the ray ends (need, in
+// bits, from the entries' codes), nothing behind m can be blended: m becomes the ray's end (end =
+// true). Otherwise, with full set, m becomes the limit of this round (the ray's later rounds start
+// behind it, see trace_ray). Either way the entries behind m are dropped. Returns m, or +inf where
+// the list stays as it is.
+template <int K>
+static __device__ __noinline__ float squeeze(uint2 *L, uint32_t S, int n, int &kept, const float *kt, const uint32_t *ki,
+                                             float need, bool full, bool &end)
+{
+    float sum = 0.f;
+#pragma unroll 4
+    for (int e = 0; e < n; ++e) sum += __uint_as_float(L[(uint32_t)e * S].x);
+    const float m = fmaxf(sum / (float)n, kt[(K - 1) * kBlock]);       // entries in the k-buffer stay within it
+    float bits = 0.f;
+#pragma unroll
+    for (int j = 0; j < K; ++j) bits += opacity_of_code(ki[j * kBlock] & ((1u << kCodeBits) - 1u));
+#pragma unroll 4
+    for (int e = 0; e < n; ++e) {
+        const uint2 v = L[(uint32_t)e * S];
+        if (!(__uint_as_float(v.x) > m)) bits += opacity_of_code(v.y & ((1u << kCodeBits) - 1u));
+    }
+    end = bits > need;
+    kept = n;
+    if (!end && !full) return GRTX_INF;
+    int k = 0;
+    for (int e = 0; e < n; ++e) {
+        const uint2 v = L[(uint32_t)e * S];
+        if (!(__uint_as_float(v.x) > m)) {
+            L[(uint32_t)k * S] = v;
+            ++k;
+        }
+    }
+    kept = k;
+    return m;
+}
+
+constexpr int kSqueeze = 64;     // entries a list may grow by before it is squeezed
+// Work (in leaf tests; a step counts as 4) after which a walk with fewer than one candidate per
+// four is given up: its rays share almost nothing, and each traces the round on its own.
+constexpr int kWalkTrial = 512;
+
+// Walks the bundles of a warp's rays. lane_ok is false for a ray that must trace the round on its
+// own: its eviction list was too small, or its bundle was left (too little stack, too little shared).
+template <int K>
+__device__ __forceinline__ void tile_walk(const TraceArgs &a, const SceneRef &sc, bool valid, WalkShared &w, float3 o,
+                                          float3 d, float tn, float tf, uint32_t ev, int &n_ev, KBuf<K> &kb, Cut &cut,
+                                          float &lim, bool &lane_ok)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const uint32_t S = (uint32_t)a.n_slots;
+    uint2 *__restrict__ const L = a.ck0;
+    n_ev = 0;
+    lane_ok = true;
+    lim = GRTX_INF;
+    if (!sc.has_tree) return;
+    // a ray that is not finite cannot be bounded, and a bundle bounds depths from 0 on
+    if (valid && !(fabsf(o.x) + fabsf(o.y) + fabsf(o.z) + fabsf(d.x) + fabsf(d.y) + fabsf(d.z) < 3e38f && tn >= 0.f)) {
+        lane_ok = false;
+        valid = false;
+    }
+    if (!__any_sync(full, valid)) return;
+    const float t0 = warp_min(valid ? tn : GRTX_INF);
+    float tile_max = warp_max(valid ? tf : 0.f);     // no ray of the bundle needs anything beyond
+    {
+        // bounds of the bundle; a direction bound of 0 is moved outwards to keep its reciprocal finite
+        const float oc[3] = {o.x, o.y, o.z}, dc[3] = {d.x, d.y, d.z};
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const float omax = warp_max(valid ? oc[q] : -GRTX_INF), omin = warp_min(valid ? oc[q] : GRTX_INF);
+            float dmax = warp_max(valid ? dc[q] : -GRTX_INF), dmin = warp_min(valid ? dc[q] : GRTX_INF);
+            if (fabsf(dmax) < 1e-30f) dmax = 1e-30f;
+            if (fabsf(dmin) < 1e-30f) dmin = -1e-30f;
+            if (lane == 0) {
+                w.c[4 * q] = omax;
+                w.c[4 * q + 1] = 1.0f / dmax;
+                w.c[4 * q + 2] = omin;
+                w.c[4 * q + 3] = 1.0f / dmin;
+            }
+        }
+        if (lane == 0) w.stack[0] = 0u;
+        __syncwarp();
+    }
+    const int cap = a.packet_stack < kPacketStack ? a.packet_stack : kWalkStack;
+    const int wide = cap - kWalkReserve;
+    int sp = 1, nl = 0, work = 0, cands = 0;
+    int squeeze_at = min(kSqueeze, max(a.evict_cap - 31, 1));
+    for (;;) {
+        // expand up to 32 pending nodes, nearest first (lane 0 takes the top of the stack)
+        if (sp >= cap || (work >= kWalkTrial && 4 * cands < work)) {   // no room for children, or nothing shared
+            lane_ok = false;
+            return;
+        }
+        const int p = min(min(32, sp), max(1, wide - sp));
+        uint32_t cn = GRTX_NONE, cf = GRTX_NONE;                     // near and far child to visit
+        if (lane < p) {
+            const float4 *nd = sc.nodes + 4 * (size_t)w.stack[sp - 1 - lane];
+            const float4 n0 = __ldg(nd), n1 = __ldg(nd + 1), n2 = __ldg(nd + 2), n3 = __ldg(nd + 3);
+            float e0 = t0, x0 = tile_max, e1 = t0, x1 = tile_max;
+            bundle_axis(w.c, n0.x, n0.w, e0, x0);
+            bundle_axis(w.c + 4, n0.y, n1.x, e0, x0);
+            bundle_axis(w.c + 8, n0.z, n1.y, e0, x0);
+            bundle_axis(w.c, n1.z, n2.y, e1, x1);
+            bundle_axis(w.c + 4, n1.w, n2.z, e1, x1);
+            bundle_axis(w.c + 8, n2.x, n2.w, e1, x1);
+            // the bounds are rounded: an entry is lowered by 4e-6 of its depth, far more than its rounding
+            cn = e0 * (1.0f - 4e-6f) <= x0 ? __float_as_uint(n3.x) : GRTX_NONE;
+            cf = e1 * (1.0f - 4e-6f) <= x1 ? __float_as_uint(n3.y) : GRTX_NONE;
+            if (e1 < e0) {
+                const uint32_t t = cn; cn = cf; cf = t;
+            }
+        }
+        __syncwarp();
+        const bool ln = cn != GRTX_NONE && (cn & GRTX_LEAF), lf = cf != GRTX_NONE && (cf & GRTX_LEAF);
+        const unsigned bn = __ballot_sync(full, cn != GRTX_NONE && !ln), bf = __ballot_sync(full, cf != GRTX_NONE && !lf);
+        const unsigned gn = __ballot_sync(full, ln), gf = __ballot_sync(full, lf);
+        const unsigned below = (1u << lane) - 1u, above = ~(below | (1u << lane));
+        sp -= p;
+        work += 4;
+        int at = sp + __popc(bn & above) + __popc(bf & above);
+        if (cf != GRTX_NONE && !lf) w.stack[at++] = cf;
+        if (cn != GRTX_NONE && !ln) w.stack[at] = cn;
+        sp += __popc(bn) + __popc(bf);
+        at = nl + __popc(gn & below) + __popc(gf & below);
+        if (ln) w.leaf[at++] = cn & ~GRTX_LEAF;
+        if (lf) w.leaf[at] = cf & ~GRTX_LEAF;
+        nl += __popc(gn) + __popc(gf);
+        __syncwarp();
+        if (sp > 0 && nl <= kWalkLeaves - 64) continue;
+        // test the gathered leaves, 32 at a time: a mask of the ray's candidates, ...
+        for (int g0 = 0; g0 < nl; g0 += 32) {
+            const int m = min(32, nl - g0);
+            unsigned mask = 0;
+            const float bound = fminf(fminf(tf, lim), cut.top(a));
+            if (valid && lane_ok) {
+                for (int i = 0; i < m; ++i) {
+                    const float4 *g = sc.geom + 4 * (size_t)w.leaf[g0 + i];
+                    float t, aa;
+                    if (sphere_candidate(__ldg(g), __ldg(g + 1), __ldg(g + 2), o, d, t, aa) && in_range(t, aa, tn, bound))
+                        mask |= 1u << i;
+                }
+            }
+            work += m;
+            cands += __reduce_add_sync(full, __popc(mask));
+            // ... then the candidates of each ray one after another
+            while (mask) {
+                const int i = __ffs(mask) - 1;
+                mask &= mask - 1u;
+                const uint32_t gi = w.leaf[g0 + i];
+                const float4 *g = sc.geom + 4 * (size_t)gi;
+                float t, D2, u[3];
+                if (sphere_test(g, o, d, t, D2, u) && D2 <= 1.0f && t > tn && t <= tf &&
+                    !(t > fminf(lim, cut.top(a)))) {
+                    float ct = t;
+                    uint32_t ci = cut.add(a, g, gi, t, D2);
+                    if (kb.insert(ct, ci)) {
+                        if (n_ev >= a.evict_cap) {
+                            lane_ok = false;
+                            break;
+                        }
+                        L[ev + (uint32_t)n_ev * S] = make_uint2(__float_as_uint(ct), ci);
+                        ++n_ev;
+                    }
+                }
+            }
+            __syncwarp();
+            // long lists: find each ray's end, or make room for the next group
+            if (__any_sync(full, n_ev >= squeeze_at)) {
+                if (n_ev >= squeeze_at && lane_ok) {
+                    const bool no_room = n_ev + 32 > a.evict_cap;
+                    bool end;
+                    const float to = squeeze<K>(L + ev, S, n_ev, n_ev, kb.t, kb.id,
+                                                a.id_shift && a.p_stop > 0.f ? -__log2f(a.p_stop) : GRTX_INF, no_room, end);
+                    if (end) {
+                        cut.P = 0.f;
+                        cut.far = to;
+                    } else if (no_room) {
+                        lim = to;
+                    }
+                    squeeze_at = min(n_ev + kSqueeze, max(a.evict_cap - 31, 1));
+                }
+                __syncwarp();
+            }
+            const float need = valid && lane_ok ? fmaxf(fminf(fminf(tf, lim), cut.top(a)), 0.f) : 0.f;
+            tile_max = __uint_as_float(__reduce_max_sync(full, __float_as_uint(need)));
+        }
+        nl = 0;
+        if (sp == 0) return;
+    }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1341,8 +1656,8 @@ __device__ __forceinline__ void save_blended(const TraceArgs &a, int64_t pix, in
 template <int K, int FORM, bool INSTR, int PASS>
 __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc, float4 *__restrict__ out, int slot,
                                           int64_t pix, float3 o, float3 d, float tn, float tf, KBuf<K> &kb,
-                                          Counters &cnt, bool r1_done = false, bool r1_ok = true, int r1_n_dst = 0,
-                                          int r1_n_ev = 0)
+                                          Counters &cnt, Cut cut, bool r1_done = false, bool r1_ok = true,
+                                          int r1_n_dst = 0, int r1_n_ev = 0, float lim = INFINITY)
 {
     constexpr bool BWD = PASS == PASS_BWD;
     const uint32_t S = (uint32_t)a.n_slots;
@@ -1390,13 +1705,19 @@ __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc
         }
         int n_dst = 0;
         bool round_ok;
-        if (r1_done && first_round) {                  // round 1 was traced as the warp's packet
-            round_ok = r1_ok;
+        if (r1_done && first_round && r1_ok) {         // round 1 was traced for the warp
+            round_ok = true;
             n_dst = r1_n_dst;
             n_ev = r1_n_ev;
         } else {
+            if (r1_done && first_round) {              // it could not finish: this ray traces it on its own
+                if (INSTR) cnt.fallbacks++;
+                kb.clear();
+                cut.clear();
+                lim = GRTX_INF;
+            }
             round_ok = trace_round<K, FORM, INSTR>(a, sc, o, d, inv, inv_len, tn, tf, Lt, Li, ckpt, from_root, src, n_src,
-                                                   dst, n_dst, ev, n_ev, kb, cnt);
+                                                   dst, n_dst, ev, n_ev, kb, cut, from_root ? a.window : 0, cnt);
         }
         if (!round_ok) {
             // a capacity was exceeded: redo this round from the root and stay in restart mode
@@ -1407,10 +1728,10 @@ __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc
             n_ev = 0;
             kb.clear();
             trace_round<K, FORM, INSTR>(a, sc, o, d, inv, inv_len, tn, tf, Lt, Li, false, true, src, 0, dst, n_dst, ev, n_ev,
-                                         kb, cnt);
+                                         kb, cut, 0, cnt);
         }
         for (int j = 0; j < kb.n; ++j) {
-            uint32_t idx = kb.I(j);
+            uint32_t idx = kb.I(j) >> a.id_shift;
             blend_one<BWD>(a, sc, st, idx, o, d);
             if (INSTR) {
                 if (a.ids && nb < a.ids_cap) a.ids[(size_t)pix * a.ids_cap + nb] = sc.gid[idx];
@@ -1421,9 +1742,20 @@ __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc
             if (st.T < a.T_min) { done = true; break; }
         }
         first_round = false;
-        if (done || kb.n < K) break;
+        if (done) break;
+        if (kb.n < K) {
+            if (!(lim < GRTX_INF)) break;
+            // every hit up to the limit of the first round is blended: go on behind it, from the root
+            Lt = lim;
+            Li = GRTX_NONE;
+            lim = GRTX_INF;
+            cut.P = st.T;
+            cut.far = 0.f;
+            from_root = true;
+            continue;
+        }
         Lt = kb.T(K - 1);
-        Li = kb.I(K - 1);
+        Li = kb.I(K - 1) >> a.id_shift;
         if (ckpt) {
             uint32_t tmp = src; src = dst; dst = tmp;
             n_src = n_dst;
@@ -1482,6 +1814,8 @@ __device__ __forceinline__ void trace_warp_restart(const TraceArgs &a, const Sce
     uint32_t Li = GRTX_NONE;
     int nb = 0;
     bool done = !valid || !sc.has_tree;
+    Cut cut;                                   // unused: without an eviction list the k-buffer bounds a round
+    cut.clear();
     while (__any_sync(0xffffffffu, !done)) {
         if (!done) {
             if (INSTR) cnt.rounds++;
@@ -1490,12 +1824,12 @@ __device__ __forceinline__ void trace_warp_restart(const TraceArgs &a, const Sce
         int n_dst = 0, n_ev = 0;
         bool lane_ok = true;
         packet_round<K, FORM, INSTR>(a, sc, !done, pst, o, d, inv, nrm, tn, tf, Lt, Li, false, 0u, n_dst, 0u, n_ev,
-                                     kb, cnt, lane_ok);
+                                     kb, cut, cnt, lane_ok);
         if (done) continue;
         if (!lane_ok) {
             kb.clear();
             trace_round<K, FORM, INSTR>(a, sc, o, d, inv, nrm, tn, tf, Lt, Li, false, true, 0u, 0, 0u, n_dst, 0u, n_ev,
-                                        kb, cnt);
+                                        kb, cut, 0, cnt);
         }
         for (int j = 0; j < kb.n; ++j) {
             uint32_t idx = kb.I(j);
@@ -1548,14 +1882,23 @@ __device__ __forceinline__ void trace_warp(const TraceArgs &a, const SceneRef &s
     float3 inv = make_float3(safe_rcp(d.x), safe_rcp(d.y), safe_rcp(d.z));
     float inv_len = rsqrtf(d.x * d.x + d.y * d.y + d.z * d.z);
     kb.clear();
+    Cut cut;
+    cut.clear();
     int n_dst = 0, n_ev = 0;
     bool lane_ok = true;
-    packet_round<K, FORM, INSTR>(a, sc, valid, pst, o, d, inv, inv_len, tn, tf, tn, GRTX_NONE,
-                                 a.traversal == GRTX_TRAVERSAL_CHECKPOINT, a.ck1_off + (uint32_t)slot, n_dst,
-                                 a.ev_off + (uint32_t)slot, n_ev, kb, cnt, lane_ok);
+    float lim = GRTX_INF;
+    static_assert(sizeof(WalkShared) <= kWarpShared * sizeof(uint4), "the walk's shared memory");
+    if (FORM == FORM_SPHERE && !INSTR && a.traversal == GRTX_TRAVERSAL_CHECKPOINT) {
+        tile_walk<K>(a, sc, valid, *reinterpret_cast<WalkShared *>(pst), o, d, tn, tf, a.ev_off + (uint32_t)slot, n_ev,
+                     kb, cut, lim, lane_ok);
+    } else {
+        packet_round<K, FORM, INSTR>(a, sc, valid, pst, o, d, inv, inv_len, tn, tf, tn, GRTX_NONE,
+                                     a.traversal == GRTX_TRAVERSAL_CHECKPOINT, a.ck1_off + (uint32_t)slot, n_dst,
+                                     a.ev_off + (uint32_t)slot, n_ev, kb, cut, cnt, lane_ok);
+    }
     // a lane whose packet could not finish (lists or the warp's stack overflowed) redoes round 1
     // from the root on its own, as after any capacity overflow
-    if (valid) trace_ray<K, FORM, INSTR, PASS>(a, sc, out, slot, pix, o, d, tn, tf, kb, cnt, true, lane_ok, n_dst, n_ev);
+    if (valid) trace_ray<K, FORM, INSTR, PASS>(a, sc, out, slot, pix, o, d, tn, tf, kb, cnt, cut, true, lane_ok, n_dst, n_ev, lim);
 }
 
 // After a tile, every checkpoint and eviction list entry of the warp's 32 ray slots is dead:
@@ -1603,7 +1946,7 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, PASS == PASS_BWD))
 {
     __shared__ float s_kt[K * kBlock];
     __shared__ uint32_t s_ki[K * kBlock];
-    __shared__ uint4 s_pst[kBlock / 32][kPacketStack];
+    __shared__ uint4 s_pst[kBlock / 32][kWarpShared];
     const int slot = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     KBuf<K> kb;
@@ -1711,7 +2054,7 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, false))
 {
     __shared__ float s_kt[K * kBlock];
     __shared__ uint32_t s_ki[K * kBlock];
-    __shared__ uint4 s_pst[kBlock / 32][kPacketStack];
+    __shared__ uint4 s_pst[kBlock / 32][kWarpShared];
     const unsigned kNoWork = 0xffffffffu;
     const int slot = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
@@ -1781,6 +2124,24 @@ inline bool set_list_offsets(TraceArgs &a, size_t entries_per_slot)
     a.ck1_off = (uint32_t)(a.ck1 - a.ck0);
     a.ev_off = (uint32_t)(a.ev - a.ck0);
     return true;
+}
+
+// The first round's window and the opacity at which a ray is known to end (see Cut). The window
+// leaves room in both lists: with the default capacities (256 / 512) it is 64 hits.
+inline void set_window(TraceArgs &a)
+{
+    const int cap = a.ckpt_cap < a.evict_cap ? a.ckpt_cap : a.evict_cap;
+    a.window = a.traversal == GRTX_TRAVERSAL_CHECKPOINT ? cap / 4 : 0;
+    a.p_stop = a.T_min >= 1e-30f ? 0.98f * a.T_min : 0.0f;
+    a.id_shift = 0;
+}
+
+// Opacity codes in the list entries: for the walk (uninstrumented sphere-form kernels), where the
+// largest scene's leaf slots leave room for them.
+inline void set_codes(TraceArgs &a, int form, bool instr, int64_t n_valid)
+{
+    const bool walk = form == FORM_SPHERE && !instr && a.traversal == GRTX_TRAVERSAL_CHECKPOINT;
+    a.id_shift = walk && n_valid < ((int64_t)1 << (32 - kCodeBits)) ? kCodeBits : 0;
 }
 
 // Whether the lists of a launch may be dropped from L2 per tile (see discard_dead_lists): the

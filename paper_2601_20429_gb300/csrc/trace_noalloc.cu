@@ -121,6 +121,7 @@ extern "C" GRTX_API int grtx_trace_forward_noalloc(grtx_scene *sc, const grtx_ca
     a.ckpt_cap = p->ckpt_capacity > 0 ? p->ckpt_capacity : GRTX_DEFAULT_CKPT_CAPACITY;
     a.evict_cap = p->evict_capacity > 0 ? p->evict_capacity : GRTX_DEFAULT_EVICT_CAPACITY;
     a.packet_stack = p->packet_stack > 0 ? std::min(p->packet_stack, kPacketStack) : kPacketStack;
+    set_window(a);
     a.rgbT = (float4 *)d_rgbT;
     bool ckpt = a.traversal == GRTX_TRAVERSAL_CHECKPOINT;
     size_t C = ckpt ? (size_t)a.ckpt_cap : 1, E = ckpt ? (size_t)a.evict_cap : 1;
@@ -148,6 +149,7 @@ extern "C" GRTX_API int grtx_trace_forward_noalloc(grtx_scene *sc, const grtx_ca
     a.queue = (unsigned *)base;
     set_list_offsets(a, 2 * C + E);          // the fixed scratch holds far fewer than 2^31 entries
     a.discard = lists_discardable(a);
+    set_codes(a, form, false, sc->n_valid);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     // the counter must start at zero; the lists are always written before they are read
     GRTX_CUDA(cudaMemsetAsync(a.queue, 0, sizeof(unsigned), s));

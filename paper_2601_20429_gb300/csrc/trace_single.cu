@@ -166,7 +166,9 @@ __device__ __forceinline__ void single_ray(const TraceArgs &a, const SceneRef &s
         if (INSTR) cnt.rounds++;
         if (n < 0) {                  // more hits than the list holds: k-buffer rounds instead
             if (INSTR) cnt.fallbacks++;
-            trace_ray<kFallbackK, FORM, INSTR, false>(a, sc, a.rgbT, slot, pix, o, d, tn, tf, kb, cnt);
+            Cut cut;
+            cut.clear();
+            trace_ray<kFallbackK, FORM, INSTR, false>(a, sc, a.rgbT, slot, pix, o, d, tn, tf, kb, cnt, cut);
             return;
         }
     }
