@@ -1106,7 +1106,7 @@ __device__ __forceinline__ bool trace_round(const TraceArgs &a, const SceneRef &
 // round from the root on its own, as after any capacity overflow in trace_ray.
 // ------------------------------------------------------------------------------------------
 constexpr int kPacketStack = GRTX_PACKET_STACK;
-constexpr int kWarpShared = 84;
+constexpr int kWarpShared = 117;
 
 template <int K, int FORM, bool INSTR>
 __device__ __forceinline__ bool packet_round(const TraceArgs &a, const SceneRef &sc, bool valid, uint4 *pst, float3 o,
@@ -1293,6 +1293,8 @@ struct __align__(16) WalkShared {
     uint32_t stack[kWalkStack];  // pending nodes
     uint32_t leaf[kWalkLeaves];  // gathered leaves
     float c[12];                 // per axis: origin max, 1 / direction max, origin min, 1 / direction min
+    float mid[4];                // middle of the direction box, and the largest distance of a ray's direction from it
+    float4 off[32];              // each ray's direction minus mid (rays of one origin)
 };
 
 __device__ __forceinline__ float warp_min(float v)
@@ -1361,6 +1363,55 @@ constexpr int kSqueeze = 64;     // entries a list may grow by before it is sque
 // four is given up: its rays share almost nothing, and each traces the round on its own.
 constexpr int kWalkTrial = 512;
 
+// Which rays of one origin o may hit a Gaussian, as one quadratic in the ray's direction. A ray
+// d = mid + x meets the Gaussian where |o_l x d_l|^2 <= |d_l|^2 (o_l = A (o - mu), d_l = A d): with
+// c0 = o_l x A mid and the columns a_k of A, C_k = o_l x a_k, that is
+//   |c0|^2 - |A mid|^2 + sum_k 2 (c0.C_k - A mid.a_k) x_k + sum_kl (C_k.C_l - a_k.a_l) x_k x_l <= 0,
+// divided by |A mid|^2. Each lane sets up one leaf (about 150 instructions), then every ray costs 9
+// FMAs a leaf instead of the 45 of sphere_candidate. The test only filters, so it is widened by its
+// rounding: |o_l| and d_l err by up to e = 2e-6 |A| |o - mu| in units of the sphere (taken as 32 ulp
+// of the products), and the sum by 2e-6 of its largest terms.
+struct ConeTest {
+    float c, bx, by, bz, xx, yy, zz, xy, xz, yz;
+    __device__ __forceinline__ void set(float4 r0, float4 r1, float4 r2, float3 o, float3 m, float r)
+    {
+        const float vx = o.x - r0.w, vy = o.y - r1.w, vz = o.z - r2.w;
+        const float o0 = r0.x * vx + r0.y * vy + r0.z * vz, o1 = r1.x * vx + r1.y * vy + r1.z * vz,
+                    o2 = r2.x * vx + r2.y * vy + r2.z * vz;
+        const float d0 = r0.x * m.x + r0.y * m.y + r0.z * m.z, d1 = r1.x * m.x + r1.y * m.y + r1.z * m.z,
+                    d2 = r2.x * m.x + r2.y * m.y + r2.z * m.z;
+        const float inv = 1.0f / (d0 * d0 + d1 * d1 + d2 * d2);
+        const float t = -(o0 * d0 + o1 * d1 + o2 * d2) * inv;
+        const float p0 = fmaf(t, d0, o0), p1 = fmaf(t, d1, o1), p2 = fmaf(t, d2, o2);
+        // c0 = p x d_l: the part of o_l along A mid drops out
+        const float c0 = p1 * d2 - p2 * d1, c1 = p2 * d0 - p0 * d2, c2 = p0 * d1 - p1 * d0;
+        const float X0 = o1 * r2.x - o2 * r1.x, X1 = o2 * r0.x - o0 * r2.x, X2 = o0 * r1.x - o1 * r0.x;
+        const float Y0 = o1 * r2.y - o2 * r1.y, Y1 = o2 * r0.y - o0 * r2.y, Y2 = o0 * r1.y - o1 * r0.y;
+        const float Z0 = o1 * r2.z - o2 * r1.z, Z1 = o2 * r0.z - o0 * r2.z, Z2 = o0 * r1.z - o1 * r0.z;
+        const float axx = r0.x * r0.x + r1.x * r1.x + r2.x * r2.x, ayy = r0.y * r0.y + r1.y * r1.y + r2.y * r2.y,
+                    azz = r0.z * r0.z + r1.z * r1.z + r2.z * r2.z;
+        const float e = 2e-6f * sqrtf((axx + ayy + azz) * (vx * vx + vy * vy + vz * vz)), g = 1.0f + 2.0f * e + e * e;
+        const float Xx = X0 * X0 + X1 * X1 + X2 * X2, Yy = Y0 * Y0 + Y1 * Y1 + Y2 * Y2, Zz = Z0 * Z0 + Z1 * Z1 + Z2 * Z2;
+        const float cc = (c0 * c0 + c1 * c1 + c2 * c2) * inv;
+        c = cc - g - 2e-6f * (cc + r * r * (Xx + Yy + Zz) * inv + g);
+        bx = 2.0f * inv * (c0 * X0 + c1 * X1 + c2 * X2 - g * (d0 * r0.x + d1 * r1.x + d2 * r2.x));
+        by = 2.0f * inv * (c0 * Y0 + c1 * Y1 + c2 * Y2 - g * (d0 * r0.y + d1 * r1.y + d2 * r2.y));
+        bz = 2.0f * inv * (c0 * Z0 + c1 * Z1 + c2 * Z2 - g * (d0 * r0.z + d1 * r1.z + d2 * r2.z));
+        xx = inv * (Xx - g * axx);
+        yy = inv * (Yy - g * ayy);
+        zz = inv * (Zz - g * azz);
+        xy = 2.0f * inv * (X0 * Y0 + X1 * Y1 + X2 * Y2 - g * (r0.x * r0.y + r1.x * r1.y + r2.x * r2.y));
+        xz = 2.0f * inv * (X0 * Z0 + X1 * Z1 + X2 * Z2 - g * (r0.x * r0.z + r1.x * r1.z + r2.x * r2.z));
+        yz = 2.0f * inv * (Y0 * Z0 + Y1 * Z1 + Y2 * Z2 - g * (r0.y * r0.z + r1.y * r1.z + r2.y * r2.z));
+    }
+    __device__ __forceinline__ bool miss(float4 x) const
+    {
+        const float a = fmaf(xz, x.z, fmaf(xy, x.y, fmaf(xx, x.x, bx)));
+        const float b = fmaf(yz, x.z, fmaf(yy, x.y, by)), d = fmaf(zz, x.z, bz);
+        return fmaf(d, x.z, fmaf(b, x.y, fmaf(a, x.x, c))) > 0.f;
+    }
+};
+
 // Walks the bundles of a warp's rays. lane_ok is false for a ray that must trace the round on its
 // own: its eviction list was too small, or its bundle was left (too little stack, too little shared).
 template <int K>
@@ -1384,14 +1435,18 @@ __device__ __forceinline__ void tile_walk(const TraceArgs &a, const SceneRef &sc
     if (!__any_sync(full, valid)) return;
     const float t0 = warp_min(valid ? tn : GRTX_INF);
     float tile_max = warp_max(valid ? tf : 0.f);     // no ray of the bundle needs anything beyond
+    bool one_origin = true;
     {
         // bounds of the bundle; a direction bound of 0 is moved outwards to keep its reciprocal finite
         const float oc[3] = {o.x, o.y, o.z}, dc[3] = {d.x, d.y, d.z};
+        float mid[3];
         __syncwarp();
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
             const float omax = warp_max(valid ? oc[q] : -GRTX_INF), omin = warp_min(valid ? oc[q] : GRTX_INF);
             float dmax = warp_max(valid ? dc[q] : -GRTX_INF), dmin = warp_min(valid ? dc[q] : GRTX_INF);
+            mid[q] = 0.5f * dmin + 0.5f * dmax;
+            one_origin = one_origin && omin == omax;
             if (fabsf(dmax) < 1e-30f) dmax = 1e-30f;
             if (fabsf(dmin) < 1e-30f) dmin = -1e-30f;
             if (lane == 0) {
@@ -1401,7 +1456,16 @@ __device__ __forceinline__ void tile_walk(const TraceArgs &a, const SceneRef &sc
                 w.c[4 * q + 3] = 1.0f / dmin;
             }
         }
-        if (lane == 0) w.stack[0] = 0u;
+        const float4 x = valid ? make_float4(d.x - mid[0], d.y - mid[1], d.z - mid[2], 0.f) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float r = sqrtf(warp_max(x.x * x.x + x.y * x.y + x.z * x.z));
+        w.off[lane] = x;
+        if (lane == 0) {
+            w.stack[0] = 0u;
+            w.mid[0] = mid[0];
+            w.mid[1] = mid[1];
+            w.mid[2] = mid[2];
+            w.mid[3] = r;
+        }
         __syncwarp();
     }
     const int cap = a.packet_stack < kPacketStack ? a.packet_stack : kWalkStack;
@@ -1455,7 +1519,19 @@ __device__ __forceinline__ void tile_walk(const TraceArgs &a, const SceneRef &sc
             const int m = min(32, nl - g0);
             unsigned mask = 0;
             const float bound = fminf(fminf(tf, lim), cut.top(a));
-            if (valid && lane_ok) {
+            if (one_origin) {
+                // a lane takes a leaf and goes through the rays
+                const float4 *g = sc.geom + 4 * (size_t)w.leaf[g0 + min(lane, m - 1)];
+                ConeTest q;
+                const float3 oo = make_float3(w.c[0], w.c[4], w.c[8]);
+                q.set(__ldg(g), __ldg(g + 1), __ldg(g + 2), oo, make_float3(w.mid[0], w.mid[1], w.mid[2]), w.mid[3]);
+#pragma unroll 8
+                for (int r = 0; r < 32; ++r) {
+                    const unsigned b = __ballot_sync(full, !q.miss(w.off[r]));
+                    if (lane == r) mask = b;
+                }
+                mask &= m == 32 ? full : (1u << m) - 1u;
+            } else {
                 for (int i = 0; i < m; ++i) {
                     const float4 *g = sc.geom + 4 * (size_t)w.leaf[g0 + i];
                     float t, aa;
@@ -1463,6 +1539,7 @@ __device__ __forceinline__ void tile_walk(const TraceArgs &a, const SceneRef &sc
                         mask |= 1u << i;
                 }
             }
+            if (!(valid && lane_ok)) mask = 0;
             work += m;
             cands += __reduce_add_sync(full, __popc(mask));
             // ... then the candidates of each ray one after another
@@ -1471,9 +1548,11 @@ __device__ __forceinline__ void tile_walk(const TraceArgs &a, const SceneRef &sc
                 mask &= mask - 1u;
                 const uint32_t gi = w.leaf[g0 + i];
                 const float4 *g = sc.geom + 4 * (size_t)gi;
-                float t, D2, u[3];
-                if (sphere_test(g, o, d, t, D2, u) && D2 <= 1.0f && t > tn && t <= tf &&
-                    !(t > fminf(lim, cut.top(a)))) {
+                float t, D2, u[3], aa;
+                const float4 r0 = __ldg(g), r1 = __ldg(g + 1), r2 = __ldg(g + 2);
+                if (!sphere_candidate(r0, r1, r2, o, d, t, aa) || !in_range(t, aa, tn, fminf(bound, cut.top(a)))) continue;
+                sphere_refine(r0, r1, r2, o, d, t, D2, u);
+                if (D2 <= 1.0f && t > tn && t <= tf && !(t > fminf(lim, cut.top(a)))) {
                     float ct = t;
                     uint32_t ci = cut.add(a, g, gi, t, D2);
                     if (kb.insert(ct, ci)) {
@@ -1487,9 +1566,10 @@ __device__ __forceinline__ void tile_walk(const TraceArgs &a, const SceneRef &sc
                 }
             }
             __syncwarp();
-            // long lists: find each ray's end, or make room for the next group
+            // long lists: find each ray's end, or make room for the next group (rays that are nearly due
+            // take part, so that the warp does this seldom)
             if (__any_sync(full, n_ev >= squeeze_at)) {
-                if (n_ev >= squeeze_at && lane_ok) {
+                if (4 * n_ev >= 3 * squeeze_at && lane_ok) {
                     const bool no_room = n_ev + 32 > a.evict_cap;
                     bool end;
                     const float to = squeeze<K>(L + ev, S, n_ev, n_ev, kb.t, kb.id,
