@@ -204,14 +204,12 @@ __device__ __forceinline__ void single_ray(const TraceArgs &a, const SceneRef &s
 template <int FORM, bool INSTR>
 __global__ void __launch_bounds__(kBlock, 8) k_trace_single(TraceArgs a)
 {
-    __shared__ float s_kt[kFallbackK * kBlock];
-    __shared__ uint32_t s_ki[kFallbackK * kBlock];
+    __shared__ uint64_t s_k[kFallbackK * kBlock];
     __shared__ uint4 s_pst[kBlock / 32][kPacketStack];
     const int slot = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     KBuf<kFallbackK> kb;
-    kb.t = s_kt + threadIdx.x;
-    kb.id = s_ki + threadIdx.x;
+    kb.k = s_k + threadIdx.x;
     Counters cnt = {0, 0, 0, 0, 0, 0, 0, 0, 0, nullptr, 0, 0};
     unsigned rays = 0, collected = 0;
     for (;;) {

@@ -459,14 +459,12 @@ __device__ __forceinline__ void world_ray(const WorldArgs &W, int slot, int64_t 
 template <int K, bool INSTR>
 __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, false)) k_trace_world(WorldArgs W)
 {
-    __shared__ float s_kt[K * kBlock];
-    __shared__ uint32_t s_ki[K * kBlock];
+    __shared__ uint64_t s_k[K * kBlock];
     __shared__ uint4 s_pst[kBlock / 32][kPacketStack];
     const int slot = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     KBuf<K> kb;
-    kb.t = s_kt + threadIdx.x;
-    kb.id = s_ki + threadIdx.x;
+    kb.k = s_k + threadIdx.x;
     Counters cnt = {0, 0, 0, 0, 0, 0, 0, 0, 0, nullptr, 0, 0};
     unsigned rays = 0;
     for (;;) {
