@@ -10,7 +10,8 @@
 
 #define GRTX_EXTERN_TRACE(K)                                                                     \
     extern template int trace_launch<K>(const TraceArgs &, int, bool, int, int, cudaStream_t); \
-    extern template int trace_occupancy<K>(int, bool, int, int *);
+    extern template int trace_occupancy<K>(int, bool, int, int *);                             \
+    extern template int trace_rays_launch<K>(const TraceArgs &, int, cudaStream_t);
 GRTX_EXTERN_TRACE(1)
 GRTX_EXTERN_TRACE(2)
 GRTX_EXTERN_TRACE(4)
@@ -47,6 +48,18 @@ int launch_k(int k, const TraceArgs &a, int form, bool instr, int pass, int bloc
     case 8: return trace_launch<8>(a, form, instr, pass, blocks, s);
     case 16: return trace_launch<16>(a, form, instr, pass, blocks, s);
     default: return trace_launch<32>(a, form, instr, pass, blocks, s);
+    }
+}
+
+int rays_launch_k(int k, const TraceArgs &a, int blocks, cudaStream_t s)
+{
+    switch (k) {
+    case 1: return trace_rays_launch<1>(a, blocks, s);
+    case 2: return trace_rays_launch<2>(a, blocks, s);
+    case 4: return trace_rays_launch<4>(a, blocks, s);
+    case 8: return trace_rays_launch<8>(a, blocks, s);
+    case 16: return trace_rays_launch<16>(a, blocks, s);
+    default: return trace_rays_launch<32>(a, blocks, s);
     }
 }
 
@@ -146,10 +159,11 @@ int sm_count()
     return cached[dev];
 }
 
-// Per-slot lists (entries_per_slot uint2 per ray slot), grown on demand; returns the base.
-int ensure_workspace(grtx_scene *sc, int n_slots, size_t entries_per_slot, cudaStream_t s, uint2 **base_out)
+// Per-slot lists (entries_per_slot uint2 per ray slot) and extra bytes behind them, grown on demand;
+// returns the base.
+int ensure_workspace(grtx_scene *sc, int n_slots, size_t entries_per_slot, size_t extra_bytes, cudaStream_t s, uint2 **base_out)
 {
-    size_t need = (size_t)n_slots * entries_per_slot * sizeof(uint2);
+    size_t need = (size_t)n_slots * entries_per_slot * sizeof(uint2) + extra_bytes;
     if (need > sc->ws_bytes) {
         if (sc->ws) {
             GRTX_CUDA(cudaDeviceSynchronize());   // earlier traces on any stream may still use it
@@ -231,9 +245,14 @@ int run(grtx_scene *sc, TraceArgs &a, int k, bool instr, int pass, unsigned *que
     // checkpoint: two ping-pong checkpoint lists and the eviction list; single: the hit list
     size_t C = ckpt ? a.ckpt_cap : 1, E = ckpt ? a.evict_cap : 1;
     size_t per_slot = single ? (size_t)a.ckpt_cap : 2 * C + E;
+    // bundles of a ray list may be left to k_trace_rays: room for all of them behind the lists
+    const bool walk = form == FORM_SPHERE && !instr && ckpt;
+    a.split = walk ? split_for(a.n_items / 32, (unsigned)blocks * (kBlock / 32)) : 0;
+    const bool leaves = walk && pass == PASS_FWD && a.cam.cam_type == GRTX_CAMERA_RAYS;
     uint2 *base = nullptr;
-    int st = ensure_workspace(sc, n_slots, per_slot, s, &base);
+    int st = ensure_workspace(sc, n_slots, per_slot, leaves ? ((size_t)a.n_items >> (5 - a.split)) * sizeof(unsigned) : 0, s, &base);
     if (st) return st;
+    a.left = leaves ? (unsigned *)(base + (size_t)n_slots * per_slot) : nullptr;
     a.ck0 = base;
     a.ck1 = single ? base : base + (size_t)n_slots * C;
     a.ev = single ? base : base + (size_t)n_slots * 2 * C;
@@ -242,9 +261,10 @@ int run(grtx_scene *sc, TraceArgs &a, int k, bool instr, int pass, unsigned *que
     if (!set_list_offsets(a, per_slot))
         return grtx_fail(GRTX_ERR_INVALID_ARG, "checkpoint/eviction capacities too large for the resident ray slots");
     a.discard = single ? 0 : lists_discardable(a);
-    GRTX_CUDA(cudaMemsetAsync(queue, 0, sizeof(unsigned), s));
+    GRTX_CUDA(cudaMemsetAsync(queue, 0, (leaves ? 6 : 1) * sizeof(unsigned), s));      // (queue[4], [5]: k_trace_rays)
     int launched = single ? trace_single_launch(a, form, instr, blocks, s)
                           : launch_k(k, a, form, instr, pass, blocks, s);
+    if (launched == GRTX_OK && leaves) launched = rays_launch_k(k, a, std::min(blocks, sm_count() * 5), s);
     if (launched != GRTX_OK) {
         cudaError_t e = cudaGetLastError();
         return grtx_cuda_fail(e == cudaSuccess ? cudaErrorLaunchFailure : e, "trace launch");
@@ -440,7 +460,7 @@ extern "C" GRTX_API int grtx_trace_forward_batch(grtx_scene *sc, const grtx_came
     size_t C = ckpt ? a.ckpt_cap : 1, E = ckpt ? a.evict_cap : 1;
     uint2 *base = nullptr;
     cudaStream_t s = S(stream);
-    st = ensure_workspace(sc, n_slots, 2 * C + E, s, &base);
+    st = ensure_workspace(sc, n_slots, 2 * C + E, 0, s, &base);
     if (st) return st;
     a.ck0 = base;
     a.ck1 = base + (size_t)n_slots * C;

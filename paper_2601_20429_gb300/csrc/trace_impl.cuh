@@ -59,6 +59,8 @@ struct TraceArgs {
     uint2 *ck0, *ck1, *ev;
     uint32_t ck1_off, ev_off;
     int n_slots;
+    int split;                   // k_trace: a warp takes 32 >> split rays at a time (see split_for)
+    unsigned *left;              // bundles left for k_trace_rays: their first items (counted in queue[4]), or NULL
     int discard;                 // drop dead list lines from L2 after each tile (lists 256-byte aligned)
     unsigned *queue;
     // outputs
@@ -355,7 +357,10 @@ struct Cut {
     __device__ __forceinline__ uint32_t add(const TraceArgs &a, const float4 *__restrict__ g, uint32_t gi, float t, float D2)
     {
         const float4 r3 = __ldg(g + 3);
-        const float q = 1.0f - fminf(r3.x * exp2f(r3.y * D2), a.alpha_max);
+        return take(a, 1.0f - fminf(r3.x * exp2f(r3.y * D2), a.alpha_max), gi, t);
+    }
+    __device__ __forceinline__ uint32_t take(const TraceArgs &a, float q, uint32_t gi, float t)      // q = 1 - alpha
+    {
         P *= q;
         far = fmaxf(far, t);
         return a.id_shift ? gi << kCodeBits | opacity_code(q) : gi;
@@ -1113,7 +1118,7 @@ __device__ __forceinline__ bool trace_round(const TraceArgs &a, const SceneRef &
 // round from the root on its own, as after any capacity overflow in trace_ray.
 // ------------------------------------------------------------------------------------------
 constexpr int kPacketStack = GRTX_PACKET_STACK;
-constexpr int kWarpShared = 117;
+constexpr int kWarpShared = 118;
 
 template <int K, int FORM, bool INSTR>
 __device__ __forceinline__ bool packet_round(const TraceArgs &a, const SceneRef &sc, bool valid, uint4 *pst, float3 o,
@@ -1301,6 +1306,7 @@ struct __align__(16) WalkShared {
     uint32_t leaf[kWalkLeaves];  // gathered leaves
     float c[12];                 // per axis: origin max, 1 / direction max, origin min, 1 / direction min
     float mid[4];                // middle of the direction box, and the largest distance of a ray's direction from it
+    unsigned item;               // the bundle's place in the queue
     float4 off[32];              // each ray's direction minus mid (rays of one origin)
 };
 
@@ -1419,30 +1425,25 @@ struct ConeTest {
     }
 };
 
-// Walks the bundles of a warp's rays. lane_ok is false for a ray that must trace the round on its
-// own: its eviction list was too small, or its bundle was left (too little stack, too little shared).
+// Walks the bundle of the warp's valid rays (the other lanes help, and keep their rays' state).
+// lane_ok becomes false for a ray whose eviction list was too small. Returns false if the bundle was
+// left: no stack, a ray that cannot be bounded, or too little shared.
 template <int K>
-__device__ __forceinline__ void tile_walk(const TraceArgs &a, const SceneRef &sc, bool valid, WalkShared &w, float3 o,
-                                          float3 d, float tn, float tf, uint32_t ev, int &n_ev, KBuf<K> &kb, Cut &cut,
-                                          float &lim, bool &lane_ok)
+__device__ __forceinline__ bool tile_walk(const TraceArgs &a, const SceneRef &sc, bool valid, WalkShared &w,
+                                          float3 o, float3 d, float tn, float tf, uint32_t ev, int &n_ev, KBuf<K> &kb,
+                                          Cut &cut, float &lim, bool &lane_ok)
 {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const uint32_t S = (uint32_t)a.n_slots;
     uint2 *__restrict__ const L = a.ck0;
-    n_ev = 0;
-    lane_ok = true;
-    lim = GRTX_INF;
-    if (!sc.has_tree) return;
+    if (!__any_sync(full, valid)) return true;
     // a ray that is not finite cannot be bounded, and a bundle bounds depths from 0 on
-    if (valid && !(fabsf(o.x) + fabsf(o.y) + fabsf(o.z) + fabsf(d.x) + fabsf(d.y) + fabsf(d.z) < 3e38f && tn >= 0.f)) {
-        lane_ok = false;
-        valid = false;
-    }
-    if (!__any_sync(full, valid)) return;
+    const bool odd = valid && !(fabsf(o.x) + fabsf(o.y) + fabsf(o.z) + fabsf(d.x) + fabsf(d.y) + fabsf(d.z) < 3e38f && tn >= 0.f);
+    if (__any_sync(full, odd)) return false;
     const float t0 = warp_min(valid ? tn : GRTX_INF);
     float tile_max = warp_max(valid ? tf : 0.f);     // no ray of the bundle needs anything beyond
-    bool one_origin = true;
+    bool one_origin = true, every_way = true;
     {
         // bounds of the bundle; a direction bound of 0 is moved outwards to keep its reciprocal finite
         const float oc[3] = {o.x, o.y, o.z}, dc[3] = {d.x, d.y, d.z};
@@ -1454,6 +1455,7 @@ __device__ __forceinline__ void tile_walk(const TraceArgs &a, const SceneRef &sc
             float dmax = warp_max(valid ? dc[q] : -GRTX_INF), dmin = warp_min(valid ? dc[q] : GRTX_INF);
             mid[q] = 0.5f * dmin + 0.5f * dmax;
             one_origin = one_origin && omin == omax;
+            every_way = every_way && dmin < 0.f && dmax > 0.f;
             if (fabsf(dmax) < 1e-30f) dmax = 1e-30f;
             if (fabsf(dmin) < 1e-30f) dmin = -1e-30f;
             if (lane == 0) {
@@ -1463,6 +1465,7 @@ __device__ __forceinline__ void tile_walk(const TraceArgs &a, const SceneRef &sc
                 w.c[4 * q + 3] = 1.0f / dmin;
             }
         }
+        if (every_way) return false;         // the direction box holds 0: it bounds nothing
         const float4 x = valid ? make_float4(d.x - mid[0], d.y - mid[1], d.z - mid[2], 0.f) : make_float4(0.f, 0.f, 0.f, 0.f);
         const float r = sqrtf(warp_max(x.x * x.x + x.y * x.y + x.z * x.z));
         w.off[lane] = x;
@@ -1481,10 +1484,7 @@ __device__ __forceinline__ void tile_walk(const TraceArgs &a, const SceneRef &sc
     int squeeze_at = min(kSqueeze, max(a.evict_cap - 31, 1));
     for (;;) {
         // expand up to 32 pending nodes, nearest first (lane 0 takes the top of the stack)
-        if (sp >= cap || (work >= kWalkTrial && 4 * cands < work)) {   // no room for children, or nothing shared
-            lane_ok = false;
-            return;
-        }
+        if (sp >= cap || (work >= kWalkTrial && 4 * cands < work)) return false;   // no room, or nothing shared
         const int p = min(min(32, sp), max(1, wide - sp));
         uint32_t cn = GRTX_NONE, cf = GRTX_NONE;                     // near and far child to visit
         if (lane < p) {
@@ -1532,10 +1532,14 @@ __device__ __forceinline__ void tile_walk(const TraceArgs &a, const SceneRef &sc
                 ConeTest q;
                 const float3 oo = make_float3(w.c[0], w.c[4], w.c[8]);
                 q.set(__ldg(g), __ldg(g + 1), __ldg(g + 2), oo, make_float3(w.mid[0], w.mid[1], w.mid[2]), w.mid[3]);
-#pragma unroll 8
-                for (int r = 0; r < 32; ++r) {
-                    const unsigned b = __ballot_sync(full, !q.miss(w.off[r]));
-                    if (lane == r) mask = b;
+                const unsigned rays = __ballot_sync(full, valid);
+                for (int r0 = 0; rays >> r0; r0 += 8) {
+#pragma unroll
+                    for (int r = r0; r < r0 + 8; ++r) {
+                        const unsigned b = __ballot_sync(full, !q.miss(w.off[r]));
+                        if (lane == r) mask = b;
+                    }
+                    if (r0 == 24) break;
                 }
                 mask &= m == 32 ? full : (1u << m) - 1u;
             } else {
@@ -1595,7 +1599,7 @@ __device__ __forceinline__ void tile_walk(const TraceArgs &a, const SceneRef &sc
             tile_max = __uint_as_float(__reduce_max_sync(full, __float_as_uint(need)));
         }
         nl = 0;
-        if (sp == 0) return;
+        if (sp == 0) return true;
     }
 }
 
@@ -1615,6 +1619,21 @@ struct BlendState {
 __device__ __forceinline__ float atomic_add_f(float *p, float v)
 {
     return atomicAdd(p, v);
+}
+
+// alpha and colour of leaf slot idx on a ray, as the forward blend_one computes them.
+__device__ __forceinline__ float blend_terms(const TraceArgs &a, const SceneRef &sc, uint32_t idx, float3 o, float3 d, float c[3])
+{
+    const float nrm = rsqrtf(d.x * d.x + d.y * d.y + d.z * d.z);
+    const float4 *g = sc.geom + 4 * (size_t)idx;
+    const float4 r0 = __ldg(g), r1 = __ldg(g + 1), r2 = __ldg(g + 2), r3 = __ldg(g + 3);
+    float t, D2, e[3], raw[3], Y[16];
+    sphere_candidate(r0, r1, r2, o, d, t);
+    sphere_refine(r0, r1, r2, o, d, t, D2, e);
+    sh_color(sc.app + (size_t)idx * sc.app_stride, sc.sh_degree, sc.app_stride,
+             make_float3(d.x * nrm, d.y * nrm, d.z * nrm), c, raw, Y);
+    const float al = r3.x * exp2f(r3.y * D2);
+    return al < a.alpha_max ? al : a.alpha_max;
 }
 
 template <bool BWD>
@@ -1976,8 +1995,15 @@ __device__ __forceinline__ void trace_warp(const TraceArgs &a, const SceneRef &s
     float lim = GRTX_INF;
     static_assert(sizeof(WalkShared) <= kWarpShared * sizeof(uint4), "the walk's shared memory");
     if (FORM == FORM_SPHERE && !INSTR && a.traversal == GRTX_TRAVERSAL_CHECKPOINT) {
-        tile_walk<K>(a, sc, valid, *reinterpret_cast<WalkShared *>(pst), o, d, tn, tf, a.ev_off + (uint32_t)slot, n_ev,
-                     kb, cut, lim, lane_ok);
+        if (sc.has_tree && !tile_walk<K>(a, sc, valid, *reinterpret_cast<WalkShared *>(pst), o, d, tn, tf,
+                                         a.ev_off + (uint32_t)slot, n_ev, kb, cut, lim, lane_ok)) {
+            // a bundle that cannot be walked: its rays trace the round on their own, here or one to a warp
+            if (PASS == PASS_FWD && a.left) {
+                if ((threadIdx.x & 31) == 0) a.left[atomicAdd(a.queue + 4, 1u)] = reinterpret_cast<WalkShared *>(pst)->item;
+                return;
+            }
+            lane_ok = false;
+        }
     } else {
         packet_round<K, FORM, INSTR>(a, sc, valid, pst, o, d, inv, inv_len, tn, tf, tn, GRTX_NONE,
                                      a.traversal == GRTX_TRAVERSAL_CHECKPOINT, a.ck1_off + (uint32_t)slot, n_dst,
@@ -2021,6 +2047,30 @@ __device__ __forceinline__ void discard_dead_lists(const TraceArgs &a, int warp_
 // memory per block allows 6; the backward keeps more live state and prefers 7).
 __host__ __device__ constexpr int trace_min_blocks(int k, bool bwd) { return k >= 32 ? 6 : (bwd ? 7 : 8); }
 
+// Item of lane `lane` of the part of a tile that starts at queue place base: an 8x4 tile is taken
+// in parts of 4x4, 4x2 or 2x2 pixels.
+__device__ __forceinline__ unsigned split_item(const TraceArgs &a, unsigned base, int lane)
+{
+    if (a.split == 0 || a.cam.tiles_x == 0) return base + (unsigned)lane;
+    const unsigned part = (base & 31u) >> (5 - a.split), l = (unsigned)lane;
+    const unsigned wx = a.split == 3 ? 1u : 2u;                              // log2 of a part's width
+    const unsigned px = 3u - wx, x = ((part & ((1u << px) - 1u)) << wx) + (l & ((1u << wx) - 1u));
+    const unsigned hy = a.split == 1 ? 2u : 1u;                              // log2 of a part's height
+    const unsigned y = ((part >> px) << hy) + (l >> wx);
+    return (base & ~31u) + y * 8u + x;
+}
+
+// How finely a launch of `tiles` 32-ray tiles is split over `warps` resident warps: halves, quarters
+// or eighths of a tile while there are warps for them, since a tile's time is one warp's serial work.
+// (256x256 preview 716 -> 553 us, 64x64 56 -> 45 us; the last part of the range, 1.25 tiles a warp,
+// still gains: the parts differ more in time than a quarter.)
+inline int split_for(unsigned tiles, unsigned warps)
+{
+    int s = 0;
+    while (s < 3 && ((uint64_t)tiles << (s + 1)) <= (uint64_t)warps + warps / 4) ++s;
+    return s;
+}
+
 // Traversal a frame kernel is compiled for: either (chosen per launch by a.traversal), or one
 // of them only. The forward sphere-form kernel has one instantiation per traversal (TRAV_CKPT
 // also serves any traversal but restart): without the other traversal's code, the register
@@ -2041,13 +2091,15 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, PASS == PASS_BWD))
     unsigned rays = 0;
     for (;;) {
         unsigned base = 0;
-        if (lane == 0) base = atomicAdd(a.queue, 32u);
+        const int take = 32 >> a.split;
+        if (lane == 0) base = atomicAdd(a.queue, (unsigned)take);
         base = __shfl_sync(0xffffffffu, base, 0);
         if (base >= a.n_items) break;
         int64_t pix;
         float3 o, d;
         float tn, tf;
-        bool valid = make_ray(a.cam, base + lane, pix, o, d, tn, tf);
+        bool valid = lane < take && make_ray(a.cam, split_item(a, base, lane), pix, o, d, tn, tf);
+        if (PASS == PASS_FWD && FORM == FORM_SPHERE && lane == 0) reinterpret_cast<WalkShared *>(s_pst[threadIdx.x >> 5])->item = base;
         rays += valid;
         if (INSTR) visits_begin(a, cnt, valid, pix);
         if constexpr (TRAV == TRAV_RESTART && PASS != PASS_BWD)
@@ -2075,6 +2127,190 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, PASS == PASS_BWD))
             for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
             if (lane == 0 && x) atomicAdd((&a.stats->rays) + q, x);
         }
+    }
+}
+
+// The walk of one ray: every lane holds it, the lanes expand its pending nodes and take its leaves
+// through the exact test side by side, and lane 0 collects the hits (its k-buffer and eviction list).
+// False if the stack or the eviction list is too small.
+template <int K>
+__device__ __forceinline__ bool ray_walk(const TraceArgs &a, const SceneRef &sc, WalkShared &w, float3 o, float3 d, float tn,
+                                         float tf, uint32_t ev, int &n_ev, KBuf<K> &kb, Cut &cut, float &lim)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const uint32_t S = (uint32_t)a.n_slots;
+    uint2 *const L = a.ck0;
+    const float3 inv = make_float3(safe_rcp(d.x), safe_rcp(d.y), safe_rcp(d.z));
+    kb.clear();
+    cut.clear();
+    lim = GRTX_INF;
+    n_ev = 0;
+    float bound = tf;
+    int squeeze_at = min(kSqueeze, max(a.evict_cap - 31, 1));
+    bool ok = true;
+    const int cap = a.packet_stack < kPacketStack ? a.packet_stack : kWalkStack, wide = cap - kWalkReserve;
+    int sp = 1, nl = 0;
+    __syncwarp();
+    if (lane == 0) w.stack[0] = 0u;
+    __syncwarp();
+    for (;;) {
+        if (sp >= cap || !__all_sync(full, ok)) return false;        // no room for children or hits
+        const int p = min(min(32, sp), max(1, wide - sp));
+        uint32_t cn = GRTX_NONE, cf = GRTX_NONE;
+        if (lane < p) {
+            const float4 *nd = sc.nodes + 4 * (size_t)w.stack[sp - 1 - lane];
+            const float4 n0 = __ldg(nd), n1 = __ldg(nd + 1), n2 = __ldg(nd + 2), n3 = __ldg(nd + 3);
+            float e0, x0, e1, x1;
+            slab(n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, o, inv, tn, bound, e0, x0);
+            slab(n1.z, n1.w, n2.x, n2.y, n2.z, n2.w, o, inv, tn, bound, e1, x1);
+            cn = e0 <= x0 ? __float_as_uint(n3.x) : GRTX_NONE;
+            cf = e1 <= x1 ? __float_as_uint(n3.y) : GRTX_NONE;
+            if (e1 < e0) {
+                const uint32_t t = cn; cn = cf; cf = t;
+            }
+        }
+        __syncwarp();
+        const bool ln = cn != GRTX_NONE && (cn & GRTX_LEAF), lf = cf != GRTX_NONE && (cf & GRTX_LEAF);
+        const unsigned bn = __ballot_sync(full, cn != GRTX_NONE && !ln), bf = __ballot_sync(full, cf != GRTX_NONE && !lf);
+        const unsigned gn = __ballot_sync(full, ln), gf = __ballot_sync(full, lf);
+        const unsigned below = (1u << lane) - 1u, above = ~(below | (1u << lane));
+        sp -= p;
+        int at = sp + __popc(bn & above) + __popc(bf & above);
+        if (cf != GRTX_NONE && !lf) w.stack[at++] = cf;
+        if (cn != GRTX_NONE && !ln) w.stack[at] = cn;
+        sp += __popc(bn) + __popc(bf);
+        at = nl + __popc(gn & below) + __popc(gf & below);
+        if (ln) w.leaf[at++] = cn & ~GRTX_LEAF;
+        if (lf) w.leaf[at] = cf & ~GRTX_LEAF;
+        nl += __popc(gn) + __popc(gf);
+        __syncwarp();
+        if (sp > 0 && nl < 32) continue;
+        for (int g0 = 0; g0 < nl; g0 += 32) {
+            const int m = min(32, nl - g0);
+            const uint32_t gi = w.leaf[g0 + min(lane, m - 1)];
+            const float4 *g = sc.geom + 4 * (size_t)gi;
+            const float4 r0 = __ldg(g), r1 = __ldg(g + 1), r2 = __ldg(g + 2), r3 = __ldg(g + 3);
+            float t = 0.f, D2 = 0.f, q = 0.f, u[3], aa;
+            bool hit = lane < m && sphere_candidate(r0, r1, r2, o, d, t, aa) && in_range(t, aa, tn, bound);
+            if (hit) {
+                sphere_refine(r0, r1, r2, o, d, t, D2, u);
+                hit = D2 <= 1.0f && t > tn && t <= tf && !(t > bound);
+                q = 1.0f - fminf(r3.x * exp2f(r3.y * D2), a.alpha_max);
+            }
+            for (unsigned hits = __ballot_sync(full, hit); hits; hits &= hits - 1u) {
+                const int h = __ffs(hits) - 1;
+                float ct = __shfl_sync(full, t, h);
+                const float hq = __shfl_sync(full, q, h);
+                uint32_t ci = __shfl_sync(full, gi, h);
+                if (lane == 0 && ok && !(ct > fminf(lim, cut.top(a)))) {
+                    ci = cut.take(a, hq, ci, ct);
+                    if (kb.insert(ct, ci)) {
+                        if (n_ev >= a.evict_cap) {
+                            ok = false;
+                        } else {
+                            L[ev + (uint32_t)n_ev * S] = make_uint2(__float_as_uint(ct), ci);
+                            ++n_ev;
+                        }
+                    }
+                }
+            }
+            if (n_ev >= squeeze_at && ok) {                          // (its own lane only: the others have no hits)
+                const bool no_room = n_ev + 32 > a.evict_cap;
+                bool end;
+                const float to = squeeze<K>(L + ev, S, n_ev, n_ev, kb.k,
+                                            a.id_shift && a.p_stop > 0.f ? -__log2f(a.p_stop) : GRTX_INF, no_room, end);
+                if (end) {
+                    cut.P = 0.f;
+                    cut.far = to;
+                } else if (no_room) {
+                    lim = to;
+                }
+                squeeze_at = min(n_ev + kSqueeze, max(a.evict_cap - 31, 1));
+            }
+            __syncwarp();
+            bound = __shfl_sync(full, fminf(fminf(tf, lim), cut.top(a)), 0);
+        }
+        nl = 0;
+        if (sp == 0) return __all_sync(full, ok);
+    }
+}
+
+// The rays of the bundles that k_trace left (rays that share nothing, as scattered secondary rays do),
+// one to a warp. Such a bundle traced per ray in k_trace is 32 lanes on 32 paths, about 500 steps that
+// wait for memory one after another (and 626 warps are all that 20,011 rays give); here a ray is
+// about 30 steps of up to 32 nodes, and every resident warp has one: 20,011 scattered rays over 1M
+// Gaussians, k = 32, 1.90 -> 0.53 ms. The blend spreads over the lanes too: lane j takes entry j of the
+// sorted k-buffer to its alpha and colour, then every lane composites them in order.
+template <int K>
+__global__ void __launch_bounds__(kBlock, 5) k_trace_rays(const __grid_constant__ TraceArgs a)
+{
+    const unsigned full = 0xffffffffu;
+    __shared__ uint64_t s_k[K * kBlock];
+    __shared__ WalkShared s_w[kBlock / 32];
+    const int slot = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    const uint32_t ev = a.ev_off + (uint32_t)slot;
+    const int take = 32 >> a.split;
+    const unsigned n_left = a.queue[4];
+    KBuf<K> kb;
+    kb.k = s_k + threadIdx.x;
+    const uint64_t *keys = s_k + (threadIdx.x & ~31);            // lane 0's
+    Counters cnt = {0, 0, 0, 0, 0, 0, 0, 0, 0, nullptr, 0, 0};
+    for (;;) {
+        unsigned i = 0;
+        if (lane == 0) i = atomicAdd(a.queue + 5, 1u);
+        i = __shfl_sync(full, i, 0);
+        if (i / (unsigned)take >= n_left) break;
+        int64_t pix;
+        float3 o, d;
+        float tn, tf;
+        if (!make_ray(a.cam, split_item(a, a.left[i / (unsigned)take], (int)(i % (unsigned)take)), pix, o, d, tn, tf)) continue;
+        Cut cut;
+        float lim;
+        int n_ev;
+        const bool ok = ray_walk<K>(a, a.sc, s_w[threadIdx.x >> 5], o, d, tn, tf, ev, n_ev, kb, cut, lim);
+        if (!ok || __shfl_sync(full, lim, 0) < GRTX_INF) {
+            if (lane == 0)
+                trace_ray<K, FORM_SPHERE, false, PASS_FWD>(a, a.sc, a.rgbT, slot, pix, o, d, tn, tf, kb, cnt, cut, true, ok, 0,
+                                                           n_ev, lim);
+            __syncwarp();
+            continue;
+        }
+        float C[3] = {0.f, 0.f, 0.f}, T = 1.f;
+        for (;;) {
+            const int n = __shfl_sync(full, kb.n, 0);
+            float al = 0.f;
+            float c[3] = {0.f, 0.f, 0.f};
+            if (lane < n) al = blend_terms(a, a.sc, (uint32_t)keys[lane * kBlock] >> a.id_shift, o, d, c);
+            bool done = false;
+            for (int j = 0; j < n && !done; ++j) {
+                const float aj = __shfl_sync(full, al, j), w = T * aj;
+                C[0] = fmaf(w, __shfl_sync(full, c[0], j), C[0]);
+                C[1] = fmaf(w, __shfl_sync(full, c[1], j), C[1]);
+                C[2] = fmaf(w, __shfl_sync(full, c[2], j), C[2]);
+                T *= 1.0f - aj;
+                done = T < a.T_min;
+            }
+            if (done || n < K) break;
+            __syncwarp();
+            if (lane == 0) {                                      // the next K hits from the eviction list
+                kb.clear();
+                int k = 0;
+                for (int e = 0; e < n_ev; ++e) {
+                    uint2 v = a.ck0[ev + (uint32_t)e * (uint32_t)a.n_slots];
+                    float ct = __uint_as_float(v.x);
+                    uint32_t ci = v.y;
+                    if (kb.insert(ct, ci)) {
+                        a.ck0[ev + (uint32_t)k * (uint32_t)a.n_slots] = make_uint2(__float_as_uint(ct), ci);
+                        ++k;
+                    }
+                }
+                n_ev = k;
+            }
+            __syncwarp();
+        }
+        if (lane == 0) a.rgbT[pix] = make_float4(C[0] + T * a.bg0, C[1] + T * a.bg1, C[2] + T * a.bg2, T);
+        __syncwarp();
     }
 }
 
@@ -2261,6 +2497,13 @@ int trace_launch(const TraceArgs &a, int form, bool instr, int pass, int blocks,
 }
 
 template <int K>
+int trace_rays_launch(const TraceArgs &a, int blocks, cudaStream_t s)
+{
+    k_trace_rays<K><<<blocks, kBlock, 0, s>>>(a);
+    return cudaGetLastError() == cudaSuccess ? GRTX_OK : GRTX_ERR_CUDA;
+}
+
+template <int K>
 int trace_occupancy(int form, bool instr, int pass, int *blocks_per_sm)
 {
     cudaError_t e;
@@ -2308,5 +2551,6 @@ int serve_occupancy(int *blocks_per_sm)
 #define GRTX_INSTANTIATE_TRACE(K)                                                                  \
     template int trace_launch<K>(const TraceArgs &, int, bool, int, int, cudaStream_t);           \
     template int trace_occupancy<K>(int, bool, int, int *);                                         \
+    template int trace_rays_launch<K>(const TraceArgs &, int, cudaStream_t);                        \
     template int serve_launch<K>(const TraceArgs &, const ServeSeg *, const unsigned *, int, int, cudaStream_t, ServeLive);   \
     template int serve_occupancy<K>(int *);

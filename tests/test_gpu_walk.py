@@ -113,6 +113,29 @@ def test_walk_ray_lists(built, n):
     _same(a[fine], b[fine])
 
 
+@pytest.mark.parametrize("size", [(8, 4), (64, 64), (250, 130), (300, 301), (640, 360)])
+def test_walk_of_split_tiles(built, size):
+    """Launches of few tiles split them over the resident warps, by up to eight."""
+    cam = scenes.pinhole_camera(*size, (0.5, 0.4, -2.5))
+    sc = built("surface")
+    _same(R.render(sc, cam, k=16)["rgbT"], R.render(sc, cam, k=16, traversal="restart")["rgbT"])
+
+
+@pytest.mark.parametrize("kind,opts", [("surface", {}), ("fog", {}), ("fog", dict(evict_capacity=40)),
+                                       ("surface", dict(packet_stack=2)), ("1", {})])
+@pytest.mark.parametrize("shape", [(5000, 1), (40, 30)])
+def test_walk_of_scattered_rays(built, kind, opts, shape):
+    """Ray lists whose bundles share nothing are traced one ray to a warp."""
+    n = shape[0] * shape[1]
+    rng = np.random.default_rng(n)
+    d = rng.standard_normal((n, 3))
+    rays = [torch.from_numpy(np.ascontiguousarray(x, dtype=np.float32)).cuda()
+            for x in (rng.uniform(-1, 1, (n, 3)), d, np.zeros(n), np.full(n, math.inf))]
+    cam = None if shape[1] == 1 else dict(scenes.pinhole_camera(*shape, (0.0, 0.0, -3.0)))
+    sc = built(kind)
+    _same(R.render(sc, cam, rays=rays, k=8, **opts)["rgbT"], R.render(sc, cam, rays=rays, k=8, traversal="restart")["rgbT"])
+
+
 @pytest.mark.parametrize("kind", ["surface", "fog"])
 def test_walk_in_batches_and_servers(built, kind):
     sc = built(kind)
