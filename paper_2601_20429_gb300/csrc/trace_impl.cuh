@@ -1427,11 +1427,12 @@ struct ConeTest {
 
 // Walks the bundle of the warp's valid rays (the other lanes help, and keep their rays' state).
 // lane_ok becomes false for a ray whose eviction list was too small. Returns false if the bundle was
-// left: no stack, a ray that cannot be bounded, or too little shared.
+// left: no stack, a ray that cannot be bounded, or too little shared. base: added to the leaf slots
+// (a world's objects; the state of the rays goes on from call to call).
 template <int K>
 __device__ __forceinline__ bool tile_walk(const TraceArgs &a, const SceneRef &sc, bool valid, WalkShared &w,
                                           float3 o, float3 d, float tn, float tf, uint32_t ev, int &n_ev, KBuf<K> &kb,
-                                          Cut &cut, float &lim, bool &lane_ok)
+                                          Cut &cut, float &lim, bool &lane_ok, uint32_t base = 0u)
 {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -1565,7 +1566,7 @@ __device__ __forceinline__ bool tile_walk(const TraceArgs &a, const SceneRef &sc
                 sphere_refine(r0, r1, r2, o, d, t, D2, u);
                 if (D2 <= 1.0f && t > tn && t <= tf && !(t > fminf(lim, cut.top(a)))) {
                     float ct = t;
-                    uint32_t ci = cut.add(a, g, gi, t, D2);
+                    uint32_t ci = cut.add(a, g, base + gi, t, D2);
                     if (kb.insert(ct, ci)) {
                         if (n_ev >= a.evict_cap) {
                             lane_ok = false;

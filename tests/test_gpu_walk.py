@@ -166,3 +166,18 @@ def test_walk_backward(built, kind, save):
     b = R.backward(sc, cam, r["rgbT"], up, k=8, traversal="restart")
     for name in a:
         assert float((a[name] - b[name]).norm()) <= 1e-5 * float(b[name].norm()), name
+
+
+@pytest.mark.parametrize("kind", ["surface", "fog", "1"])
+@pytest.mark.parametrize("k,opts", [(8, {}), (16, {}), (32, {}), (8, dict(evict_capacity=40)), (8, dict(evict_capacity=1)),
+                                    (16, dict(packet_stack=1)), (16, dict(T_min=0.0))])
+def test_walk_of_worlds(built, kind, k, opts):
+    """Overlapping, rotated, sheared and distant placements, walked object by object, against restart rounds."""
+    M = [np.eye(4)[:3], np.array([[0.0, -0.6, 0.0, 0.5], [0.6, 0.0, 0.1, 0.2], [0.0, 0.0, 0.8, 0.3]]),
+         np.array([[1.3, 0.0, 0.2, -0.9], [0.0, 0.7, 0.0, 0.1], [0.0, 0.0, 1.0, 1.5]]), np.eye(4)[:3] + [[0, 0, 0, 40.0]] * 3]
+    world = R.World([(built(n), m) for n, m in zip((kind, "outdoor", kind, kind), M)])
+    same = {a: v for a, v in opts.items() if a == "T_min"}
+    for cam in ("ragged", "one", "axis"):
+        _same(R.render_world(world, CAMS[cam], k=k, **opts)["rgbT"],
+              R.render_world(world, CAMS[cam], k=k, traversal="restart", **same)["rgbT"])
+    world.close()
