@@ -712,133 +712,330 @@ __global__ void k_unpack_tree(const float4 *__restrict__ nodes, int n, uint32_t 
 // ------------------------------------------------------------------------------------------
 constexpr int kPlocBlock = 256;
 constexpr int kPlocRadius = GRTX_PLOC_RADIUS;
+constexpr int kPlocTile = kPlocBlock + 4 * kPlocRadius;     // clusters a block looks at
+constexpr int kPlocSmall = 2048;           // clusters that one block finishes on its own
+constexpr int kPlocSmallThreads = 1024;
 constexpr int kPlocBatch = 8;              // rounds between host checks once few clusters are left
+constexpr int kPlocBatchBig = 4;           // the same while many are
 constexpr int kPlocBatchBelow = 65536;     // "few": below this many clusters
 
 // Surface area of the union of two boxes, 2 (ex ey + ey ez + ez ex) with every operation
 // rounded as written (no contraction), so that both members of a pair see the same value.
-__device__ __forceinline__ float ploc_area(const float *a, const float *b)
+__device__ __forceinline__ float ploc_area(const float a[6], float b0, float b1, float b2, float b3, float b4, float b5)
 {
-    float e0 = __fsub_rn(fmaxf(a[3], b[3]), fminf(a[0], b[0]));
-    float e1 = __fsub_rn(fmaxf(a[4], b[4]), fminf(a[1], b[1]));
-    float e2 = __fsub_rn(fmaxf(a[5], b[5]), fminf(a[2], b[2]));
+    float e0 = __fsub_rn(fmaxf(a[3], b3), fminf(a[0], b0));
+    float e1 = __fsub_rn(fmaxf(a[4], b4), fminf(a[1], b1));
+    float e2 = __fsub_rn(fmaxf(a[5], b5), fminf(a[2], b2));
     float s = __fmul_rn(e0, e1);
     s = __fadd_rn(s, __fmul_rn(e1, e2));
     s = __fadd_rn(s, __fmul_rn(e2, e0));
     return __fmul_rn(2.0f, s);
 }
 
-// Device loop state of the clustering: [0] clusters left m, [1] nodes made, [2] rounds run,
-// [3] error (a round that made no progress or made too many nodes). A round with m <= 1 does
-// nothing, so several rounds can be enqueued between host checks.
-enum { kPlocM = 0, kPlocMade = 1, kPlocRounds = 2, kPlocErr = 3 };
-
-__global__ void k_ploc_init(uint32_t *__restrict__ id, int n, int *__restrict__ st)
+// Nearest neighbour of cluster i among clusters max(i - radius, 0)..min(i + radius, m - 1); cluster g
+// is entry g - first of the structure-of-arrays tile sb (stride per component). Ascending j: a tie
+// keeps the lower index.
+__device__ __forceinline__ int ploc_nearest(const float *sb, int stride, int i, int m, int first)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) id[i] = GRTX_LEAF | (uint32_t)i;
-    if (i == 0) {
-        st[kPlocM] = n;
-        st[kPlocMade] = 0;
-        st[kPlocRounds] = 0;
-        st[kPlocErr] = 0;
-    }
-}
-
-__global__ void __launch_bounds__(kPlocBlock) k_ploc_nn(const float *__restrict__ cb, const int *__restrict__ st,
-                                                        int *__restrict__ nn)
-{
-    __shared__ float sb[(kPlocBlock + 2 * kPlocRadius) * 6];
-    const int m = st[kPlocM];
-    if (m <= 1) return;
-    const int b0 = blockIdx.x * kPlocBlock;
-    if (b0 >= m) return;
-    for (int t = threadIdx.x; t < (kPlocBlock + 2 * kPlocRadius) * 6; t += blockDim.x) {
-        int g = b0 - kPlocRadius + t / 6;
-        sb[t] = (g >= 0 && g < m) ? cb[6 * (size_t)g + t % 6] : 0.f;
-    }
-    __syncthreads();
-    int i = b0 + threadIdx.x;
-    if (i >= m) return;
-    const float *me = sb + 6 * (threadIdx.x + kPlocRadius);
-    int lo = max(i - kPlocRadius, 0), hi = min(i + kPlocRadius, m - 1);
+    const float *me = sb + (i - first);
+    const float a[6] = {me[0], me[stride], me[2 * stride], me[3 * stride], me[4 * stride], me[5 * stride]};
+    const int lo = max(i - kPlocRadius, 0), hi = min(i + kPlocRadius, m - 1);
     float best = INFINITY;
     int bj = -1;
     for (int j = lo; j <= hi; ++j) {
-        if (j == i) continue;
-        float a = ploc_area(me, sb + 6 * (j - b0 + kPlocRadius));
-        if (a < best) {                       // ascending j: a tie keeps the lower index
-            best = a;
+        const float *o = sb + (j - first);
+        const float d = ploc_area(a, o[0], o[stride], o[2 * stride], o[3 * stride], o[4 * stride], o[5 * stride]);
+        if (j != i && d < best) {
+            best = d;
             bj = j;
         }
     }
-    nn[i] = bj;
+    return bj;
 }
 
-// create[i]: cluster i starts a merge (mutual pair, i the lower); keep[i]: cluster i survives
-// (as itself or as the merged node); tail: the two flags of the last cluster.
-__global__ void k_ploc_flags(const int *__restrict__ nn, const int *__restrict__ st, uint32_t *__restrict__ create,
-                             uint32_t *__restrict__ keep, uint32_t *__restrict__ tail)
+// Device loop state of the clustering: [0] clusters left m, [1] nodes made, [2] rounds run, [3] error
+// (a round that made no progress or made too many nodes). Two copies: round r reads copy r & 1 and
+// writes the other, so that several rounds can be enqueued between host checks; a round with m <= 1
+// only copies. Word 8: a look-back that ran out of its bounded wait.
+enum { kPlocM = 0, kPlocMade = 1, kPlocRounds = 2, kPlocErr = 3, kPlocWait = 8, kPlocWords = 12 };
+
+// The clusters of a round: their boxes [m][6], ids (leaf with the top bit, or the node that was
+// created id-th) and numbers of nodes below them.
+struct PlocClusters {
+    float *box;
+    uint32_t *id, *size;
+};
+
+// What the rounds record of the node created k-th: its children, and at place n - 2 - k (its node
+// index) its box and the number of nodes of its subtree.
+struct PlocNodes {
+    uint32_t *lc, *rc;
+    float *box;
+    uint32_t *size;
+    int n;
+};
+
+__global__ void k_ploc_init(PlocClusters c, int n, int *__restrict__ st, unsigned *__restrict__ tickets)
 {
-    const int m = st[kPlocM];
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m <= 1 || i >= m) return;
-    int j = nn[i];
-    bool mutual = j >= 0 && nn[j] == i;
-    uint32_t c = mutual && i < j, k = !(mutual && j < i);
-    create[i] = c;
-    keep[i] = k;
-    if (i == m - 1) {
-        tail[0] = c;
-        tail[1] = k;
+    if (i < n) {
+        c.id[i] = GRTX_LEAF | (uint32_t)i;
+        c.size[i] = 0;
+    }
+    if (i < kPlocWords) st[i] = i == kPlocM ? n : 0;
+    if (i < 2) tickets[i] = 0;
+}
+
+// Cluster i of the round, merged with the mutual neighbour j > i (node k) or kept, at place w of the next.
+__device__ __forceinline__ void ploc_put(const PlocClusters &out, size_t w, const float a[6], uint32_t id, uint32_t size)
+{
+#pragma unroll
+    for (int c = 0; c < 6; ++c) out.box[6 * w + c] = a[c];
+    out.id[w] = id;
+    out.size[w] = size;
+}
+__device__ __forceinline__ void ploc_node(const PlocNodes &nd, uint32_t k, const float a[6], uint32_t l, uint32_t r,
+                                          uint32_t size)
+{
+    nd.lc[k] = l;
+    nd.rc[k] = r;
+    const size_t at = (size_t)(nd.n - 2) - k;
+    if (nd.box) {
+#pragma unroll
+        for (int c = 0; c < 6; ++c) nd.box[6 * at + c] = a[c];
+        nd.size[at] = size;
     }
 }
 
-// The round's totals (nodes created, clusters kept) and the next loop state, with the progress
-// checks: every round must merge at least one pair and keep exactly m - created clusters.
-__global__ void k_ploc_advance(const uint32_t *__restrict__ create_off, const uint32_t *__restrict__ keep_off,
-                               const uint32_t *__restrict__ tail, int n, int *__restrict__ st)
+// Exclusive scan of v over the block; total: the block's sum (the same in every thread).
+template <int THREADS>
+__device__ __forceinline__ uint64_t block_scan(uint64_t v, uint64_t *sums, uint64_t &total)
 {
-    const int m = st[kPlocM];
-    if (m <= 1 || st[kPlocErr]) return;
-    const uint32_t created = create_off[m - 1] + tail[0];
-    const uint32_t kept = keep_off[m - 1] + tail[1];
-    const int made = st[kPlocMade];
-    if (created == 0 || (int64_t)kept != (int64_t)m - created || (int64_t)made + created > n - 1) {
-        st[kPlocErr] = 1;
-        st[kPlocM] = 1;                       // stop the enqueued rounds
-        return;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint64_t x = v;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint64_t t = __shfl_up_sync(0xffffffffu, x, off);
+        if (lane >= off) x += t;
     }
-    st[kPlocMade] = made + (int)created;
-    st[kPlocM] = (int)kept;
-    st[kPlocRounds] += 1;
+    if (lane == 31) sums[wid] = x;
+    __syncthreads();
+    uint64_t before = 0;
+    total = 0;
+#pragma unroll
+    for (int q = 0; q < THREADS / 32; ++q) {
+        const uint64_t t = sums[q];
+        if (q < wid) before += t;
+        total += t;
+    }
+    __syncthreads();
+    return before + x - v;
 }
 
-__global__ void k_ploc_merge(const float *__restrict__ cb, const uint32_t *__restrict__ id, const int *__restrict__ nn,
-                             const uint32_t *__restrict__ create_off, const uint32_t *__restrict__ keep_off,
-                             const int *__restrict__ st, float *__restrict__ cb_out, uint32_t *__restrict__ id_out,
-                             uint32_t *__restrict__ lc, uint32_t *__restrict__ rc)
+// A block's entry of a round's look-back: what it holds in the top bits (0 nothing yet, 1 its own
+// counts, 2 the counts of all blocks up to it), then clusters created and clusters kept, 31 bits each.
+constexpr uint64_t kLookOwn = 1ull << 62, kLookAll = 2ull << 62, kLookCounts = kLookOwn - 1;
+constexpr int kLookWaits = 1 << 22;
+
+// One round in one launch: nearest neighbours of the block's clusters and of 16 on either side
+// (recomputed, so that mutual pairs need no second pass), flags, their scan over all blocks by
+// decoupled look-back (Merrill and Garland 2016; blocks number themselves by a ticket, so every block
+// waits only for blocks that have started), and the merged or kept clusters. Nine launches a round and
+// a host check after most of them took 71 rounds x 36 us for 1M boxes; this is one launch a round, and
+// the last rounds are k_ploc_small's. 1M Gaussians: @@BUILD@@
+__global__ void __launch_bounds__(kPlocBlock) k_ploc_round(PlocClusters in, PlocClusters out, PlocNodes nd, int *st, int parity,
+                                                           uint64_t *status, size_t n_status, unsigned *tickets)
 {
-    const int m = st[kPlocM];
-    const uint32_t node_base = (uint32_t)st[kPlocMade];
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m <= 1 || i >= m) return;
-    int j = nn[i];
-    bool mutual = j >= 0 && nn[j] == i;
-    if (mutual && j < i) return;              // merged into cluster j
-    size_t w = keep_off[i];
-    if (mutual) {
-        uint32_t k = node_base + create_off[i];
-        lc[k] = id[i];
-        rc[k] = id[j];
-        for (int c = 0; c < 3; ++c) {
-            cb_out[6 * w + c] = fminf(cb[6 * (size_t)i + c], cb[6 * (size_t)j + c]);
-            cb_out[6 * w + 3 + c] = fmaxf(cb[6 * (size_t)i + 3 + c], cb[6 * (size_t)j + 3 + c]);
+    __shared__ float sb[6 * kPlocTile];
+    __shared__ int snn[kPlocBlock + 2 * kPlocRadius];
+    __shared__ uint64_t sums[kPlocBlock / 32], s_before;
+    __shared__ unsigned s_block;
+    const int tid = threadIdx.x;
+    if (tid == 0) s_block = atomicAdd(tickets + parity, 1u);
+    __syncthreads();
+    const unsigned b = s_block;
+    const int *cur = st + 4 * parity;
+    int *nxt = st + 4 * (parity ^ 1);
+    const int m = cur[kPlocM], made = cur[kPlocMade], rounds = cur[kPlocRounds], err = cur[kPlocErr];
+    if (b == 0 && tid == 0) {
+        tickets[parity ^ 1] = 0;
+        if (m <= 1 || err) {
+            nxt[kPlocM] = m;
+            nxt[kPlocMade] = made;
+            nxt[kPlocRounds] = rounds;
+            nxt[kPlocErr] = err;
         }
-        id_out[w] = k;
-    } else {
-        for (int c = 0; c < 6; ++c) cb_out[6 * w + c] = cb[6 * (size_t)i + c];
-        id_out[w] = id[i];
+    }
+    if (m <= 1 || err) return;
+    const unsigned blocks = (unsigned)(m + kPlocBlock - 1) / kPlocBlock;
+    if (b >= blocks) return;
+    uint64_t *const look = status + (size_t)parity * n_status;
+    if (tid == 0) status[(size_t)(parity ^ 1) * n_status + b] = 0ull;      // for the next round
+    const int b0 = (int)b * kPlocBlock, first = b0 - 2 * kPlocRadius;
+    for (int e = tid; e < 6 * kPlocTile; e += kPlocBlock) {
+        const int g = first + e / 6, c = e % 6;
+        sb[c * kPlocTile + e / 6] = g >= 0 && g < m ? in.box[6 * (size_t)g + c] : 0.f;
+    }
+    __syncthreads();
+    for (int q = tid; q < kPlocBlock + 2 * kPlocRadius; q += kPlocBlock) {
+        const int i = b0 - kPlocRadius + q;
+        snn[q] = i >= 0 && i < m ? ploc_nearest(sb, kPlocTile, i, m, first) : -1;
+    }
+    __syncthreads();
+    const int i = b0 + tid, j = snn[tid + kPlocRadius];
+    const bool mutual = i < m && j >= 0 && snn[j - b0 + kPlocRadius] == i;
+    const bool create = mutual && i < j, keep = i < m && !(mutual && j < i);
+    uint64_t total;
+    const uint64_t local = block_scan<kPlocBlock>(((uint64_t)create << 31) | (uint64_t)keep, sums, total);
+    if (tid < 32) {
+        uint64_t before = 0;
+        volatile uint64_t *const lk = look;
+        if (tid == 0) {
+            if (b == 0) lk[b] = kLookAll | total;
+            else lk[b] = kLookOwn | total;
+        }
+        if (b > 0) {
+            int64_t pred = (int64_t)b - 1;
+            for (int w = 0;;) {
+                const int64_t at = pred - tid;
+                uint64_t v = kLookAll;
+                if (at >= 0) v = lk[at];
+                const unsigned none = __ballot_sync(0xffffffffu, v < kLookOwn), all = __ballot_sync(0xffffffffu, v >= kLookAll);
+                const int last = all ? __ffs(all) - 1 : 31;               // entries 0..last count
+                if (none & (0xffffffffu >> (31 - last))) {
+                    if (++w > kLookWaits) {                               // (never expected)
+                        if (tid == 0) st[kPlocWait] = 1;
+                        break;
+                    }
+                    continue;
+                }
+                uint64_t x = tid <= last ? v & kLookCounts : 0ull;
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+                before += x;
+                if (all) break;
+                pred -= 32;
+            }
+            if (tid == 0) lk[b] = kLookAll | (before + total);
+        }
+        if (tid == 0) {
+            s_before = before;
+            if (b == blocks - 1) {                                        // the next round's state
+                const int64_t created = (int64_t)((before + total) >> 31), kept = (int64_t)((before + total) & 0x7fffffffull);
+                const bool bad = created == 0 || kept != (int64_t)m - created || (int64_t)made + created > nd.n - 1;
+                nxt[kPlocM] = bad ? 1 : (int)kept;
+                nxt[kPlocMade] = bad ? made : made + (int)created;
+                nxt[kPlocRounds] = rounds + (bad ? 0 : 1);
+                nxt[kPlocErr] = bad ? 1 : 0;
+            }
+        }
+    }
+    __syncthreads();
+    if (!keep) return;
+    const uint64_t at = s_before + local;
+    const size_t w = (size_t)(at & 0x7fffffffull);
+    float a[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) a[c] = sb[c * kPlocTile + (i - first)];
+    uint32_t id = in.id[i], size = in.size[i];
+    if (create) {
+        const uint32_t k = (uint32_t)made + (uint32_t)(at >> 31);
+        if (k >= (uint32_t)(nd.n - 1)) return;                            // (the state reports it)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            a[c] = fminf(a[c], sb[c * kPlocTile + (j - first)]);
+            a[3 + c] = fmaxf(a[3 + c], sb[(3 + c) * kPlocTile + (j - first)]);
+        }
+        size += in.size[j] + 1u;
+        ploc_node(nd, k, a, id, in.id[j], size);
+        id = k;
+    }
+    ploc_put(out, w, a, id, size);
+}
+
+// All rounds from at most kPlocSmall clusters on, in one block (shared memory: boxes, neighbours). Most
+// rounds of a build have few clusters left (50 of 71 for 1M boxes), and are a few microseconds each
+// this way. With more clusters left it does nothing.
+__global__ void __launch_bounds__(kPlocSmallThreads) k_ploc_small(PlocClusters c, PlocNodes nd, int *cur)
+{
+    extern __shared__ float sb[];                 // [6][kPlocSmall] boxes, then neighbours, ids and sizes
+    int *const snn = reinterpret_cast<int *>(sb + 6 * kPlocSmall);
+    uint32_t *const sid = reinterpret_cast<uint32_t *>(snn + kPlocSmall), *const ssz = sid + kPlocSmall;
+    __shared__ uint64_t sums[kPlocSmallThreads / 32];
+    const int tid = threadIdx.x;
+    int m = cur[kPlocM], made = cur[kPlocMade], rounds = cur[kPlocRounds], err = cur[kPlocErr];
+    if (m <= 1 || m > kPlocSmall || err) return;
+    for (int e = tid; e < 6 * m; e += kPlocSmallThreads) sb[(e % 6) * kPlocSmall + e / 6] = c.box[e];
+    for (int e = tid; e < m; e += kPlocSmallThreads) {
+        sid[e] = c.id[e];
+        ssz[e] = c.size[e];
+    }
+    __syncthreads();
+    while (m > 1 && !err) {
+        for (int i = tid; i < m; i += kPlocSmallThreads) snn[i] = ploc_nearest(sb, kPlocSmall, i, m, 0);
+        __syncthreads();
+        // a thread's two clusters are neighbours, so that the scan keeps their order
+        float a[2][6];
+        uint32_t id[2], size[2];
+        bool create[2], keep[2];
+        uint64_t mine = 0;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int i = 2 * tid + q, j = i < m ? snn[i] : -1;
+            const bool mutual = j >= 0 && snn[j] == i;
+            create[q] = mutual && i < j;
+            keep[q] = i < m && !(mutual && j < i);
+            mine += ((uint64_t)create[q] << 31) | (uint64_t)keep[q];
+            if (keep[q]) {
+                id[q] = sid[i];
+                size[q] = ssz[i] + (create[q] ? ssz[j] + 1u : 0u);
+#pragma unroll
+                for (int x = 0; x < 6; ++x) a[q][x] = sb[x * kPlocSmall + i];
+                if (create[q]) {
+#pragma unroll
+                    for (int x = 0; x < 3; ++x) {
+                        a[q][x] = fminf(a[q][x], sb[x * kPlocSmall + j]);
+                        a[q][3 + x] = fmaxf(a[q][3 + x], sb[(3 + x) * kPlocSmall + j]);
+                    }
+                }
+            }
+        }
+        uint64_t total;
+        uint64_t at = block_scan<kPlocSmallThreads>(mine, sums, total);   // (ends with a barrier after the reads above)
+        const int created = (int)(total >> 31), kept = (int)(total & 0x7fffffffull);
+        if (created == 0 || kept != m - created || (int64_t)made + created > nd.n - 1) {
+            err = 1;
+            break;
+        }
+        uint32_t child[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) child[q] = create[q] ? sid[snn[2 * tid + q]] : 0u;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            if (!keep[q]) continue;
+            const int w = (int)(at & 0x7fffffffull);
+            if (create[q]) {
+                const uint32_t k = (uint32_t)made + (uint32_t)(at >> 31);
+                ploc_node(nd, k, a[q], id[q], child[q], size[q]);
+                id[q] = k;
+            }
+#pragma unroll
+            for (int x = 0; x < 6; ++x) sb[x * kPlocSmall + w] = a[q][x];
+            sid[w] = id[q];
+            ssz[w] = size[q];
+            at += ((uint64_t)create[q] << 31) | 1ull;
+        }
+        m = kept;
+        made += created;
+        ++rounds;
+        __syncthreads();
+    }
+    if (tid == 0) {
+        cur[kPlocM] = 1;
+        cur[kPlocMade] = made;
+        cur[kPlocRounds] = rounds;
+        cur[kPlocErr] = err;
     }
 }
 
@@ -864,39 +1061,29 @@ __global__ void k_ploc_finish(const uint32_t *__restrict__ lc, const uint32_t *_
 // subtree, then its right subtree), so that every subtree occupies a contiguous range of the
 // node array and a parent sits next to its left child.
 // ------------------------------------------------------------------------------------------
-__global__ void k_subtree_sizes(const uint32_t *__restrict__ left, const uint32_t *__restrict__ right,
-                                const uint32_t *__restrict__ parent, int n, uint32_t *size, uint32_t *counters)
-{
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    uint32_t node = parent[n - 1 + j];
-    while (node != GRTX_NONE) {
-        __threadfence();
-        if (atomicAdd(&counters[node], 1u) == 0u) return;   // the sibling subtree is not done yet
-        __threadfence();
-        uint32_t L = left[node], R = right[node];
-        uint32_t sl = (L & GRTX_LEAF) ? 0u : __ldcg(size + L);
-        uint32_t sr = (R & GRTX_LEAF) ? 0u : __ldcg(size + R);
-        __stcg(size + node, 1u + sl + sr);
-        node = parent[node];
-    }
-}
-
-// max_depth bounds the walk to the root (a clustering tree is no deeper than its rounds).
-__global__ void k_preorder(const uint32_t *__restrict__ left, const uint32_t *__restrict__ parent,
-                           const uint32_t *__restrict__ size, int n, int max_depth, uint32_t *__restrict__ pre)
+// max_depth bounds the walk to the root (a clustering tree is no deeper than its rounds). *depth: the
+// deepest leaf, one below the deepest node that has a leaf.
+__global__ void k_preorder(const uint32_t *__restrict__ left, const uint32_t *__restrict__ right,
+                           const uint32_t *__restrict__ parent, const uint32_t *__restrict__ size, int n, int max_depth,
+                           uint32_t *__restrict__ pre, int *__restrict__ depth)
 {
     int v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= n - 1) return;
-    uint32_t idx = 0, c = (uint32_t)v;
-    for (int guard = 0; guard <= max_depth; ++guard) {
-        uint32_t p = parent[c];
-        if (p == GRTX_NONE) break;
-        uint32_t L = left[p];
-        idx += 1u + ((L == c) ? 0u : ((L & GRTX_LEAF) ? 0u : size[L]));
-        c = p;
+    int deep = 0;
+    if (v < n - 1) {
+        uint32_t idx = 0, c = (uint32_t)v;
+        int d = 0;
+        for (; d <= max_depth; ++d) {
+            uint32_t p = parent[c];
+            if (p == GRTX_NONE) break;
+            uint32_t L = left[p];
+            idx += 1u + ((L == c) ? 0u : ((L & GRTX_LEAF) ? 0u : size[L]));
+            c = p;
+        }
+        pre[v] = idx;
+        if ((left[v] | right[v]) & GRTX_LEAF) deep = d + 1;
     }
-    pre[v] = idx;
+    deep = __reduce_max_sync(0xffffffffu, deep);
+    if ((threadIdx.x & 31) == 0 && deep) atomicMax(depth, deep);
 }
 
 __global__ void k_permute_tree(const uint32_t *__restrict__ left, const uint32_t *__restrict__ right,
@@ -914,6 +1101,26 @@ __global__ void k_permute_tree(const uint32_t *__restrict__ left, const uint32_t
     parent_out[(L & GRTX_LEAF) ? (n - 1 + (L & ~GRTX_LEAF)) : L] = d;
     parent_out[(R & GRTX_LEAF) ? (n - 1 + (R & ~GRTX_LEAF)) : R] = d;
     if (d == 0) parent_out[0] = GRTX_NONE;
+}
+
+// BVH2 nodes at their depth-first places, from a tree in its old numbering whose node boxes are known.
+__global__ void k_emit_renumbered(const uint32_t *__restrict__ left, const uint32_t *__restrict__ right,
+                                  const uint32_t *__restrict__ pre, const float *__restrict__ leaf_aabb,
+                                  const float *__restrict__ node_aabb, int n, float4 *__restrict__ nodes)
+{
+    int v = blockIdx.x * blockDim.x + threadIdx.x;
+    if (v >= n - 1) return;
+    float a[6], b[6];
+    uint32_t L = left[v], R = right[v];
+    load_box(L, leaf_aabb, node_aabb, a);
+    load_box(R, leaf_aabb, node_aabb, b);
+    L = (L & GRTX_LEAF) ? L : pre[L];
+    R = (R & GRTX_LEAF) ? R : pre[R];
+    float4 *out = nodes + 4 * (size_t)pre[v];
+    out[0] = make_float4(a[0], a[1], a[2], a[3]);
+    out[1] = make_float4(a[4], a[5], b[0], b[1]);
+    out[2] = make_float4(b[2], b[3], b[4], b[5]);
+    out[3] = make_float4(__uint_as_float(L), __uint_as_float(R), 0.f, 0.f);
 }
 
 // One-leaf scene: a root whose second child is an empty box that no ray hits.
@@ -1125,61 +1332,61 @@ int build_tree(grtx_scene *sc, Alloc &A, float *leaf_aabb, int64_t n, uint32_t *
     return GRTX_OK;
 }
 
-// PLOC tree over n >= 2 boxes in order: left/right/parent in the radix tree's layout. The loop
-// state lives on the device (k_ploc_advance). The host reads it after every round while many
-// clusters are left (a round then costs far more than the round trip), and after every
-// kPlocBatch rounds once few are left, each launch sized by the last count it read (an upper
-// bound; rounds after the last do nothing). Every round merges at least one pair, so at most
-// n - 1 rounds make progress; a round that does not fails the build.
+// PLOC tree over n >= 2 boxes in order: left/right/parent in the radix tree's layout, and with
+// node_box / node_size the nodes' boxes and subtree sizes. The loop state lives on the device. The host
+// reads it after every kPlocBatchBig rounds while many clusters are left and every kPlocBatch rounds
+// after that, each launch sized by the last count it read (an upper bound; rounds after the last do
+// nothing), with k_ploc_small behind each batch. Every round merges at least one pair, so at most n - 1
+// rounds make progress; a round that does not fails the build.
 int ploc_tree(Alloc &A, const float *leaf_aabb, int64_t n, uint32_t *left, uint32_t *right, uint32_t *parent,
-              cudaStream_t s, int *iterations)
+              cudaStream_t s, int *iterations, float *node_box = nullptr, uint32_t *node_size = nullptr)
 {
-    float *cb[2];
-    uint32_t *id[2], *create, *keep, *lc, *rc, *small;
-    int *nn, *st;
-    void *scan_tmp;
-    TRY(A.get(&cb[0], 6 * (size_t)n, true));
-    TRY(A.get(&cb[1], 6 * (size_t)n, true));
-    TRY(A.get(&id[0], n, true));
-    TRY(A.get(&id[1], n, true));
-    TRY(A.get(&nn, n, true));
-    TRY(A.get(&create, n, true));
-    TRY(A.get(&keep, n, true));
-    TRY(A.get(&lc, n - 1, true));
-    TRY(A.get(&rc, n - 1, true));
-    TRY(A.get(&small, 4, true));
-    TRY(A.get(&st, 4, true));
-    TRY(A.get((char **)&scan_tmp, grtx_scan_temp_bytes(n), true));
-    GRTX_CUDA(cudaMemcpyAsync(cb[0], leaf_aabb, sizeof(float) * 6 * (size_t)n, cudaMemcpyDeviceToDevice, s));
-    k_ploc_init<<<grtx_div_up(n, kThreads), kThreads, 0, s>>>(id[0], (int)n, st);
+    PlocClusters c[2];
+    PlocNodes nd = {nullptr, nullptr, node_box, node_size, (int)n};
+    int *st;
+    uint64_t *status;
+    unsigned *tickets;
+    const size_t n_status = (size_t)grtx_div_up(n, kPlocBlock);
+    for (int q = 0; q < 2; ++q) {
+        TRY(A.get(&c[q].box, 6 * (size_t)n, true));
+        TRY(A.get(&c[q].id, n, true));
+        TRY(A.get(&c[q].size, n, true));
+    }
+    TRY(A.get(&nd.lc, n - 1, true));
+    TRY(A.get(&nd.rc, n - 1, true));
+    TRY(A.get(&st, kPlocWords, true));
+    TRY(A.get(&tickets, 2, true));
+    TRY(A.get(&status, 2 * n_status, true));
+    const int small_bytes = 9 * kPlocSmall * (int)sizeof(float);
+    GRTX_CUDA(cudaFuncSetAttribute(k_ploc_small, cudaFuncAttributeMaxDynamicSharedMemorySize, small_bytes));
+    GRTX_CUDA(cudaMemcpyAsync(c[0].box, leaf_aabb, sizeof(float) * 6 * (size_t)n, cudaMemcpyDeviceToDevice, s));
+    GRTX_CUDA(cudaMemsetAsync(status, 0, 2 * n_status * sizeof(uint64_t), s));
+    k_ploc_init<<<std::max(grtx_div_up(n, kThreads), 1), kThreads, 0, s>>>(c[0], (int)n, st, tickets);
     int64_t m = n;                            // clusters left as last read by the host
     int cur = 0, checks = 0;
-    int h[4] = {(int)n, 0, 0, 0};
+    int h[kPlocWords] = {(int)n};
     while (m > 1) {
         if (++checks > n) return grtx_fail(GRTX_ERR_OVERFLOW_FATAL, "clustering did not converge");
-        const int rounds = m > kPlocBatchBelow ? 1 : kPlocBatch;
-        const int blocks = grtx_div_up(m, kPlocBlock);
+        const int rounds = m <= kPlocSmall ? 0 : m > kPlocBatchBelow ? kPlocBatchBig : kPlocBatch;
         for (int r = 0; r < rounds; ++r) {
-            k_ploc_nn<<<blocks, kPlocBlock, 0, s>>>(cb[cur], st, nn);
-            k_ploc_flags<<<blocks, kPlocBlock, 0, s>>>(nn, st, create, keep, small);
-            TRY(grtx_scan_exclusive(create, m, scan_tmp, s));
-            TRY(grtx_scan_exclusive(keep, m, scan_tmp, s));
-            k_ploc_merge<<<blocks, kPlocBlock, 0, s>>>(cb[cur], id[cur], nn, create, keep, st, cb[cur ^ 1],
-                                                       id[cur ^ 1], lc, rc);
-            k_ploc_advance<<<1, 1, 0, s>>>(create, keep, small, (int)n, st);
+            k_ploc_round<<<grtx_div_up(m, kPlocBlock), kPlocBlock, 0, s>>>(c[cur], c[cur ^ 1], nd, st, cur, status, n_status,
+                                                                          tickets);
             cur ^= 1;
         }
+        k_ploc_small<<<1, kPlocSmallThreads, small_bytes, s>>>(c[cur], nd, st + 4 * cur);
         GRTX_CHECK_LAUNCH("clustering");
         GRTX_CUDA(cudaMemcpyAsync(h, st, sizeof(h), cudaMemcpyDeviceToHost, s));
         GRTX_CUDA(cudaStreamSynchronize(s));
-        if (h[kPlocErr]) return grtx_fail(GRTX_ERR_OVERFLOW_FATAL, "clustering made no progress");
-        if ((int64_t)h[kPlocM] >= m) return grtx_fail(GRTX_ERR_OVERFLOW_FATAL, "clustering made no progress");
-        m = h[kPlocM];
+        const int *now = h + 4 * cur;
+        if (now[kPlocErr] || h[kPlocWait]) return grtx_fail(GRTX_ERR_OVERFLOW_FATAL, "clustering made no progress");
+        if ((int64_t)now[kPlocM] >= m) return grtx_fail(GRTX_ERR_OVERFLOW_FATAL, "clustering made no progress");
+        m = now[kPlocM];
     }
-    if (h[kPlocMade] != n - 1) return grtx_fail(GRTX_ERR_OVERFLOW_FATAL, "clustering made a wrong number of nodes");
-    k_ploc_finish<<<grtx_div_up(n - 1, kThreads), kThreads, 0, s>>>(lc, rc, (int)n, left, right, parent);
+    if (h[4 * cur + kPlocMade] != n - 1)
+        return grtx_fail(GRTX_ERR_OVERFLOW_FATAL, "clustering made a wrong number of nodes");
+    k_ploc_finish<<<grtx_div_up(n - 1, kThreads), kThreads, 0, s>>>(nd.lc, nd.rc, (int)n, left, right, parent);
     GRTX_CHECK_LAUNCH("clustering finish");
-    if (iterations) *iterations = h[kPlocRounds];
+    if (iterations) *iterations = h[4 * cur + kPlocRounds];
     return GRTX_OK;
 }
 
@@ -1198,37 +1405,49 @@ int finish_tree(grtx_scene *sc, Alloc &A, const float *leaf_aabb_sorted, int64_t
     } else {
         uint32_t *left, *right, *parent, *cnt;
         float *node_aabb, *node_slack = nullptr;
-        if (leaf_slack) TRY(A.get(&node_slack, n - 1, true));
         TRY(A.get(&left, n - 1, true));
         TRY(A.get(&right, n - 1, true));
         TRY(A.get(&parent, 2 * n - 1, true));
-        TRY(A.get(&cnt, n - 1, true));
         TRY(A.get(&node_aabb, 6 * (n - 1), true));
-        GRTX_CUDA(cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * (n - 1), s));
+        const int node_blocks = grtx_div_up(n - 1, kThreads);
+        bool known = false;                       // the nodes are written
         if (builder == GRTX_BUILDER_PLOC) {
             // clustering numbers nodes by creation round, scattering subtrees over the array:
-            // renumber them depth-first for locality
-            uint32_t *l0, *r0, *p0, *sz, *pre;
-            TRY(A.get(&l0, n - 1, true));
-            TRY(A.get(&r0, n - 1, true));
-            TRY(A.get(&p0, 2 * n - 1, true));
+            // renumber them depth-first for locality. It knows the nodes' boxes and subtree sizes.
+            uint32_t *sz, *pre;
             TRY(A.get(&sz, n - 1, true));
             TRY(A.get(&pre, n - 1, true));
             int rounds = 0;
-            TRY(ploc_tree(A, leaf_aabb_sorted, n, l0, r0, p0, s, &rounds));
-            k_subtree_sizes<<<grtx_div_up(n, kThreads), kThreads, 0, s>>>(l0, r0, p0, (int)n, sz, cnt);
-            k_preorder<<<grtx_div_up(n - 1, kThreads), kThreads, 0, s>>>(l0, p0, sz, (int)n, rounds, pre);
-            k_permute_tree<<<grtx_div_up(n - 1, kThreads), kThreads, 0, s>>>(l0, r0, pre, (int)n, left, right, parent);
-            GRTX_CUDA(cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * (n - 1), s));
+            TRY(ploc_tree(A, leaf_aabb_sorted, n, left, right, parent, s, &rounds, node_aabb, sz));
+            k_preorder<<<node_blocks, kThreads, 0, s>>>(left, right, parent, sz, (int)n, rounds, pre, d_depth);
+            if (!leaf_slack) {
+                k_emit_renumbered<<<node_blocks, kThreads, 0, s>>>(left, right, pre, leaf_aabb_sorted, node_aabb, (int)n,
+                                                                   sc->nodes);
+                known = true;
+            } else {
+                uint32_t *l1, *r1, *p1;
+                TRY(A.get(&l1, n - 1, true));
+                TRY(A.get(&r1, n - 1, true));
+                TRY(A.get(&p1, 2 * n - 1, true));
+                k_permute_tree<<<node_blocks, kThreads, 0, s>>>(left, right, pre, (int)n, l1, r1, p1);
+                left = l1;
+                right = r1;
+                parent = p1;
+            }
             GRTX_CHECK_LAUNCH("depth-first renumbering");
         } else {
-            k_radix_tree<<<grtx_div_up(n - 1, kThreads), kThreads, 0, s>>>(sc->codes, (int)n, left, right, parent);
+            k_radix_tree<<<node_blocks, kThreads, 0, s>>>(sc->codes, (int)n, left, right, parent);
+            k_depth<<<grtx_div_up(n, kThreads), kThreads, 0, s>>>(parent, (int)n, d_depth);
         }
-        k_refit<<<grtx_div_up(n, kThreads), kThreads, 0, s>>>(left, right, parent, leaf_aabb_sorted, (int)n,
-                                                              node_aabb, cnt, leaf_slack, node_slack);
-        k_depth<<<grtx_div_up(n, kThreads), kThreads, 0, s>>>(parent, (int)n, d_depth);
-        k_emit_nodes<<<grtx_div_up(n - 1, kThreads), kThreads, 0, s>>>(left, right, leaf_aabb_sorted, node_aabb,
-                                                                       (int)n, sc->nodes, leaf_slack, node_slack);
+        if (!known) {
+            if (leaf_slack) TRY(A.get(&node_slack, n - 1, true));
+            TRY(A.get(&cnt, n - 1, true));
+            GRTX_CUDA(cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * (n - 1), s));
+            k_refit<<<grtx_div_up(n, kThreads), kThreads, 0, s>>>(left, right, parent, leaf_aabb_sorted, (int)n,
+                                                                  node_aabb, cnt, leaf_slack, node_slack);
+            k_emit_nodes<<<node_blocks, kThreads, 0, s>>>(left, right, leaf_aabb_sorted, node_aabb, (int)n, sc->nodes,
+                                                          leaf_slack, node_slack);
+        }
         GRTX_CHECK_LAUNCH("radix tree / refit");
     }
     int h_depth = 0;
