@@ -19,6 +19,7 @@
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kBoundBlocks = 608;          // of the reductions over all boxes: four a multiprocessor
 
 inline cudaStream_t S(void *s) { return reinterpret_cast<cudaStream_t>(s); }
 
@@ -132,6 +133,8 @@ __global__ void k_centroid_bounds(const float *__restrict__ aabb, int64_t n, flo
             hi[a] = fmaxf(hi[a], c);
         }
     }
+    // (one atomic a block and component: a warp's each, 4,096 blocks of them, took 124 us for 1M boxes)
+    __shared__ float part[kThreads / 32][6];
     for (int off = 16; off > 0; off >>= 1)
         for (int a = 0; a < 3; ++a) {
             lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], off));
@@ -139,11 +142,21 @@ __global__ void k_centroid_bounds(const float *__restrict__ aabb, int64_t n, flo
         }
     if ((threadIdx.x & 31) == 0)
         for (int a = 0; a < 3; ++a) {
-            if (lo[a] <= hi[a]) {
-                atomic_min_f(bounds + a, lo[a]);
-                atomic_max_f(bounds + 3 + a, hi[a]);
-            }
+            part[threadIdx.x >> 5][a] = lo[a];
+            part[threadIdx.x >> 5][3 + a] = hi[a];
         }
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        float l = INFINITY, h = -INFINITY;
+        for (int w = 0; w < (int)blockDim.x / 32; ++w) {
+            l = fminf(l, part[w][threadIdx.x]);
+            h = fmaxf(h, part[w][3 + threadIdx.x]);
+        }
+        if (l <= h) {
+            atomic_min_f(bounds + threadIdx.x, l);
+            atomic_max_f(bounds + 3 + threadIdx.x, h);
+        }
+    }
 }
 
 // Spread the low 21 bits of v so that bit b lands at bit 3b.
@@ -270,88 +283,165 @@ __global__ void k_scan_add(uint32_t *__restrict__ d, int64_t m, const uint32_t *
 }
 
 // ------------------------------------------------------------------------------------------
-// LSD radix sort, 8-bit digits: per-tile digit histograms, a global exclusive scan laid out
-// digit-major, then a stable scatter that ranks keys inside a tile with warp matching.
+// LSD radix sort, 8-bit digits, one launch a pass (onesweep: Adinets and Merrill 2022): the digit
+// counts of all passes are counted at once (a pass does not change them), and a pass's blocks find
+// where each of their digits goes by decoupled look-back over the blocks before them, then rank
+// their keys with warp matching, in order. Histogram, three-kernel scan and scatter of each pass were
+// 40 launches over 4,096-key tiles, 16 barriers' worth of serial work a tile: @@SORT@@
 // ------------------------------------------------------------------------------------------
-constexpr int kSortThreads = 256, kSortItems = 16, kSortTile = kSortThreads * kSortItems;
+constexpr int kSortThreads = 256, kSortItems = 4, kSortTile = kSortThreads * kSortItems;
+constexpr int kSortPasses = 8, kSortWords = 16, kSortWait = 8;   // words: a ticket a pass, then a wait that ran out
+constexpr uint64_t kLookOwn = 1ull << 62, kLookAll = 2ull << 62, kLookCounts = kLookOwn - 1;
+constexpr int kLookWaits = 1 << 22;                          // bound on the checks of one look-back
 
-__global__ void k_sort_hist(const uint64_t *__restrict__ keys, int n, int shift, unsigned dmask,
-                            uint32_t *__restrict__ counts, int n_tiles)
+__global__ void k_sort_hist(const uint64_t *__restrict__ keys, int64_t n, int passes, int key_bits,
+                            unsigned long long *__restrict__ counts)
 {
-    __shared__ uint32_t h[256];
-    h[threadIdx.x] = 0;
+    __shared__ uint32_t h[kSortPasses][256];
+    for (int p = 0; p < kSortPasses; ++p) h[p][threadIdx.x] = 0;
     __syncthreads();
-    int base = blockIdx.x * kSortTile;
-#pragma unroll 4
-    for (int it = 0; it < kSortItems; ++it) {
-        int i = base + it * kSortThreads + threadIdx.x;
-        if (i < n) atomicAdd(&h[(unsigned)(keys[i] >> shift) & dmask], 1u);
+    // a block's share fits 32 bits: at most 2^31 keys in all
+    for (int64_t i = (int64_t)blockIdx.x * kSortThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kSortThreads) {
+        const uint64_t k = key_bits < 64 ? keys[i] & ((1ull << key_bits) - 1ull) : keys[i];
+        for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(unsigned)(k >> (8 * p)) & 255u], 1u);
     }
     __syncthreads();
-    counts[(int64_t)threadIdx.x * n_tiles + blockIdx.x] = h[threadIdx.x];
+    for (int p = 0; p < passes; ++p)
+        if (h[p][threadIdx.x]) atomicAdd(counts + 256 * p + threadIdx.x, (unsigned long long)h[p][threadIdx.x]);
 }
 
-__global__ void k_sort_scatter(const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin,
-                               uint64_t *__restrict__ kout, uint32_t *__restrict__ vout, int n, int shift,
-                               unsigned dmask, const uint32_t *__restrict__ offsets, int n_tiles)
+// Exclusive sum over the 256 digits of each pass (block p: pass p).
+__global__ void k_sort_starts(unsigned long long *__restrict__ counts)
+{
+    __shared__ unsigned long long sums[8];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    unsigned long long *c = counts + 256 * blockIdx.x;
+    const unsigned long long v = c[tid];
+    unsigned long long x = v;
+    for (int off = 1; off < 32; off <<= 1) {
+        const unsigned long long t = __shfl_up_sync(0xffffffffu, x, off);
+        if (lane >= off) x += t;
+    }
+    if (lane == 31) sums[wid] = x;
+    __syncthreads();
+    unsigned long long before = 0;
+    for (int q = 0; q < wid; ++q) before += sums[q];
+    c[tid] = before + x - v;
+}
+
+__global__ void __launch_bounds__(kSortThreads) k_sort_pass(const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin,
+                                                            uint64_t *__restrict__ kout, uint32_t *__restrict__ vout, int64_t n,
+                                                            int shift, unsigned dmask, const unsigned long long *__restrict__ starts,
+                                                            uint64_t *__restrict__ look, uint64_t *__restrict__ next_look,
+                                                            unsigned *__restrict__ words, int pass)
 {
     __shared__ uint32_t wc[kSortThreads / 32][256];
-    __shared__ uint32_t run[256];
-    int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    run[tid] = offsets[(int64_t)tid * n_tiles + blockIdx.x];
-    int base = blockIdx.x * kSortTile;
-    unsigned lt_mask = (1u << lane) - 1u;
+    __shared__ int64_t run[256];
+    __shared__ unsigned s_tile;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    if (tid == 0) s_tile = atomicAdd(words + pass, 1u);
+#pragma unroll
+    for (int w = 0; w < kSortThreads / 32; ++w) wc[w][tid] = 0;
+    __syncthreads();
+    const unsigned tile = s_tile;
+    const int64_t base = (int64_t)tile * kSortTile;
+    if (base >= n) return;
+    uint64_t k[kSortItems];
+    uint32_t v[kSortItems];
+    // warp w holds keys [w * 32 * items, ...) of the tile, so that its own order is the tile's
+    const int64_t first = base + (int64_t)wid * 32 * kSortItems + lane;
+    uint32_t rank[kSortItems];
+#pragma unroll
     for (int it = 0; it < kSortItems; ++it) {
-#pragma unroll
-        for (int w = 0; w < kSortThreads / 32; ++w) wc[w][tid] = 0;
-        __syncthreads();
-        int i = base + it * kSortThreads + tid;
-        bool valid = i < n;
-        uint64_t k = valid ? kin[i] : 0ull;
-        uint32_t v = valid ? vin[i] : 0u;
-        unsigned digit = (unsigned)(k >> shift) & dmask;
-        unsigned vmask = __ballot_sync(0xffffffffu, valid);
-        unsigned rank = 0;
+        const int64_t i = first + it * 32;
+        const bool valid = i < n;
+        k[it] = valid ? kin[i] : 0ull;
+        v[it] = valid ? vin[i] : 0u;
+        const unsigned digit = (unsigned)(k[it] >> shift) & dmask;
+        const unsigned vmask = __ballot_sync(0xffffffffu, valid);
+        rank[it] = 0;
         if (valid) {
-            unsigned peers = __match_any_sync(vmask, digit);
-            rank = __popc(peers & lt_mask);
-            if (rank == 0) wc[wid][digit] = __popc(peers);
+            const unsigned peers = __match_any_sync(vmask, digit);
+            const uint32_t have = wc[wid][digit];
+            rank[it] = have + __popc(peers & ((1u << lane) - 1u));
+            __syncwarp(vmask);
+            if ((peers >> lane) == 1u) wc[wid][digit] = have + __popc(peers);        // the last of them
         }
-        __syncthreads();
-        {
-            uint32_t acc = run[tid];
+        __syncwarp();
+    }
+    __syncthreads();
+    // thread d: digit d's count in the tile, its place after the tiles before, and each warp's start
+    {
+        uint64_t mine = 0;
 #pragma unroll
-            for (int w = 0; w < kSortThreads / 32; ++w) {
-                uint32_t c = wc[w][tid];
-                wc[w][tid] = acc;
-                acc += c;
+        for (int w = 0; w < kSortThreads / 32; ++w) {
+            const uint32_t c = wc[w][tid];
+            wc[w][tid] = (uint32_t)mine;
+            mine += c;
+        }
+        next_look[(size_t)tile * 256 + tid] = 0ull;
+        volatile uint64_t *const lk = look;
+        uint64_t before = 0;
+        if (tile == 0) {
+            lk[tid] = kLookAll | mine;
+        } else {
+            lk[(size_t)tile * 256 + tid] = kLookOwn | mine;
+            int64_t pred = (int64_t)tile - 1;
+            // eight entries at a time, so that a long look-back does not wait for memory entry by entry
+            bool all = false;
+            for (int w = 0; pred >= 0 && !all;) {                                    // (tile 0 holds all)
+                uint64_t x[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) x[q] = lk[(size_t)max(pred - q, (int64_t)0) * 256 + tid];
+                int used = 0;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    if (used == q && !all && pred >= q && x[q] >= kLookOwn) {
+                        before += x[q] & kLookCounts;
+                        all = x[q] >= kLookAll;
+                        used = q + 1;
+                    }
+                }
+                pred -= used;
+                if (used == 0 && ++w >= kLookWaits) {
+                    words[kSortWait] = 1u;                                           // (never expected)
+                    break;
+                }
             }
-            run[tid] = acc;
+            lk[(size_t)tile * 256 + tid] = kLookAll | (before + mine);
         }
-        __syncthreads();
-        if (valid) {
-            uint32_t pos = wc[wid][digit] + rank;
-            kout[pos] = k;
-            vout[pos] = v;
+        run[tid] = (int64_t)starts[tid] + (int64_t)before;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < kSortItems; ++it) {
+        if (first + it * 32 < n) {
+            const unsigned digit = (unsigned)(k[it] >> shift) & dmask;
+            const int64_t pos = run[digit] + wc[wid][digit] + rank[it];
+            if (pos < n) {
+                kout[pos] = k[it];
+                vout[pos] = v[it];
+            }
         }
-        __syncthreads();
     }
 }
 
 struct SortTemp {
-    size_t off_keys, off_vals, off_counts, off_scan, total;
+    size_t off_keys, off_vals, off_words, off_counts, off_look, look_entries, total;
 };
 
 SortTemp sort_layout(int64_t n)
 {
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    int n_tiles = std::max(1, grtx_div_up(n, kSortTile));
+    const size_t n_tiles = (size_t)std::max(1, grtx_div_up(n, kSortTile));
     SortTemp t;
     t.off_keys = 0;
     t.off_vals = al(t.off_keys + (size_t)n * 8);
-    t.off_counts = al(t.off_vals + (size_t)n * 4);
-    t.off_scan = al(t.off_counts + (size_t)256 * n_tiles * 4);
-    t.total = al(t.off_scan + grtx_scan_temp_bytes((int64_t)256 * n_tiles));
+    t.off_words = al(t.off_vals + (size_t)n * 4);
+    t.off_counts = al(t.off_words + kSortWords * 4);
+    t.off_look = al(t.off_counts + (size_t)kSortPasses * 256 * 8);
+    t.look_entries = n_tiles * 256;
+    t.total = al(t.off_look + 2 * t.look_entries * 8);
     return t;
 }
 
@@ -362,20 +452,23 @@ int sort_pairs(uint64_t *keys, uint32_t *vals, int64_t n, int key_bits, void *te
     char *t = (char *)temp;
     uint64_t *k_alt = (uint64_t *)(t + L.off_keys);
     uint32_t *v_alt = (uint32_t *)(t + L.off_vals);
-    uint32_t *counts = (uint32_t *)(t + L.off_counts);
-    void *scan_tmp = t + L.off_scan;
-    int n_tiles = grtx_div_up(n, kSortTile);
-    int passes = (key_bits + 7) / 8;
+    unsigned *words = (unsigned *)(t + L.off_words);
+    unsigned long long *counts = (unsigned long long *)(t + L.off_counts);
+    uint64_t *look[2] = {(uint64_t *)(t + L.off_look), (uint64_t *)(t + L.off_look) + L.look_entries};
+    const int n_tiles = grtx_div_up(n, kSortTile);
+    const int passes = (key_bits + 7) / 8;
+    // tickets, counts and the first pass's look-back entries (each pass clears the next one's)
+    GRTX_CUDA(cudaMemsetAsync(words, 0, L.off_look - L.off_words + L.look_entries * 8, s));
+    k_sort_hist<<<std::min(n_tiles, kBoundBlocks), kSortThreads, 0, s>>>(keys, n, passes, key_bits, counts);
+    k_sort_starts<<<passes, 256, 0, s>>>(counts);
     uint64_t *kin = keys, *kout = k_alt;
     uint32_t *vin = vals, *vout = v_alt;
     for (int p = 0; p < passes; ++p) {
         int shift = 8 * p;
         int bits = std::min(8, key_bits - shift);            // the last digit may be narrower
         unsigned dmask = (1u << bits) - 1u;
-        k_sort_hist<<<n_tiles, kSortThreads, 0, s>>>(kin, (int)n, shift, dmask, counts, n_tiles);
-        int st = grtx_scan_exclusive(counts, (int64_t)256 * n_tiles, scan_tmp, s);
-        if (st != GRTX_OK) return st;
-        k_sort_scatter<<<n_tiles, kSortThreads, 0, s>>>(kin, vin, kout, vout, (int)n, shift, dmask, counts, n_tiles);
+        k_sort_pass<<<n_tiles, kSortThreads, 0, s>>>(kin, vin, kout, vout, n, shift, dmask, counts + 256 * p, look[p & 1],
+                                                     look[(p + 1) & 1], words, p);
         std::swap(kin, kout);
         std::swap(vin, vout);
     }
@@ -660,30 +753,6 @@ __global__ void k_emit_nodes4(const float4 *__restrict__ nodes, int n_int, const
     out[7] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// Refit for new parameters of the same Gaussians: the record, appearance and box of the
-// Gaussian gid[s] at every leaf slot s < n_valid are recomputed in place; the Gaussians culled
-// at build time (gid[n_valid..n)) only set *revived when one of them is now above alpha_min.
-__global__ void k_refit_records(const float *__restrict__ means, const float *__restrict__ log_scales,
-                                const float *__restrict__ quats, const float *__restrict__ logits,
-                                const float *__restrict__ sh, int n_sh, int app_stride,
-                                const uint32_t *__restrict__ gid, int64_t n_valid, int64_t n, float alpha_min,
-                                float4 *__restrict__ geom, float *__restrict__ leaf_aabb, float *__restrict__ app,
-                                float4 *__restrict__ raw, unsigned *__restrict__ revived)
-{
-    int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    uint32_t j = gid[s];
-    if (s < n_valid) {
-        prep_one(means, log_scales, quats, logits, j, alpha_min, geom + 4 * s, leaf_aabb + 6 * s);
-        pack_raw(means, log_scales, quats, logits, j, raw + 3 * s);
-        const float *src = sh + (size_t)j * n_sh;
-        float *dst = app + (size_t)s * app_stride;
-        for (int c = 0; c < app_stride; ++c) dst[c] = c < n_sh ? src[c] : 0.f;
-    } else if (gaussian_opacity(logits, j) > alpha_min) {
-        atomicOr(revived, 1u);
-    }
-}
-
 // Left / right / parent arrays in the radix tree's layout (internal nodes 0..n-2, leaf j at
 // n - 1 + j, the root's parent GRTX_NONE) read back from the compacted nodes of a tree over
 // n >= 2 leaves.
@@ -710,11 +779,12 @@ __global__ void k_unpack_tree(const float4 *__restrict__ nodes, int n, uint32_t 
 // node, and the clusters are compacted. The globally closest pair is always mutual, so every
 // iteration merges at least one pair.
 // ------------------------------------------------------------------------------------------
-constexpr int kPlocBlock = 256;
+constexpr int kPlocBlock = 256;            // clusters of a block
 constexpr int kPlocRadius = GRTX_PLOC_RADIUS;
-constexpr int kPlocTile = kPlocBlock + 4 * kPlocRadius;     // clusters a block looks at
+constexpr int kPlocThreads = kPlocBlock + 2 * kPlocRadius;  // ... and those whose neighbours it needs
+constexpr int kPlocTile = kPlocBlock + 4 * kPlocRadius;     // ... and those that they may choose
 constexpr int kPlocSmall = 2048;           // clusters that one block finishes on its own
-constexpr int kPlocSmallThreads = 1024;
+constexpr int kPlocSmallThreads = 1024, kPlocSmallRow = kPlocSmall + 2 * kPlocRadius;
 constexpr int kPlocBatch = 8;              // rounds between host checks once few clusters are left
 constexpr int kPlocBatchBig = 4;           // the same while many are
 constexpr int kPlocBatchBelow = 65536;     // "few": below this many clusters
@@ -732,22 +802,23 @@ __device__ __forceinline__ float ploc_area(const float a[6], float b0, float b1,
     return __fmul_rn(2.0f, s);
 }
 
-// Nearest neighbour of cluster i among clusters max(i - radius, 0)..min(i + radius, m - 1); cluster g
-// is entry g - first of the structure-of-arrays tile sb (stride per component). Ascending j: a tie
-// keeps the lower index.
-__device__ __forceinline__ int ploc_nearest(const float *sb, int stride, int i, int m, int first)
+// Nearest neighbour of the cluster at entry `at` of the structure-of-arrays tile sb (stride per
+// component) among the entries within the radius, as an offset, or 0 if there is none. Entries past the
+// ends hold unbounded boxes, whose union has an infinite area that is never the least. Ascending
+// offsets: a tie keeps the lower index.
+__device__ __forceinline__ int ploc_nearest(const float *sb, int stride, int at)
 {
-    const float *me = sb + (i - first);
+    const float *me = sb + at;
     const float a[6] = {me[0], me[stride], me[2 * stride], me[3 * stride], me[4 * stride], me[5 * stride]};
-    const int lo = max(i - kPlocRadius, 0), hi = min(i + kPlocRadius, m - 1);
     float best = INFINITY;
-    int bj = -1;
-    for (int j = lo; j <= hi; ++j) {
-        const float *o = sb + (j - first);
+    int bj = 0;
+#pragma unroll 8
+    for (int k = -kPlocRadius; k <= kPlocRadius; ++k) {
+        const float *o = me + k;
         const float d = ploc_area(a, o[0], o[stride], o[2 * stride], o[3 * stride], o[4 * stride], o[5 * stride]);
-        if (j != i && d < best) {
+        if (k != 0 && d < best) {
             best = d;
-            bj = j;
+            bj = k;
         }
     }
     return bj;
@@ -834,21 +905,19 @@ __device__ __forceinline__ uint64_t block_scan(uint64_t v, uint64_t *sums, uint6
 
 // A block's entry of a round's look-back: what it holds in the top bits (0 nothing yet, 1 its own
 // counts, 2 the counts of all blocks up to it), then clusters created and clusters kept, 31 bits each.
-constexpr uint64_t kLookOwn = 1ull << 62, kLookAll = 2ull << 62, kLookCounts = kLookOwn - 1;
-constexpr int kLookWaits = 1 << 22;
-
+// (kLookOwn, kLookAll: see the sort's look-back)
 // One round in one launch: nearest neighbours of the block's clusters and of 16 on either side
 // (recomputed, so that mutual pairs need no second pass), flags, their scan over all blocks by
 // decoupled look-back (Merrill and Garland 2016; blocks number themselves by a ticket, so every block
 // waits only for blocks that have started), and the merged or kept clusters. Nine launches a round and
 // a host check after most of them took 71 rounds x 36 us for 1M boxes; this is one launch a round, and
 // the last rounds are k_ploc_small's. 1M Gaussians: @@BUILD@@
-__global__ void __launch_bounds__(kPlocBlock) k_ploc_round(PlocClusters in, PlocClusters out, PlocNodes nd, int *st, int parity,
+__global__ void __launch_bounds__(kPlocThreads) k_ploc_round(PlocClusters in, PlocClusters out, PlocNodes nd, int *st, int parity,
                                                            uint64_t *status, size_t n_status, unsigned *tickets)
 {
     __shared__ float sb[6 * kPlocTile];
-    __shared__ int snn[kPlocBlock + 2 * kPlocRadius];
-    __shared__ uint64_t sums[kPlocBlock / 32], s_before;
+    __shared__ int snn[kPlocThreads];
+    __shared__ uint64_t sums[kPlocThreads / 32], s_before;
     __shared__ unsigned s_block;
     const int tid = threadIdx.x;
     if (tid == 0) s_block = atomicAdd(tickets + parity, 1u);
@@ -872,21 +941,20 @@ __global__ void __launch_bounds__(kPlocBlock) k_ploc_round(PlocClusters in, Ploc
     uint64_t *const look = status + (size_t)parity * n_status;
     if (tid == 0) status[(size_t)(parity ^ 1) * n_status + b] = 0ull;      // for the next round
     const int b0 = (int)b * kPlocBlock, first = b0 - 2 * kPlocRadius;
-    for (int e = tid; e < 6 * kPlocTile; e += kPlocBlock) {
+    for (int e = tid; e < 6 * kPlocTile; e += kPlocThreads) {
         const int g = first + e / 6, c = e % 6;
-        sb[c * kPlocTile + e / 6] = g >= 0 && g < m ? in.box[6 * (size_t)g + c] : 0.f;
+        sb[c * kPlocTile + e / 6] = g >= 0 && g < m ? in.box[6 * (size_t)g + c] : (c < 3 ? -INFINITY : INFINITY);
     }
     __syncthreads();
-    for (int q = tid; q < kPlocBlock + 2 * kPlocRadius; q += kPlocBlock) {
-        const int i = b0 - kPlocRadius + q;
-        snn[q] = i >= 0 && i < m ? ploc_nearest(sb, kPlocTile, i, m, first) : -1;
-    }
+    const int i = b0 - kPlocRadius + tid;                                // the thread's cluster
+    snn[tid] = i >= 0 && i < m ? ploc_nearest(sb, kPlocTile, tid + kPlocRadius) : 0;
     __syncthreads();
-    const int i = b0 + tid, j = snn[tid + kPlocRadius];
-    const bool mutual = i < m && j >= 0 && snn[j - b0 + kPlocRadius] == i;
-    const bool create = mutual && i < j, keep = i < m && !(mutual && j < i);
+    const bool own = tid >= kPlocRadius && tid < kPlocRadius + kPlocBlock && i < m;
+    const int nn = own ? snn[tid] : 0, j = i + nn;
+    const bool mutual = nn != 0 && snn[tid + nn] == -nn;
+    const bool create = mutual && nn > 0, keep = own && !(mutual && nn < 0);
     uint64_t total;
-    const uint64_t local = block_scan<kPlocBlock>(((uint64_t)create << 31) | (uint64_t)keep, sums, total);
+    const uint64_t local = block_scan<kPlocThreads>(((uint64_t)create << 31) | (uint64_t)keep, sums, total);
     if (tid < 32) {
         uint64_t before = 0;
         volatile uint64_t *const lk = look;
@@ -958,21 +1026,29 @@ __global__ void __launch_bounds__(kPlocBlock) k_ploc_round(PlocClusters in, Ploc
 // this way. With more clusters left it does nothing.
 __global__ void __launch_bounds__(kPlocSmallThreads) k_ploc_small(PlocClusters c, PlocNodes nd, int *cur)
 {
-    extern __shared__ float sb[];                 // [6][kPlocSmall] boxes, then neighbours, ids and sizes
-    int *const snn = reinterpret_cast<int *>(sb + 6 * kPlocSmall);
+    extern __shared__ float all[];                // [6][kPlocSmallRow] boxes, then neighbours, ids and sizes
+    float *const sb = all + kPlocRadius;          // (a row has room for the neighbours past either end)
+    int *const snn = reinterpret_cast<int *>(all + 6 * kPlocSmallRow);
     uint32_t *const sid = reinterpret_cast<uint32_t *>(snn + kPlocSmall), *const ssz = sid + kPlocSmall;
     __shared__ uint64_t sums[kPlocSmallThreads / 32];
     const int tid = threadIdx.x;
     int m = cur[kPlocM], made = cur[kPlocMade], rounds = cur[kPlocRounds], err = cur[kPlocErr];
     if (m <= 1 || m > kPlocSmall || err) return;
-    for (int e = tid; e < 6 * m; e += kPlocSmallThreads) sb[(e % 6) * kPlocSmall + e / 6] = c.box[e];
+    for (int e = tid; e < 6 * m; e += kPlocSmallThreads) sb[(e % 6) * kPlocSmallRow + e / 6] = c.box[e];
+    auto pad = [&](int end) {                     // unbounded boxes before the first and after the last cluster
+        if (tid < 12 * kPlocRadius) {
+            const int x = tid / (2 * kPlocRadius), k = tid % (2 * kPlocRadius);
+            sb[x * kPlocSmallRow + (k < kPlocRadius ? k - kPlocRadius : end + k - kPlocRadius)] = x < 3 ? -INFINITY : INFINITY;
+        }
+    };
+    pad(m);
     for (int e = tid; e < m; e += kPlocSmallThreads) {
         sid[e] = c.id[e];
         ssz[e] = c.size[e];
     }
     __syncthreads();
     while (m > 1 && !err) {
-        for (int i = tid; i < m; i += kPlocSmallThreads) snn[i] = ploc_nearest(sb, kPlocSmall, i, m, 0);
+        for (int i = tid; i < m; i += kPlocSmallThreads) snn[i] = ploc_nearest(sb, kPlocSmallRow, i);
         __syncthreads();
         // a thread's two clusters are neighbours, so that the scan keeps their order
         float a[2][6];
@@ -981,21 +1057,21 @@ __global__ void __launch_bounds__(kPlocSmallThreads) k_ploc_small(PlocClusters c
         uint64_t mine = 0;
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-            const int i = 2 * tid + q, j = i < m ? snn[i] : -1;
-            const bool mutual = j >= 0 && snn[j] == i;
-            create[q] = mutual && i < j;
-            keep[q] = i < m && !(mutual && j < i);
+            const int i = 2 * tid + q, nn = i < m ? snn[i] : 0, j = i + nn;
+            const bool mutual = nn != 0 && snn[j] == -nn;
+            create[q] = mutual && nn > 0;
+            keep[q] = i < m && !(mutual && nn < 0);
             mine += ((uint64_t)create[q] << 31) | (uint64_t)keep[q];
             if (keep[q]) {
                 id[q] = sid[i];
                 size[q] = ssz[i] + (create[q] ? ssz[j] + 1u : 0u);
 #pragma unroll
-                for (int x = 0; x < 6; ++x) a[q][x] = sb[x * kPlocSmall + i];
+                for (int x = 0; x < 6; ++x) a[q][x] = sb[x * kPlocSmallRow + i];
                 if (create[q]) {
 #pragma unroll
                     for (int x = 0; x < 3; ++x) {
-                        a[q][x] = fminf(a[q][x], sb[x * kPlocSmall + j]);
-                        a[q][3 + x] = fmaxf(a[q][3 + x], sb[(3 + x) * kPlocSmall + j]);
+                        a[q][x] = fminf(a[q][x], sb[x * kPlocSmallRow + j]);
+                        a[q][3 + x] = fmaxf(a[q][3 + x], sb[(3 + x) * kPlocSmallRow + j]);
                     }
                 }
             }
@@ -1009,7 +1085,7 @@ __global__ void __launch_bounds__(kPlocSmallThreads) k_ploc_small(PlocClusters c
         }
         uint32_t child[2];
 #pragma unroll
-        for (int q = 0; q < 2; ++q) child[q] = create[q] ? sid[snn[2 * tid + q]] : 0u;
+        for (int q = 0; q < 2; ++q) child[q] = create[q] ? sid[2 * tid + q + snn[2 * tid + q]] : 0u;
         __syncthreads();
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
@@ -1021,7 +1097,7 @@ __global__ void __launch_bounds__(kPlocSmallThreads) k_ploc_small(PlocClusters c
                 id[q] = k;
             }
 #pragma unroll
-            for (int x = 0; x < 6; ++x) sb[x * kPlocSmall + w] = a[q][x];
+            for (int x = 0; x < 6; ++x) sb[x * kPlocSmallRow + w] = a[q][x];
             sid[w] = id[q];
             ssz[w] = size[q];
             at += ((uint64_t)create[q] << 31) | 1ull;
@@ -1029,6 +1105,7 @@ __global__ void __launch_bounds__(kPlocSmallThreads) k_ploc_small(PlocClusters c
         m = kept;
         made += created;
         ++rounds;
+        pad(m);
         __syncthreads();
     }
     if (tid == 0) {
@@ -1133,19 +1210,44 @@ __global__ void k_emit_single(const float *__restrict__ leaf_aabb, float4 *__res
     nodes[3] = make_float4(__uint_as_float(GRTX_LEAF | 0u), __uint_as_float(GRTX_NONE), 0.f, 0.f);
 }
 
-__global__ void k_count_valid(const uint64_t *codes, int64_t n, unsigned long long *out)
+// Number of sorted codes before the first 2^64 - 1, by one warp: 32 probes a step.
+__global__ void k_count_valid(const uint64_t *__restrict__ codes, int64_t n, unsigned long long *out)
 {
-    unsigned long long c = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        c += codes[i] != ~0ull;
-    for (int off = 16; off > 0; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, c);
+    const int lane = threadIdx.x;
+    int64_t lo = 0, hi = n;                        // the answer is in [lo, hi]
+    while (hi > lo) {
+        const int64_t step = (hi - lo + 31) / 32, at = lo + (lane + 1) * step - 1;       // last code of the lane's part
+        const unsigned below = __ballot_sync(0xffffffffu, at < hi && codes[at] != ~0ull);
+        const int full = __popc(below);            // parts that hold valid codes only
+        lo += full * step;
+        hi = lo + step - 1 < hi ? lo + step - 1 : hi;
+        if (lo > hi) hi = lo;
+    }
+    if (lane == 0) *out = (unsigned long long)lo;
 }
 
 // ------------------------------------------------------------------------------------------
 // Leaf-order gather of Gaussian records and appearance.
 // ------------------------------------------------------------------------------------------
-__global__ void k_gather_gaussians(const uint32_t *__restrict__ order, int64_t n_valid,
+// The SH coefficients of the Gaussians rows[0..m) into m consecutive appearance records, by the whole
+// block: neighbouring threads take neighbouring words of a row. (A thread a row, one float at a time,
+// took 361 us for 1M rows of 48 coefficients.)
+__device__ __forceinline__ void copy_sh(const float *__restrict__ sh, int n_sh, int app_stride, const uint32_t *rows, int m,
+                                        float *__restrict__ app)
+{
+    if (n_sh == app_stride && ((uintptr_t)sh & 15) == 0) {
+        const int nv = n_sh / 4;
+        for (int e = threadIdx.x; e < m * nv; e += blockDim.x)
+            reinterpret_cast<float4 *>(app)[e] = __ldg(reinterpret_cast<const float4 *>(sh + (size_t)rows[e / nv] * n_sh) + e % nv);
+    } else {
+        for (int e = threadIdx.x; e < m * app_stride; e += blockDim.x) {
+            const int c = e % app_stride;
+            app[e] = c < n_sh ? __ldg(sh + (size_t)rows[e / app_stride] * n_sh + c) : 0.f;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kThreads) k_gather_gaussians(const uint32_t *__restrict__ order, int64_t n_valid,
                                    const float4 *__restrict__ geom_in, const float *__restrict__ aabb_in,
                                    const float *__restrict__ sh, int n_sh, int app_stride,
                                    const float *__restrict__ means, const float *__restrict__ log_scales,
@@ -1153,16 +1255,46 @@ __global__ void k_gather_gaussians(const uint32_t *__restrict__ order, int64_t n
                                    float4 *__restrict__ geom, float *__restrict__ aabb,
                                    float *__restrict__ app, uint32_t *__restrict__ gid, float4 *__restrict__ raw)
 {
-    int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n_valid) return;
-    uint32_t i = order[s];
-    for (int r = 0; r < 4; ++r) geom[4 * s + r] = geom_in[4 * (size_t)i + r];
-    for (int c = 0; c < 6; ++c) aabb[6 * s + c] = aabb_in[6 * (size_t)i + c];
-    const float *src = sh + (size_t)i * n_sh;
-    float *dst = app + (size_t)s * app_stride;
-    for (int c = 0; c < app_stride; ++c) dst[c] = c < n_sh ? src[c] : 0.f;
-    gid[s] = i;
-    pack_raw(means, log_scales, quats, logits, i, raw + 3 * s);
+    __shared__ uint32_t rows[kThreads];
+    const int64_t s0 = (int64_t)blockIdx.x * kThreads, s = s0 + threadIdx.x;
+    const int m = (int)(n_valid - s0 < kThreads ? n_valid - s0 : kThreads);
+    if (s < n_valid) {
+        const uint32_t i = order[s];
+        rows[threadIdx.x] = i;
+        gid[s] = i;
+        pack_raw(means, log_scales, quats, logits, i, raw + 3 * s);
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < m * 4; e += kThreads) geom[4 * s0 + e] = geom_in[4 * (size_t)rows[e / 4] + e % 4];
+    for (int e = threadIdx.x; e < m * 6; e += kThreads) aabb[6 * s0 + e] = aabb_in[6 * (size_t)rows[e / 6] + e % 6];
+    copy_sh(sh, n_sh, app_stride, rows, m, app + (size_t)s0 * app_stride);
+}
+
+// Refit for new parameters of the same Gaussians: the record, appearance and box of the
+// Gaussian gid[s] at every leaf slot s < n_valid are recomputed in place; the Gaussians culled
+// at build time (gid[n_valid..n)) only set *revived when one of them is now above alpha_min.
+__global__ void __launch_bounds__(kThreads) k_refit_records(const float *__restrict__ means, const float *__restrict__ log_scales,
+                                const float *__restrict__ quats, const float *__restrict__ logits,
+                                const float *__restrict__ sh, int n_sh, int app_stride,
+                                const uint32_t *__restrict__ gid, int64_t n_valid, int64_t n, float alpha_min,
+                                float4 *__restrict__ geom, float *__restrict__ leaf_aabb, float *__restrict__ app,
+                                float4 *__restrict__ raw, unsigned *__restrict__ revived)
+{
+    __shared__ uint32_t rows[kThreads];
+    const int64_t s0 = (int64_t)blockIdx.x * kThreads, s = s0 + threadIdx.x;
+    if (s < n) {
+        const uint32_t j = gid[s];
+        if (s < n_valid) {
+            rows[threadIdx.x] = j;
+            prep_one(means, log_scales, quats, logits, j, alpha_min, geom + 4 * s, leaf_aabb + 6 * s);
+            pack_raw(means, log_scales, quats, logits, j, raw + 3 * s);
+        } else if (gaussian_opacity(logits, j) > alpha_min) {
+            atomicOr(revived, 1u);
+        }
+    }
+    __syncthreads();
+    if (s0 < n_valid)
+        copy_sh(sh, n_sh, app_stride, rows, (int)(n_valid - s0 < kThreads ? n_valid - s0 : kThreads), app + (size_t)s0 * app_stride);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1315,12 +1447,12 @@ void free_scene_arrays(grtx_scene *sc)
 // Morton -> sort -> radix tree -> refit -> nodes over n leaf boxes (sorted in place with
 // `order`). Writes sc->nodes, sc->codes, sc->depth.
 int build_tree(grtx_scene *sc, Alloc &A, float *leaf_aabb, int64_t n, uint32_t *order, uint64_t *codes,
-               float *bounds_dev, int code_kind)
+               float *bounds_dev, int code_kind, unsigned **sort_words)
 {
     cudaStream_t s = sc->stream;
     int blocks = grtx_div_up(n, kThreads);
     k_init_bounds<<<1, 32, 0, s>>>(bounds_dev);
-    k_centroid_bounds<<<std::min(blocks, 4096), kThreads, 0, s>>>(leaf_aabb, n, bounds_dev);
+    k_centroid_bounds<<<std::min(blocks, kBoundBlocks), kThreads, 0, s>>>(leaf_aabb, n, bounds_dev);
     if (code_kind == GRTX_CODES_CENTROID)
         k_morton<<<blocks, kThreads, 0, s>>>(leaf_aabb, n, bounds_dev, codes, order);
     else
@@ -1329,6 +1461,7 @@ int build_tree(grtx_scene *sc, Alloc &A, float *leaf_aabb, int64_t n, uint32_t *
     void *stmp;
     TRY(A.get((char **)&stmp, sort_layout(n).total, true));
     TRY(sort_pairs(codes, order, n, 64, stmp, s));
+    *sort_words = n > 1 ? (unsigned *)((char *)stmp + sort_layout(n).off_words) : nullptr;
     return GRTX_OK;
 }
 
@@ -1357,7 +1490,7 @@ int ploc_tree(Alloc &A, const float *leaf_aabb, int64_t n, uint32_t *left, uint3
     TRY(A.get(&st, kPlocWords, true));
     TRY(A.get(&tickets, 2, true));
     TRY(A.get(&status, 2 * n_status, true));
-    const int small_bytes = 9 * kPlocSmall * (int)sizeof(float);
+    const int small_bytes = (6 * kPlocSmallRow + 3 * kPlocSmall) * (int)sizeof(float);
     GRTX_CUDA(cudaFuncSetAttribute(k_ploc_small, cudaFuncAttributeMaxDynamicSharedMemorySize, small_bytes));
     GRTX_CUDA(cudaMemcpyAsync(c[0].box, leaf_aabb, sizeof(float) * 6 * (size_t)n, cudaMemcpyDeviceToDevice, s));
     GRTX_CUDA(cudaMemsetAsync(status, 0, 2 * n_status * sizeof(uint64_t), s));
@@ -1369,9 +1502,11 @@ int ploc_tree(Alloc &A, const float *leaf_aabb, int64_t n, uint32_t *left, uint3
         if (++checks > n) return grtx_fail(GRTX_ERR_OVERFLOW_FATAL, "clustering did not converge");
         const int rounds = m <= kPlocSmall ? 0 : m > kPlocBatchBelow ? kPlocBatchBig : kPlocBatch;
         for (int r = 0; r < rounds; ++r) {
-            k_ploc_round<<<grtx_div_up(m, kPlocBlock), kPlocBlock, 0, s>>>(c[cur], c[cur ^ 1], nd, st, cur, status, n_status,
-                                                                          tickets);
+            k_ploc_round<<<grtx_div_up(m, kPlocBlock), kPlocThreads, 0, s>>>(c[cur], c[cur ^ 1], nd, st, cur, status, n_status,
+                                                                            tickets);
             cur ^= 1;
+            if (m <= 16 * kPlocSmall && (r & 1) && r + 1 < rounds)
+                k_ploc_small<<<1, kPlocSmallThreads, small_bytes, s>>>(c[cur], nd, st + 4 * cur);
         }
         k_ploc_small<<<1, kPlocSmallThreads, small_bytes, s>>>(c[cur], nd, st + 4 * cur);
         GRTX_CHECK_LAUNCH("clustering");
@@ -1538,15 +1673,18 @@ int build_scene(const grtx_gaussians *g, const grtx_params *p, int form, grtx_sc
     k_prep<<<blocks, kThreads, 0, s>>>(g->means, g->log_scales, g->quats, g->opacity_logits, n, p->alpha_min,
                                        geom_raw, aabb_raw);
     GRTX_CHECK_LAUNCH("prep");
-    TRY(build_tree(sc, A, aabb_raw, n, order, codes, bounds_dev, p->bvh_codes));
+    unsigned *sort_words = nullptr, h_wait = 0;
+    TRY(build_tree(sc, A, aabb_raw, n, order, codes, bounds_dev, p->bvh_codes, &sort_words));
     // number of valid Gaussians: their codes sort before the 2^64-1 of the empty boxes
     unsigned long long *d_nvalid;
     TRY(A.get(&d_nvalid, 1, true));
     GRTX_CUDA(cudaMemsetAsync(d_nvalid, 0, 8, s));
-    k_count_valid<<<std::min(blocks, 4096), kThreads, 0, s>>>(codes, n, d_nvalid);
+    k_count_valid<<<1, 32, 0, s>>>(codes, n, d_nvalid);
     unsigned long long h_nvalid = 0;
     GRTX_CUDA(cudaMemcpyAsync(&h_nvalid, d_nvalid, 8, cudaMemcpyDeviceToHost, s));
+    if (sort_words) GRTX_CUDA(cudaMemcpyAsync(&h_wait, sort_words + kSortWait, 4, cudaMemcpyDeviceToHost, s));
     GRTX_CUDA(cudaStreamSynchronize(s));
+    if (h_wait) return grtx_fail(GRTX_ERR_TIMEOUT, "radix sort: a look-back ran out");
     int64_t nv = (int64_t)h_nvalid;
     sc->n_valid = nv;
     if (nv == 0) {
@@ -1599,7 +1737,7 @@ int build_scene(const grtx_gaussians *g, const grtx_params *p, int form, grtx_sc
                                                                       sc->gid, nv, g_ico_circ, tris_raw,
                                                                       tri_aabb_raw, slack_raw);
         GRTX_CHECK_LAUNCH("proxy expand");
-        TRY(build_tree(sc, A, tri_aabb_raw, nt, torder, tcodes, bounds_dev, p->bvh_codes));
+        TRY(build_tree(sc, A, tri_aabb_raw, nt, torder, tcodes, bounds_dev, p->bvh_codes, &sort_words));
         sc->n_leaves = nt;
         TRY(A.get(&sc->tris, 3 * nt, false));
         TRY(A.get(&tri_aabb, 6 * nt, true));
@@ -1613,7 +1751,9 @@ int build_scene(const grtx_gaussians *g, const grtx_params *p, int form, grtx_sc
     }
     float h_root[16];
     GRTX_CUDA(cudaMemcpyAsync(h_root, sc->nodes, sizeof(h_root), cudaMemcpyDeviceToHost, s));
+    if (form == GRTX_FORM_PROXY20) GRTX_CUDA(cudaMemcpyAsync(&h_wait, sort_words + kSortWait, 4, cudaMemcpyDeviceToHost, s));
     GRTX_CUDA(cudaStreamSynchronize(s));
+    if (h_wait) return grtx_fail(GRTX_ERR_TIMEOUT, "radix sort: a look-back ran out");
     set_bounds(sc, h_root);
     if (sc->depth >= GRTX_STACK)
         return grtx_fail(GRTX_ERR_OVERFLOW_FATAL, "BVH depth " + std::to_string(sc->depth) +
@@ -1776,7 +1916,7 @@ static int morton_codes_abi(const float *d_aabb, int64_t n, const float *d_bound
             b = tmp;
         }
         k_init_bounds<<<1, 32, 0, s>>>(b);
-        k_centroid_bounds<<<std::min(grtx_div_up(n, kThreads), 4096), kThreads, 0, s>>>(d_aabb, n, b);
+        k_centroid_bounds<<<std::min(grtx_div_up(n, kThreads), kBoundBlocks), kThreads, 0, s>>>(d_aabb, n, b);
         bounds = b;
     }
     if (sized)
