@@ -60,7 +60,8 @@ struct TraceArgs {
     uint32_t ck1_off, ev_off;
     int n_slots;
     int split;                   // k_trace: a warp takes 32 >> split rays at a time (see split_for)
-    unsigned *left;              // bundles left for k_trace_rays: their first items (counted in queue[4]), or NULL
+    uint2 *left;                 // bundles left for k_trace_rays (counted in queue[4]), or NULL: the queue place, or
+                                 // (batched views) the first item and the view
     int discard;                 // drop dead list lines from L2 after each tile (lists 256-byte aligned)
     unsigned *queue;
     // outputs
@@ -1306,7 +1307,7 @@ struct __align__(16) WalkShared {
     uint32_t leaf[kWalkLeaves];  // gathered leaves
     float c[12];                 // per axis: origin max, 1 / direction max, origin min, 1 / direction min
     float mid[4];                // middle of the direction box, and the largest distance of a ray's direction from it
-    unsigned item;               // the bundle's place in the queue
+    uint2 place;                 // what the bundle's entry in the left list would be
     float4 off[32];              // each ray's direction minus mid (rays of one origin)
 };
 
@@ -2000,7 +2001,7 @@ __device__ __forceinline__ void trace_warp(const TraceArgs &a, const SceneRef &s
                                          a.ev_off + (uint32_t)slot, n_ev, kb, cut, lim, lane_ok)) {
             // a bundle that cannot be walked: its rays trace the round on their own, here or one to a warp
             if (PASS == PASS_FWD && a.left) {
-                if ((threadIdx.x & 31) == 0) a.left[atomicAdd(a.queue + 4, 1u)] = reinterpret_cast<WalkShared *>(pst)->item;
+                if ((threadIdx.x & 31) == 0) a.left[atomicAdd(a.queue + 4, 1u)] = reinterpret_cast<WalkShared *>(pst)->place;
                 return;
             }
             lane_ok = false;
@@ -2100,7 +2101,7 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, PASS == PASS_BWD))
         float3 o, d;
         float tn, tf;
         bool valid = lane < take && make_ray(a.cam, split_item(a, base, lane), pix, o, d, tn, tf);
-        if (PASS == PASS_FWD && FORM == FORM_SPHERE && lane == 0) reinterpret_cast<WalkShared *>(s_pst[threadIdx.x >> 5])->item = base;
+        if (PASS == PASS_FWD && FORM == FORM_SPHERE && lane == 0) reinterpret_cast<WalkShared *>(s_pst[threadIdx.x >> 5])->place = make_uint2(base, 0u);
         rays += valid;
         if (INSTR) visits_begin(a, cnt, valid, pix);
         if constexpr (TRAV == TRAV_RESTART && PASS != PASS_BWD)
@@ -2244,7 +2245,7 @@ __device__ __forceinline__ bool ray_walk(const TraceArgs &a, const SceneRef &sc,
 // Gaussians, k = 32, 1.90 -> 0.53 ms. The blend spreads over the lanes too: lane j takes entry j of the
 // sorted k-buffer to its alpha and colour, then every lane composites them in order.
 template <int K>
-__global__ void __launch_bounds__(kBlock, 5) k_trace_rays(const __grid_constant__ TraceArgs a)
+__global__ void __launch_bounds__(kBlock, 5) k_trace_rays(const __grid_constant__ TraceArgs a, const ServeSeg *segs)
 {
     const unsigned full = 0xffffffffu;
     __shared__ uint64_t s_k[K * kBlock];
@@ -2265,14 +2266,20 @@ __global__ void __launch_bounds__(kBlock, 5) k_trace_rays(const __grid_constant_
         int64_t pix;
         float3 o, d;
         float tn, tf;
-        if (!make_ray(a.cam, split_item(a, a.left[i / (unsigned)take], (int)(i % (unsigned)take)), pix, o, d, tn, tf)) continue;
+        const uint2 at = a.left[i / (unsigned)take];
+        const int r = (int)(i % (unsigned)take);
+        if (!(segs ? make_ray(segs[at.y].cam, at.x + (unsigned)r, pix, o, d, tn, tf)
+                   : make_ray(a.cam, split_item(a, at.x, r), pix, o, d, tn, tf)))
+            continue;
+        const SceneRef sc = segs ? segs[at.y].sc : a.sc;
+        float4 *const out = segs ? segs[at.y].out : a.rgbT;
         Cut cut;
         float lim;
         int n_ev;
-        const bool ok = ray_walk<K>(a, a.sc, s_w[threadIdx.x >> 5], o, d, tn, tf, ev, n_ev, kb, cut, lim);
+        const bool ok = ray_walk<K>(a, sc, s_w[threadIdx.x >> 5], o, d, tn, tf, ev, n_ev, kb, cut, lim);
         if (!ok || __shfl_sync(full, lim, 0) < GRTX_INF) {
             if (lane == 0)
-                trace_ray<K, FORM_SPHERE, false, PASS_FWD>(a, a.sc, a.rgbT, slot, pix, o, d, tn, tf, kb, cnt, cut, true, ok, 0,
+                trace_ray<K, FORM_SPHERE, false, PASS_FWD>(a, sc, out, slot, pix, o, d, tn, tf, kb, cnt, cut, true, ok, 0,
                                                            n_ev, lim);
             __syncwarp();
             continue;
@@ -2282,7 +2289,7 @@ __global__ void __launch_bounds__(kBlock, 5) k_trace_rays(const __grid_constant_
             const int n = __shfl_sync(full, kb.n, 0);
             float al = 0.f;
             float c[3] = {0.f, 0.f, 0.f};
-            if (lane < n) al = blend_terms(a, a.sc, (uint32_t)keys[lane * kBlock] >> a.id_shift, o, d, c);
+            if (lane < n) al = blend_terms(a, sc, (uint32_t)keys[lane * kBlock] >> a.id_shift, o, d, c);
             bool done = false;
             for (int j = 0; j < n && !done; ++j) {
                 const float aj = __shfl_sync(full, al, j), w = T * aj;
@@ -2310,7 +2317,7 @@ __global__ void __launch_bounds__(kBlock, 5) k_trace_rays(const __grid_constant_
             }
             __syncwarp();
         }
-        if (lane == 0) a.rgbT[pix] = make_float4(C[0] + T * a.bg0, C[1] + T * a.bg1, C[2] + T * a.bg2, T);
+        if (lane == 0) out[pix] = make_float4(C[0] + T * a.bg0, C[1] + T * a.bg1, C[2] + T * a.bg2, T);
         __syncwarp();
     }
 }
@@ -2412,6 +2419,8 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, false))
         float3 o, d;
         float tn, tf;
         bool valid = make_ray(cam, item, pix, o, d, tn, tf);
+        if (TRAV == TRAV_CKPT && a.left && lane == 0)
+            reinterpret_cast<WalkShared *>(s_pst[threadIdx.x >> 5])->place = make_uint2(item, (unsigned)lo);
         if constexpr (TRAV == TRAV_RESTART)
             trace_warp_restart<K, FORM_SPHERE, false, false>(a, sc, sg.out, slot, valid, pix, o, d, tn, tf, kb, cnt,
                                                       s_pst[threadIdx.x >> 5]);
@@ -2498,9 +2507,9 @@ int trace_launch(const TraceArgs &a, int form, bool instr, int pass, int blocks,
 }
 
 template <int K>
-int trace_rays_launch(const TraceArgs &a, int blocks, cudaStream_t s)
+int trace_rays_launch(const TraceArgs &a, const ServeSeg *segs, int blocks, cudaStream_t s)
 {
-    k_trace_rays<K><<<blocks, kBlock, 0, s>>>(a);
+    k_trace_rays<K><<<blocks, kBlock, 0, s>>>(a, segs);
     return cudaGetLastError() == cudaSuccess ? GRTX_OK : GRTX_ERR_CUDA;
 }
 
@@ -2552,6 +2561,6 @@ int serve_occupancy(int *blocks_per_sm)
 #define GRTX_INSTANTIATE_TRACE(K)                                                                  \
     template int trace_launch<K>(const TraceArgs &, int, bool, int, int, cudaStream_t);           \
     template int trace_occupancy<K>(int, bool, int, int *);                                         \
-    template int trace_rays_launch<K>(const TraceArgs &, int, cudaStream_t);                        \
+    template int trace_rays_launch<K>(const TraceArgs &, const ServeSeg *, int, cudaStream_t);                        \
     template int serve_launch<K>(const TraceArgs &, const ServeSeg *, const unsigned *, int, int, cudaStream_t, ServeLive);   \
     template int serve_occupancy<K>(int *);
