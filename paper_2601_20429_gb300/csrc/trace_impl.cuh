@@ -1119,7 +1119,8 @@ __device__ __forceinline__ bool trace_round(const TraceArgs &a, const SceneRef &
 // round from the root on its own, as after any capacity overflow in trace_ray.
 // ------------------------------------------------------------------------------------------
 constexpr int kPacketStack = GRTX_PACKET_STACK;
-constexpr int kWarpShared = 118;
+constexpr int kDiscardRows = 64;      // see discard_dead_lists
+constexpr int kWarpShared = 119;
 
 template <int K, int FORM, bool INSTR>
 __device__ __forceinline__ bool packet_round(const TraceArgs &a, const SceneRef &sc, bool valid, uint4 *pst, float3 o,
@@ -1307,6 +1308,8 @@ struct __align__(16) WalkShared {
     uint32_t leaf[kWalkLeaves];  // gathered leaves
     float c[12];                 // per axis: origin max, 1 / direction max, origin min, 1 / direction min
     float mid[4];                // middle of the direction box, and the largest distance of a ray's direction from it
+    int rows;                    // of the eviction lists that the walk's rays filled, or -1 if rays went on per ray
+    int pad;
     uint2 place;                 // what the bundle's entry in the left list would be
     float4 off[32];              // each ray's direction minus mid (rays of one origin)
 };
@@ -2001,11 +2004,16 @@ __device__ __forceinline__ void trace_warp(const TraceArgs &a, const SceneRef &s
                                          a.ev_off + (uint32_t)slot, n_ev, kb, cut, lim, lane_ok)) {
             // a bundle that cannot be walked: its rays trace the round on their own, here or one to a warp
             if (PASS == PASS_FWD && a.left) {
+                if ((threadIdx.x & 31) == 0) reinterpret_cast<WalkShared *>(pst)->rows = -1;
                 if ((threadIdx.x & 31) == 0) a.left[atomicAdd(a.queue + 4, 1u)] = reinterpret_cast<WalkShared *>(pst)->place;
                 return;
             }
             lane_ok = false;
         }
+        const int most = __reduce_max_sync(0xffffffffu, valid && (!lane_ok || lim < GRTX_INF) ? 1 << 20 : n_ev);
+        if ((threadIdx.x & 31) == 0)
+            reinterpret_cast<WalkShared *>(pst)->rows = most >= (1 << 20) ? -1 : min(most, kDiscardRows);
+        __syncwarp();
     } else {
         packet_round<K, FORM, INSTR>(a, sc, valid, pst, o, d, inv, inv_len, tn, tf, tn, GRTX_NONE,
                                      a.traversal == GRTX_TRAVERSAL_CHECKPOINT, a.ck1_off + (uint32_t)slot, n_dst,
@@ -2024,12 +2032,23 @@ __device__ __forceinline__ void trace_warp(const TraceArgs &a, const SceneRef &s
 // The first kDiscardRows rows of each list are dropped (a ray rarely writes more entries per
 // round; a row past that is only written back as before); rows past a list's capacity would
 // belong to the next list or lie past the workspace, and are skipped.
-constexpr int kDiscardRows = 64;
 
-__device__ __forceinline__ void discard_dead_lists(const TraceArgs &a, int warp_slot0)
+// After a walk only the eviction lists hold entries (rows: the longest list left, at most
+// kDiscardRows; a list that was longer before it was shortened is seldom): 16 rows at a time.
+__device__ __forceinline__ void discard_dead_lists(const TraceArgs &a, int warp_slot0, int rows)
 {
     const size_t S = (size_t)a.n_slots;
     const int lane = threadIdx.x & 31;
+    if (rows >= 0) {
+        for (int r0 = 0; r0 < rows; r0 += 16) {
+            const int row = r0 + (lane >> 1);
+            if (row < rows) {
+                const char *p = reinterpret_cast<const char *>(a.ev + (size_t)row * S + warp_slot0) + 128 * (lane & 1);
+                asm volatile("discard.global.L2 [%0], 128;" ::"l"(p) : "memory");
+            }
+        }
+        return;
+    }
 #pragma unroll
     for (int q = 0; q < (3 * kDiscardRows * 2) / 32; ++q) {
         const int l = q * 32 + lane;
@@ -2118,7 +2137,10 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, PASS == PASS_BWD))
                                              s_pst[threadIdx.x >> 5]);
         if (INSTR) visits_end(a, cnt, pix);
         __syncwarp();
-        if (a.discard) discard_dead_lists(a, slot & ~31);
+        if (a.discard) {
+            constexpr bool walks = FORM == FORM_SPHERE && !INSTR;
+            discard_dead_lists(a, slot & ~31, walks ? reinterpret_cast<WalkShared *>(s_pst[threadIdx.x >> 5])->rows : -1);
+        }
     }
     if (INSTR && a.stats) {
         unsigned long long v[11] = {rays, cnt.nodes, cnt.leaves, cnt.blended, cnt.rounds, cnt.ckpt, cnt.evictions,
@@ -2441,7 +2463,10 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, false))
             }
         }
         __syncwarp();
-        if (a.discard) discard_dead_lists(a, slot & ~31);
+        if (a.discard) {
+            constexpr bool walks = TRAV == TRAV_CKPT;
+            discard_dead_lists(a, slot & ~31, walks ? reinterpret_cast<WalkShared *>(s_pst[threadIdx.x >> 5])->rows : -1);
+        }
     }
 }
 
