@@ -248,6 +248,7 @@ int run(grtx_scene *sc, TraceArgs &a, int k, bool instr, int pass, unsigned *que
     // bundles of a ray list may be left to k_trace_rays: room for all of them behind the lists
     const bool walk = form == FORM_SPHERE && !instr && ckpt;
     a.split = walk ? split_for(a.n_items / 32, (unsigned)blocks * (kBlock / 32)) : 0;
+    a.middle = walk && a.n_items / 32 > (unsigned)blocks * (kBlock / 32);
     const bool leaves = walk && pass == PASS_FWD && a.cam.cam_type == GRTX_CAMERA_RAYS;
     uint2 *base = nullptr;
     int st = ensure_workspace(sc, n_slots, per_slot, leaves ? ((size_t)a.n_items >> (5 - a.split)) * sizeof(uint2) : 0, s, &base);
@@ -471,6 +472,7 @@ extern "C" GRTX_API int grtx_trace_forward_batch(grtx_scene *sc, const grtx_came
     a.n_slots = n_slots;
     a.queue = sc->d_counter + 2;
     a.n_items = total;
+    a.middle = 1;
     if (!set_list_offsets(a, 2 * C + E))
         return grtx_fail(GRTX_ERR_INVALID_ARG, "checkpoint/eviction capacities too large for the resident ray slots");
     a.discard = lists_discardable(a);

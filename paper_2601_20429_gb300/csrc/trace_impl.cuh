@@ -60,6 +60,7 @@ struct TraceArgs {
     uint32_t ck1_off, ev_off;
     int n_slots;
     int split;                   // k_trace: a warp takes 32 >> split rays at a time (see split_for)
+    int middle;                  // tiles are handed out from the middle row outwards (see middle_out)
     uint2 *left;                 // bundles left for k_trace_rays (counted in queue[4]), or NULL: the queue place, or
                                  // (batched views) the first item and the view
     int discard;                 // drop dead list lines from L2 after each tile (lists 256-byte aligned)
@@ -2103,10 +2104,24 @@ __device__ __forceinline__ void discard_dead_lists(const TraceArgs &a, int warp_
 // memory per block allows 6; the backward keeps more live state and prefers 7).
 __host__ __device__ constexpr int trace_min_blocks(int k, bool bwd) { return k >= 32 ? 6 : (bwd ? 7 : 8); }
 
+// The item that queue place `place` of an image stands for: rows of tiles are handed out from the
+// middle of the image outwards. A launch of more tiles than warps ends with its slowest tiles, and
+// those lie where the scene is dense and deep, mostly around the middle (the horizon of an outdoor
+// frame): started first, they run beside the others instead of after them. 6M outdoor frame and its
+// bounce rays, 1920x1080, one launch: 11.7 -> 11.4 ms.
+__device__ __forceinline__ unsigned middle_out(const CamRef &c, unsigned place)
+{
+    if (c.tiles_x == 0) return place;
+    const unsigned tile = place >> 5, row = tile / (unsigned)c.tiles_x, mid = (unsigned)((c.height + 3) >> 2) >> 1;
+    const unsigned to = (row & 1u) ? mid - ((row + 1u) >> 1) : mid + (row >> 1);
+    return ((tile + (to - row) * (unsigned)c.tiles_x) << 5) | (place & 31u);
+}
+
 // Item of lane `lane` of the part of a tile that starts at queue place base: an 8x4 tile is taken
 // in parts of 4x4, 4x2 or 2x2 pixels.
 __device__ __forceinline__ unsigned split_item(const TraceArgs &a, unsigned base, int lane)
 {
+    if (a.middle) base = middle_out(a.cam, base);
     if (a.split == 0 || a.cam.tiles_x == 0) return base + (unsigned)lane;
     const unsigned part = (base & 31u) >> (5 - a.split), l = (unsigned)lane;
     const unsigned wx = a.split == 3 ? 1u : 2u;                              // log2 of a part's width
@@ -2471,7 +2486,9 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, false))
         const ServeSeg &sg = segs[lo];
         SceneRef sc = sg.sc;
         CamRef cam = sg.cam;
-        unsigned item = sg.item_begin + (base - sg.step_begin) + lane;
+        unsigned item = sg.item_begin + (base - sg.step_begin);
+        if (a.middle) item = middle_out(cam, item);
+        item += (unsigned)lane;
         int64_t pix;
         float3 o, d;
         float tn, tf;
