@@ -354,7 +354,7 @@ GRTX_API int grtx_radix_tree(const uint64_t *d_sorted_keys, int64_t n, uint32_t 
  * compacted in order. The node created k-th becomes internal node n - 2 - k (the root is 0).
  * Writes d_left / d_right [n-1] and d_parent [2n-1] in grtx_radix_tree's layout and, if not
  * NULL, *iterations (host). Allocates scratch stream-ordered and synchronises the stream
- * once per iteration (to read how many clusters are left). Device, caller-owned. */
+ * every 4 to 8 iterations (to read how many clusters are left). Device, caller-owned. */
 GRTX_API int grtx_ploc_tree(const float *d_leaf_aabb, int64_t n, uint32_t *d_left, uint32_t *d_right,
                             uint32_t *d_parent, int *iterations, void *stream);
 
