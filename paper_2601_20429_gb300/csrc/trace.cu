@@ -245,13 +245,14 @@ int run(grtx_scene *sc, TraceArgs &a, int k, bool instr, int pass, unsigned *que
     // checkpoint: two ping-pong checkpoint lists and the eviction list; single: the hit list
     size_t C = ckpt ? a.ckpt_cap : 1, E = ckpt ? a.evict_cap : 1;
     size_t per_slot = single ? (size_t)a.ckpt_cap : 2 * C + E;
-    // bundles of a ray list may be left to k_trace_rays: room for all of them behind the lists
+    // bundles of a ray list may be left to k_trace_rays: their list lies behind the others (room for it
+    // whether this call leaves any or not, so that the workspace does not grow from call to call)
     const bool walk = form == FORM_SPHERE && !instr && ckpt;
     a.split = walk ? split_for(a.n_items / 32, (unsigned)blocks * (kBlock / 32)) : 0;
     a.middle = walk && a.n_items / 32 > (unsigned)blocks * (kBlock / 32);
     const bool leaves = walk && pass == PASS_FWD && a.cam.cam_type == GRTX_CAMERA_RAYS;
     uint2 *base = nullptr;
-    int st = ensure_workspace(sc, n_slots, per_slot, leaves ? ((size_t)a.n_items >> (5 - a.split)) * sizeof(uint2) : 0, s, &base);
+    int st = ensure_workspace(sc, n_slots, per_slot, ckpt ? kLeftCap * sizeof(uint2) : 0, s, &base);
     if (st) return st;
     a.left = leaves ? base + (size_t)n_slots * per_slot : nullptr;
     a.ck0 = base;
@@ -463,7 +464,7 @@ extern "C" GRTX_API int grtx_trace_forward_batch(grtx_scene *sc, const grtx_came
     cudaStream_t s = S(stream);
     // (a bundle that is left, as scattered bounce rays are, held its warp for as long as half the
     // launch: 6M outdoor frame and its bounce rays 13.3 -> 11.8 ms with k_trace_rays behind it)
-    st = ensure_workspace(sc, n_slots, 2 * C + E, ckpt ? (size_t)total / 32 * sizeof(uint2) : 0, s, &base);
+    st = ensure_workspace(sc, n_slots, 2 * C + E, ckpt ? kLeftCap * sizeof(uint2) : 0, s, &base);
     if (st) return st;
     a.left = ckpt ? base + (size_t)n_slots * (2 * C + E) : nullptr;
     a.ck0 = base;

@@ -1146,6 +1146,7 @@ __device__ __forceinline__ bool trace_round(const TraceArgs &a, const SceneRef &
 // round from the root on its own, as after any capacity overflow in trace_ray.
 // ------------------------------------------------------------------------------------------
 constexpr int kPacketStack = GRTX_PACKET_STACK;
+constexpr unsigned kLeftCap = 1u << 18, kLeftRoom = 1u << 15;   // bundles that a launch can leave to k_trace_rays
 constexpr int kDiscardRows = 64;      // see discard_dead_lists
 constexpr int kWarpShared = 119;
 
@@ -2038,10 +2039,15 @@ __device__ __forceinline__ void trace_warp(const TraceArgs &a, const SceneRef &s
     if (FORM == FORM_SPHERE && !INSTR && a.traversal == GRTX_TRAVERSAL_CHECKPOINT) {
         if (sc.has_tree && !tile_walk<K>(a, sc, valid, *reinterpret_cast<WalkShared *>(pst), o, d, tn, tf,
                                          a.ev_off + (uint32_t)slot, n_ev, kb, cut, lim, lane_ok)) {
-            // a bundle that cannot be walked: its rays trace the round on their own, here or one to a warp
-            if (PASS == PASS_FWD && a.left) {
-                if ((threadIdx.x & 31) == 0) reinterpret_cast<WalkShared *>(pst)->rows = -1;
-                if ((threadIdx.x & 31) == 0) a.left[atomicAdd(a.queue + 4, 1u)] = reinterpret_cast<WalkShared *>(pst)->place;
+            // a bundle that cannot be walked: its rays trace the round on their own, one to a warp where
+            // the left list has room, or here
+            // (kLeftRoom: more than the warps that can add to it after this check)
+            if (PASS == PASS_FWD && a.left &&
+                __all_sync(0xffffffffu, *reinterpret_cast<volatile unsigned *>(a.queue + 4) < kLeftCap - kLeftRoom)) {
+                if ((threadIdx.x & 31) == 0) {
+                    reinterpret_cast<WalkShared *>(pst)->rows = -1;
+                    a.left[atomicAdd(a.queue + 4, 1u)] = reinterpret_cast<WalkShared *>(pst)->place;
+                }
                 return;
             }
             lane_ok = false;
@@ -2153,7 +2159,10 @@ template <int K, int FORM, bool INSTR, int PASS, int TRAV = TRAV_ANY>
 __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, PASS == PASS_BWD)) k_trace(TraceArgs a)
 {
     __shared__ uint64_t s_k[K * kBlock];
-    __shared__ uint4 s_pst[kBlock / 32][kWarpShared];
+    // the walk's shared memory or the packet's stack (with 3 KB instead of 7.6 a block, one more block
+    // of a k = 32 restart launch fits)
+    constexpr bool walks = FORM == FORM_SPHERE && !INSTR && TRAV != TRAV_RESTART;
+    __shared__ uint4 s_pst[kBlock / 32][walks ? kWarpShared : kPacketStack];
     const int slot = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     KBuf<K> kb;
@@ -2170,7 +2179,7 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, PASS == PASS_BWD))
         float3 o, d;
         float tn, tf;
         bool valid = lane < take && make_ray(a.cam, split_item(a, base, lane), pix, o, d, tn, tf);
-        if (PASS == PASS_FWD && FORM == FORM_SPHERE && lane == 0) reinterpret_cast<WalkShared *>(s_pst[threadIdx.x >> 5])->place = make_uint2(base, 0u);
+        if (walks && PASS == PASS_FWD && lane == 0) reinterpret_cast<WalkShared *>(s_pst[threadIdx.x >> 5])->place = make_uint2(base, 0u);
         rays += valid;
         if (INSTR) visits_begin(a, cnt, valid, pix);
         if constexpr (TRAV == TRAV_RESTART && PASS != PASS_BWD)
@@ -2188,7 +2197,6 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, PASS == PASS_BWD))
         if (INSTR) visits_end(a, cnt, pix);
         __syncwarp();
         if (a.discard) {
-            constexpr bool walks = FORM == FORM_SPHERE && !INSTR;
             discard_dead_lists(a, slot & ~31, walks ? reinterpret_cast<WalkShared *>(s_pst[threadIdx.x >> 5])->rows : -1);
         }
     }
@@ -2325,7 +2333,7 @@ __global__ void __launch_bounds__(kBlock, 5) k_trace_rays(const __grid_constant_
     const int slot = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
     const uint32_t ev = a.ev_off + (uint32_t)slot;
     const int take = 32 >> a.split;
-    const unsigned n_left = a.queue[4];
+    const unsigned n_left = min(a.queue[4], kLeftCap);
     KBuf<K> kb;
     kb.k = s_k + threadIdx.x;
     const uint64_t *keys = s_k + (threadIdx.x & ~31);            // lane 0's
@@ -2454,7 +2462,8 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, false))
     k_serve(TraceArgs a, const ServeSeg *segs, const unsigned *begins, int n_segs, ServeLive live)
 {
     __shared__ uint64_t s_k[K * kBlock];
-    __shared__ uint4 s_pst[kBlock / 32][kWarpShared];
+    constexpr bool walks = TRAV == TRAV_CKPT;
+    __shared__ uint4 s_pst[kBlock / 32][walks ? kWarpShared : kPacketStack];
     const unsigned kNoWork = 0xffffffffu;
     const int slot = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
@@ -2493,7 +2502,7 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, false))
         float3 o, d;
         float tn, tf;
         bool valid = make_ray(cam, item, pix, o, d, tn, tf);
-        if (TRAV == TRAV_CKPT && a.left && lane == 0)
+        if (walks && a.left && lane == 0)
             reinterpret_cast<WalkShared *>(s_pst[threadIdx.x >> 5])->place = make_uint2(item, (unsigned)lo);
         if constexpr (TRAV == TRAV_RESTART)
             trace_warp_restart<K, FORM_SPHERE, false, false>(a, sc, sg.out, slot, valid, pix, o, d, tn, tf, kb, cnt,
@@ -2516,7 +2525,6 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, false))
         }
         __syncwarp();
         if (a.discard) {
-            constexpr bool walks = TRAV == TRAV_CKPT;
             discard_dead_lists(a, slot & ~31, walks ? reinterpret_cast<WalkShared *>(s_pst[threadIdx.x >> 5])->rows : -1);
         }
     }
