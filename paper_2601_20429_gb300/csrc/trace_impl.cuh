@@ -1321,14 +1321,18 @@ __device__ __forceinline__ bool packet_round(const TraceArgs &a, const SceneRef 
 // Why: a packet that tests one node at a time for 32 rays is a chain of about 340 node steps, 150
 // pops and 130 leaf steps a tile on the 1M surface frame, and its exact tests run with a quarter
 // of the lanes. The walk takes 27 steps, 145 filters and 51 exact tests with 23 lanes each:
-// 3.3 G instead of 7.8 G warp instructions a frame. 1920x1080, k = 16: 9.8 ms with packets and
-// per-ray later rounds, 6.8 ms with packets bounded by opacity (Cut), 3.9 ms with the walk. What
-// bounds it now: instruction issue (69 % of the slots) and the L1 pipe (70 %: each lane gathers
-// its own records and SH coefficients).
+// 2.6 G instead of 7.8 G warp instructions a frame. 1920x1080, k = 16: 9.8 ms with packets and
+// per-ray later rounds, 6.8 ms with packets bounded by opacity (Cut), 3.9 ms with the walk, 3.5 with
+// the quadratic filter below, 3.2 with 64-bit keys and 256-bit gathers. What bounds it now: the L1
+// pipe (78 %: each lane gathers its own records and SH coefficients) and instruction issue (65 %).
+// Keeping the hits' alphas instead of testing again at the blend, colours by groups of four lanes, and
+// 5 to 7 blocks an SM with the registers for it were measured: none was faster.
 // Groups of 8 or 16 rays with a stack each took 7.9 and 4.7 ms against 4.0 for one of 32.
 // ------------------------------------------------------------------------------------------
 // The stack keeps kWalkReserve entries for walking one node at a time: past kWalkStack -
 // kWalkReserve pending nodes a step takes the top one only, as a depth-first walk does.
+// (A stack of 128 with 96 leaves: preview 847 instead of 556 us, since wide tiles then walk node by
+// node; 96 leaves with this stack: frame +1 %.)
 constexpr int kWalkStack = 192, kWalkReserve = 48, kWalkLeaves = 128;
 
 struct __align__(16) WalkShared {
@@ -1403,9 +1407,13 @@ static __device__ __noinline__ float squeeze(uint2 *L, uint32_t S, int n, int &k
     return m;
 }
 
-constexpr int kSqueeze = 64;     // entries a list may grow by before it is squeezed
+// Entries a list may grow by before it is squeezed: 48 / 64 / 96 gave 3.28 / 3.25 / 3.22 ms for the
+// 1M 1080p frame (few rays ever do) and 12.0 / 11.8 / 12.2 ms for the 6M outdoor frame (fog).
+constexpr int kSqueeze = 64;
 // Work (in leaf tests; a step counts as 4) after which a walk with fewer than one candidate per
-// four is given up: its rays share almost nothing, and each traces the round on its own.
+// four is given up: its rays share almost nothing, and each traces the round on its own. Given up
+// after 128 / 256 / 512 / 1024, the 256x256 preview took 860 / 725 / 604 / 604 us (its wide tiles are
+// still far cheaper than rays on their own) and the 1080p frame 4.24 / 3.47 / 3.47 / 3.47 ms.
 constexpr int kWalkTrial = 512;
 
 // Which rays of one origin o may hit a Gaussian, as one quadratic in the ray's direction. A ray
