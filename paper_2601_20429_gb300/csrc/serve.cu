@@ -236,7 +236,7 @@ void fill_segments(grtx_server *v, SrvStep &st, const std::vector<Piece> &pieces
         g.item_begin = pc.begin;
         g.step_begin = st.n_items;
         g.count = pc.count;
-        g.pad = 0;
+        g.split = 0;
         st.h_begins[j] = st.n_items;
         st.seg_req.push_back(pc.r);
         st.seg_seen.push_back(0);

@@ -97,7 +97,8 @@ struct __align__(256) ServeSeg {
     SceneRef sc;
     CamRef cam;
     float4 *out;
-    unsigned item_begin, step_begin, count, pad;
+    unsigned item_begin, step_begin, count;
+    unsigned split;              // batched ray lists: a 32-item tile of the queue stands for 32 >> split rays
 };
 
 // Controls of a serving launch (all NULL / 0 for a plain batched launch):
@@ -2149,10 +2150,10 @@ __device__ __forceinline__ unsigned split_item(const TraceArgs &a, unsigned base
 // or eighths of a tile while there are warps for them, since a tile's time is one warp's serial work.
 // (256x256 preview 716 -> 553 us, 64x64 56 -> 45 us; the last part of the range, 1.25 tiles a warp,
 // still gains: the parts differ more in time than a quarter.)
-inline int split_for(unsigned tiles, unsigned warps)
+inline int split_for(unsigned tiles, unsigned warps, int most = 3)
 {
     int s = 0;
-    while (s < 3 && ((uint64_t)tiles << (s + 1)) <= (uint64_t)warps + warps / 4) ++s;
+    while (s < most && ((uint64_t)tiles << (s + 1)) <= (uint64_t)warps + warps / 4) ++s;
     return s;
 }
 
@@ -2179,14 +2180,16 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, PASS == PASS_BWD))
     unsigned rays = 0;
     for (;;) {
         unsigned base = 0;
-        const int take = 32 >> a.split;
+        const int take = walks ? 32 >> a.split : 32;
         if (lane == 0) base = atomicAdd(a.queue, (unsigned)take);
         base = __shfl_sync(0xffffffffu, base, 0);
         if (base >= a.n_items) break;
         int64_t pix;
         float3 o, d;
         float tn, tf;
-        bool valid = lane < take && make_ray(a.cam, split_item(a, base, lane), pix, o, d, tn, tf);
+        // (the kernels without a walk take whole tiles, and do without this arithmetic)
+        bool valid = walks ? lane < take && make_ray(a.cam, split_item(a, base, lane), pix, o, d, tn, tf)
+                           : make_ray(a.cam, base + lane, pix, o, d, tn, tf);
         if (walks && PASS == PASS_FWD && lane == 0) reinterpret_cast<WalkShared *>(s_pst[threadIdx.x >> 5])->place = make_uint2(base, 0u);
         rays += valid;
         if (INSTR) visits_begin(a, cnt, valid, pix);
@@ -2356,7 +2359,7 @@ __global__ void __launch_bounds__(kBlock, 5) k_trace_rays(const __grid_constant_
         float tn, tf;
         const uint2 at = a.left[i / (unsigned)take];
         const int r = (int)(i % (unsigned)take);
-        if (!(segs ? make_ray(segs[at.y].cam, at.x + (unsigned)r, pix, o, d, tn, tf)
+        if (!(segs ? r < (32 >> segs[at.y].split) && make_ray(segs[at.y].cam, at.x + (unsigned)r, pix, o, d, tn, tf)
                    : make_ray(a.cam, split_item(a, at.x, r), pix, o, d, tn, tf)))
             continue;
         const SceneRef sc = segs ? segs[at.y].sc : a.sc;
@@ -2505,11 +2508,12 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, false))
         CamRef cam = sg.cam;
         unsigned item = sg.item_begin + (base - sg.step_begin);
         if (a.middle) item = middle_out(cam, item);
-        item += (unsigned)lane;
+        const int take = 32 >> sg.split;
+        item = (item >> sg.split) + (unsigned)lane;
         int64_t pix;
         float3 o, d;
         float tn, tf;
-        bool valid = make_ray(cam, item, pix, o, d, tn, tf);
+        bool valid = lane < take && make_ray(cam, item, pix, o, d, tn, tf);
         if (walks && a.left && lane == 0)
             reinterpret_cast<WalkShared *>(s_pst[threadIdx.x >> 5])->place = make_uint2(item, (unsigned)lo);
         if constexpr (TRAV == TRAV_RESTART)
