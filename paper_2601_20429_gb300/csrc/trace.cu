@@ -445,10 +445,14 @@ extern "C" GRTX_API int grtx_trace_forward_batch(grtx_scene *sc, const grtx_came
     bool ckpt = a.traversal == GRTX_TRAVERSAL_CHECKPOINT;
     // Short ray lists go in bundles of 16 or 8 rays: bounce rays share little, and a wide bundle of 32
     // holds its warp longer than the rest of the launch takes (6 M Gaussians at 1080p with 70,354 bounce
-    // rays in one launch: 13.6 ms in bundles of 32, 9.5 ms so).
+    // rays in one launch: 13.6 ms in bundles of 32, 9.5 ms so). Not where the launch has fewer tiles
+    // than warps: there the whole tiles of the image take as long, beside more bundles (a small image
+    // with its bounce rays: 233 us, 248 us with the split).
+    const unsigned warps = (unsigned)blocks * (kBlock / 32);
+    const bool fills = all / 32 > warps;
     for (int i = 0; i < n_cams; ++i)
-        if (ckpt && v[i].cam.cam_type == GRTX_CAMERA_RAYS && v[i].cam.tiles_x == 0) {
-            v[i].split = (unsigned)split_for(items[i] / 32, 2u * (unsigned)blocks * (kBlock / 32), 2);
+        if (ckpt && fills && v[i].cam.cam_type == GRTX_CAMERA_RAYS && v[i].cam.tiles_x == 0) {
+            v[i].split = (unsigned)split_for(items[i] / 32, 2u * warps, 2);
             if (all + ((uint64_t)items[i] << v[i].split) - items[i] >= (1ull << 31)) v[i].split = 0;
             all += ((uint64_t)items[i] << v[i].split) - items[i];
             items[i] <<= v[i].split;

@@ -153,15 +153,16 @@ def test_walk_in_batches_and_servers(built, kind):
 
 @pytest.mark.parametrize("n", [1, 33, 900, 5001])
 @pytest.mark.parametrize("opts", [{}, dict(evict_capacity=40), dict(packet_stack=2)])
-def test_walk_of_lists_in_batches(built, n, opts):
-    """Short ray lists beside a camera in one launch (split into smaller bundles, scattered ones left to the
-    one-ray kernel)."""
+@pytest.mark.parametrize("image", [CAMS["ragged"], scenes.pinhole_camera(701, 401, (0.3, 0.2, -3.5), (0, 0, 0), 60.0)])
+def test_walk_of_lists_in_batches(built, n, opts, image):
+    """Short ray lists beside an image in one launch (beside one that fills the GPU in smaller bundles;
+    scattered ones left to the one-ray kernel)."""
     sc = built("surface")
     rng = np.random.default_rng(n)
     near = rng.uniform(-0.02, 0.02, (n, 3)) + [0.0, 0.0, 1.0]
     lists = [tuple(torch.from_numpy(np.ascontiguousarray(x, dtype=np.float32)).cuda() for x in (o, d, np.full(n, 1e-3), np.full(n, 9.0)))
              for o, d in ((rng.uniform(-2, 2, (n, 3)), rng.standard_normal((n, 3))), (np.tile([0.1, 0.2, -3.0], (n, 1)), near))]
-    views = [(CAMS["ragged"], None), (None, lists[0]), (None, lists[1])]
+    views = [(image, None), (None, lists[0]), (None, lists[1])]
     outs = R.render_batch(sc, views, k=8, **opts)
     for (cam, rays), a in zip(views, outs):
         _same(a, R.render(sc, cam, rays=rays, k=8, traversal="restart")["rgbT"])
