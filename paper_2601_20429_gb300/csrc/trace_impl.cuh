@@ -1427,7 +1427,8 @@ constexpr int kWalkTrial = 512;
 // divided by |A mid|^2. Each lane sets up one leaf (about 150 instructions), then every ray costs 9
 // FMAs a leaf instead of the 45 of sphere_candidate. The test only filters, so it is widened by its
 // rounding: |o_l| and d_l err by up to e = 2e-6 |A| |o - mu| in units of the sphere (taken as 32 ulp
-// of the products), and the sum by 2e-6 of its largest terms.
+// of the products), and the sum by 2e-6 of its largest terms: c0, the C_k and the a_k over the
+// tile's radius r (the last weigh most where the middle ray lies in a thin Gaussian's plane).
 struct ConeTest {
     float c, bx, by, bz, xx, yy, zz, xy, xz, yz;
     __device__ __forceinline__ void set(float4 r0, float4 r1, float4 r2, float3 o, float3 m, float r)
@@ -1450,7 +1451,7 @@ struct ConeTest {
         const float e = 2e-6f * sqrtf((axx + ayy + azz) * (vx * vx + vy * vy + vz * vz)), g = 1.0f + 2.0f * e + e * e;
         const float Xx = X0 * X0 + X1 * X1 + X2 * X2, Yy = Y0 * Y0 + Y1 * Y1 + Y2 * Y2, Zz = Z0 * Z0 + Z1 * Z1 + Z2 * Z2;
         const float cc = (c0 * c0 + c1 * c1 + c2 * c2) * inv;
-        c = cc - g - 2e-6f * (cc + r * r * (Xx + Yy + Zz) * inv + g);
+        c = cc - g - 2e-6f * (cc + r * r * (Xx + Yy + Zz + g * (axx + ayy + azz)) * inv + g);
         bx = 2.0f * inv * (c0 * X0 + c1 * X1 + c2 * X2 - g * (d0 * r0.x + d1 * r1.x + d2 * r2.x));
         by = 2.0f * inv * (c0 * Y0 + c1 * Y1 + c2 * Y2 - g * (d0 * r0.y + d1 * r1.y + d2 * r2.y));
         bz = 2.0f * inv * (c0 * Z0 + c1 * Z1 + c2 * Z2 - g * (d0 * r0.z + d1 * r1.z + d2 * r2.z));

@@ -9,6 +9,53 @@ from paper_2601_20429_gb300 import render as R
 from paper_2601_20429_gb300 import scenes
 
 
+def _discs(cam, o, n, ratio, size, at, aside, offset, seed):
+    """Faint discs of aspect 1:ratio whose planes hold one of the camera's rays: their means lie at depth `at`
+    on it (an array), `aside` in the plane beside it and `offset` half-thicknesses off it."""
+    rng = np.random.default_rng(seed)
+    W, H, th = cam["width"], cam["height"], np.tan(0.5 * cam["fov"])
+    p = rng.integers(0, W * H, n)
+    u, v = (2 * (p % W + 0.5) / W - 1) * th * W / H, (1 - 2 * (p // W + 0.5) / H) * th
+    d = np.asarray(cam["forward"]) + u[:, None] * np.asarray(cam["right"]) + v[:, None] * np.asarray(cam["up"])
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    nrm = np.cross(d, rng.standard_normal((n, 3)))
+    nrm /= np.linalg.norm(nrm, axis=1, keepdims=True)
+    e2 = np.cross(nrm, d)
+    M = np.stack([d, e2, nrm], 2)                       # columns: the disc's axes (a rotation)
+    w = np.sqrt(np.maximum(1 + np.trace(M, axis1=1, axis2=2), 1e-12)) / 2
+    q = np.stack([w, (M[:, 2, 1] - M[:, 1, 2]) / (4 * w), (M[:, 0, 2] - M[:, 2, 0]) / (4 * w),
+                  (M[:, 1, 0] - M[:, 0, 1]) / (4 * w)], 1)
+    opacity = 0.015
+    s = np.tile([size, size, size / ratio], (n, 1)) / np.sqrt(2 * np.log(opacity / 0.01))
+    mean = np.asarray(o) + at[:, None] * d + aside[:, None] * e2 + (offset * size / ratio)[:, None] * nrm
+    return scenes.GaussianParams(mean.astype(np.float32), np.log(s).astype(np.float32), q.astype(np.float32),
+                                 np.full(n, np.log(opacity / (1 - opacity)), np.float32),
+                                 rng.normal(0, 0.3, (n, 1, 3)).astype(np.float32), 0)
+
+
+def _equal_transmittance(g, cam, **opts):
+    sc = R.Scene.from_params(g)
+    a = R.render(sc, cam, T_min=0.0, **opts)["rgbT"]
+    b = R.render(sc, cam, T_min=0.0, traversal="restart", **opts)["rgbT"]
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(a[:, 3].cpu().numpy(), b[:, 3].cpu().numpy())
+    sc.close()
+
+
+@pytest.mark.parametrize("seed", range(4))
+@pytest.mark.parametrize("ratio", [1e2, 1e3, 1e4, 1e5])
+def test_camera_inside_thin_discs(ratio, seed):
+    """A wide tile whose camera lies in the discs' planes, within the discs: the walk filters no hit out (the same
+    transmittances, bit for bit, as rounds that test every leaf that a ray's boxes reach)."""
+    o = (0.1, 0.2, -0.3)
+    cam = scenes.pinhole_camera(8, 4, o, (0.4, 0.1, 1.0), 100.0)
+    rng = np.random.default_rng(seed + 50)
+    n = 400
+    g = _discs(cam, o, n, ratio, 3.0, 10 ** rng.uniform(-3, -0.5, n), 10 ** rng.uniform(-4, -1, n), rng.uniform(-0.99, 0.99, n),
+               seed)
+    _equal_transmittance(g, cam, k=16)
+
+
 @pytest.mark.parametrize("traversal", ["restart", "checkpoint", "single"])
 @pytest.mark.parametrize("k", [1, 2, 8])
 def test_depths_of_both_zeros(traversal, k):
