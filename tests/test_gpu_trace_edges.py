@@ -56,6 +56,18 @@ def test_camera_inside_thin_discs(ratio, seed):
     _equal_transmittance(g, cam, k=16)
 
 
+@pytest.mark.parametrize("seed", range(3))
+@pytest.mark.parametrize("ratio", [1e4, 1e6, 3e6])
+def test_thin_discs_behind_t_near(ratio, seed):
+    """Depths just behind t_near (within 2 %) of discs seen along their planes: none is taken for one before it."""
+    o = (0.1, 0.2, -0.3)
+    cam = scenes.pinhole_camera(8, 4, o, (0.4, 0.1, 1.0), 60.0, t_near=1.0)
+    rng = np.random.default_rng(seed + 70)
+    n = 1500
+    g = _discs(cam, o, n, ratio, 0.3, 1.0 + rng.uniform(0.0, 0.02, n), rng.uniform(-0.1, 0.1, n), np.zeros(n), seed)
+    _equal_transmittance(g, cam, k=16)
+
+
 @pytest.mark.parametrize("traversal", ["restart", "checkpoint", "single"])
 @pytest.mark.parametrize("k", [1, 2, 8])
 def test_depths_of_both_zeros(traversal, k):
