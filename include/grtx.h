@@ -335,6 +335,12 @@ GRTX_API int grtx_morton_codes_sized(const float *d_aabb, int64_t n, const float
 GRTX_API int grtx_sort_pairs(uint64_t *d_keys, uint32_t *d_values, int64_t n, int key_bits,
                              void *d_temp, size_t *temp_bytes, void *stream);
 
+/* The same sort with a bound on its waiting: a block of a pass waits for the digit counts of the
+ * blocks before it, and one that has found nothing new max_waits times (>= 0) counts their keys
+ * itself. The result is the same whatever the bound; grtx_sort_pairs uses 2^22. */
+GRTX_API int grtx_sort_pairs_bounded(uint64_t *d_keys, uint32_t *d_values, int64_t n, int key_bits,
+                                     void *d_temp, size_t *temp_bytes, int max_waits, void *stream);
+
 /* Binary radix tree over n >= 2 sorted keys (index appended to break ties between equal
  * keys): internal node 0 is the root; node i covers a key range with i at one end; a range
  * [a, b] split at g has children [a, g] and [g+1, b], numbered g and g+1 if internal or

@@ -289,10 +289,12 @@ __global__ void k_scan_add(uint32_t *__restrict__ d, int64_t m, const uint32_t *
 // their keys with warp matching, in order. Histogram, three-kernel scan and scatter of each pass were
 // 40 launches over 4,096-key tiles, 16 rounds of four barriers a tile. Kernels of a 64-bit sort: 1M
 // keys 310 -> 240 us, 20,000 keys 250 -> 80 us (bound by the look-back and the scattered writes; 2, 8
-// or 16 keys a thread instead of 4: a build within 6 %).
+// or 16 keys a thread instead of 4: a build within 6 %). A look-back that has waited long enough for
+// the tile before counts that tile's keys itself (the pass only reads them): a wait is bounded and
+// the result is the same, so no caller has an error to read.
 // ------------------------------------------------------------------------------------------
 constexpr int kSortThreads = 256, kSortItems = 4, kSortTile = kSortThreads * kSortItems;
-constexpr int kSortPasses = 8, kSortWords = 16, kSortWait = 8;   // words: a ticket a pass, then a wait that ran out
+constexpr int kSortPasses = 8, kSortWords = 16;              // words: a ticket a pass
 constexpr uint64_t kLookOwn = 1ull << 62, kLookAll = 2ull << 62, kLookCounts = kLookOwn - 1;
 constexpr int kLookWaits = 1 << 22;                          // bound on the checks of one look-back
 
@@ -335,7 +337,7 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_pass(const uint64_t *__re
                                                             uint64_t *__restrict__ kout, uint32_t *__restrict__ vout, int64_t n,
                                                             int shift, unsigned dmask, const unsigned long long *__restrict__ starts,
                                                             uint64_t *__restrict__ look, uint64_t *__restrict__ next_look,
-                                                            unsigned *__restrict__ words, int pass)
+                                                            unsigned *__restrict__ words, int pass, int waits)
 {
     __shared__ uint32_t wc[kSortThreads / 32][256];
     __shared__ int64_t run[256];
@@ -405,9 +407,12 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_pass(const uint64_t *__re
                     }
                 }
                 pred -= used;
-                if (used == 0 && ++w >= kLookWaits) {
-                    words[kSortWait] = 1u;                                           // (never expected)
-                    break;
+                if (used == 0 && w++ >= waits) {                                     // count tile pred, which is full
+                    const uint64_t *const kp = kin + pred * kSortTile;
+                    uint64_t found = 0;
+                    for (int q = 0; q < kSortTile; ++q) found += ((unsigned)(kp[q] >> shift) & dmask) == (unsigned)tid;
+                    before += found;
+                    --pred;
                 }
             }
             lk[(size_t)tile * 256 + tid] = kLookAll | (before + mine);
@@ -447,7 +452,7 @@ SortTemp sort_layout(int64_t n)
     return t;
 }
 
-int sort_pairs(uint64_t *keys, uint32_t *vals, int64_t n, int key_bits, void *temp, cudaStream_t s)
+int sort_pairs(uint64_t *keys, uint32_t *vals, int64_t n, int key_bits, void *temp, cudaStream_t s, int waits = kLookWaits)
 {
     if (n <= 1) return GRTX_OK;
     SortTemp L = sort_layout(n);
@@ -470,7 +475,7 @@ int sort_pairs(uint64_t *keys, uint32_t *vals, int64_t n, int key_bits, void *te
         int bits = std::min(8, key_bits - shift);            // the last digit may be narrower
         unsigned dmask = (1u << bits) - 1u;
         k_sort_pass<<<n_tiles, kSortThreads, 0, s>>>(kin, vin, kout, vout, n, shift, dmask, counts + 256 * p, look[p & 1],
-                                                     look[(p + 1) & 1], words, p);
+                                                     look[(p + 1) & 1], words, p, waits);
         std::swap(kin, kout);
         std::swap(vin, vout);
     }
@@ -1449,7 +1454,7 @@ void free_scene_arrays(grtx_scene *sc)
 // Morton -> sort -> radix tree -> refit -> nodes over n leaf boxes (sorted in place with
 // `order`). Writes sc->nodes, sc->codes, sc->depth.
 int build_tree(grtx_scene *sc, Alloc &A, float *leaf_aabb, int64_t n, uint32_t *order, uint64_t *codes,
-               float *bounds_dev, int code_kind, unsigned **sort_words)
+               float *bounds_dev, int code_kind)
 {
     cudaStream_t s = sc->stream;
     int blocks = grtx_div_up(n, kThreads);
@@ -1463,7 +1468,6 @@ int build_tree(grtx_scene *sc, Alloc &A, float *leaf_aabb, int64_t n, uint32_t *
     void *stmp;
     TRY(A.get((char **)&stmp, sort_layout(n).total, true));
     TRY(sort_pairs(codes, order, n, 64, stmp, s));
-    *sort_words = n > 1 ? (unsigned *)((char *)stmp + sort_layout(n).off_words) : nullptr;
     return GRTX_OK;
 }
 
@@ -1675,8 +1679,7 @@ int build_scene(const grtx_gaussians *g, const grtx_params *p, int form, grtx_sc
     k_prep<<<blocks, kThreads, 0, s>>>(g->means, g->log_scales, g->quats, g->opacity_logits, n, p->alpha_min,
                                        geom_raw, aabb_raw);
     GRTX_CHECK_LAUNCH("prep");
-    unsigned *sort_words = nullptr, h_wait = 0;
-    TRY(build_tree(sc, A, aabb_raw, n, order, codes, bounds_dev, p->bvh_codes, &sort_words));
+    TRY(build_tree(sc, A, aabb_raw, n, order, codes, bounds_dev, p->bvh_codes));
     // number of valid Gaussians: their codes sort before the 2^64-1 of the empty boxes
     unsigned long long *d_nvalid;
     TRY(A.get(&d_nvalid, 1, true));
@@ -1684,9 +1687,7 @@ int build_scene(const grtx_gaussians *g, const grtx_params *p, int form, grtx_sc
     k_count_valid<<<1, 32, 0, s>>>(codes, n, d_nvalid);
     unsigned long long h_nvalid = 0;
     GRTX_CUDA(cudaMemcpyAsync(&h_nvalid, d_nvalid, 8, cudaMemcpyDeviceToHost, s));
-    if (sort_words) GRTX_CUDA(cudaMemcpyAsync(&h_wait, sort_words + kSortWait, 4, cudaMemcpyDeviceToHost, s));
     GRTX_CUDA(cudaStreamSynchronize(s));
-    if (h_wait) return grtx_fail(GRTX_ERR_TIMEOUT, "radix sort: a look-back ran out");
     int64_t nv = (int64_t)h_nvalid;
     sc->n_valid = nv;
     if (nv == 0) {
@@ -1739,7 +1740,7 @@ int build_scene(const grtx_gaussians *g, const grtx_params *p, int form, grtx_sc
                                                                       sc->gid, nv, g_ico_circ, tris_raw,
                                                                       tri_aabb_raw, slack_raw);
         GRTX_CHECK_LAUNCH("proxy expand");
-        TRY(build_tree(sc, A, tri_aabb_raw, nt, torder, tcodes, bounds_dev, p->bvh_codes, &sort_words));
+        TRY(build_tree(sc, A, tri_aabb_raw, nt, torder, tcodes, bounds_dev, p->bvh_codes));
         sc->n_leaves = nt;
         TRY(A.get(&sc->tris, 3 * nt, false));
         TRY(A.get(&tri_aabb, 6 * nt, true));
@@ -1753,9 +1754,7 @@ int build_scene(const grtx_gaussians *g, const grtx_params *p, int form, grtx_sc
     }
     float h_root[16];
     GRTX_CUDA(cudaMemcpyAsync(h_root, sc->nodes, sizeof(h_root), cudaMemcpyDeviceToHost, s));
-    if (form == GRTX_FORM_PROXY20) GRTX_CUDA(cudaMemcpyAsync(&h_wait, sort_words + kSortWait, 4, cudaMemcpyDeviceToHost, s));
     GRTX_CUDA(cudaStreamSynchronize(s));
-    if (h_wait) return grtx_fail(GRTX_ERR_TIMEOUT, "radix sort: a look-back ran out");
     set_bounds(sc, h_root);
     if (sc->depth >= GRTX_STACK)
         return grtx_fail(GRTX_ERR_OVERFLOW_FATAL, "BVH depth " + std::to_string(sc->depth) +
@@ -1951,12 +1950,13 @@ extern "C" GRTX_API int grtx_ploc_tree(const float *d_leaf_aabb, int64_t n, uint
     return ploc_tree(A, d_leaf_aabb, n, d_left, d_right, d_parent, S(stream), iterations);
 }
 
-extern "C" GRTX_API int grtx_sort_pairs(uint64_t *d_keys, uint32_t *d_values, int64_t n, int key_bits, void *d_temp,
-                                        size_t *temp_bytes, void *stream)
+extern "C" GRTX_API int grtx_sort_pairs_bounded(uint64_t *d_keys, uint32_t *d_values, int64_t n, int key_bits, void *d_temp,
+                                                size_t *temp_bytes, int max_waits, void *stream)
 {
     if (!temp_bytes) return grtx_fail(GRTX_ERR_INVALID_ARG, "temp_bytes is NULL");
     if (n < 0 || n >= ((int64_t)1 << 31)) return grtx_fail(GRTX_ERR_INVALID_ARG, "n out of range");
     if (key_bits < 1 || key_bits > 64) return grtx_fail(GRTX_ERR_INVALID_ARG, "key_bits must be 1..64");
+    if (max_waits < 0) return grtx_fail(GRTX_ERR_INVALID_ARG, "max_waits must not be negative");
     size_t need = sort_layout(std::max<int64_t>(n, 1)).total;
     if (!d_temp) {
         *temp_bytes = need;
@@ -1964,7 +1964,13 @@ extern "C" GRTX_API int grtx_sort_pairs(uint64_t *d_keys, uint32_t *d_values, in
     }
     if (*temp_bytes < need) return grtx_fail(GRTX_ERR_INVALID_ARG, "temp buffer too small");
     if (n > 1 && (!d_keys || !d_values)) return grtx_fail(GRTX_ERR_INVALID_ARG, "NULL pointer");
-    return sort_pairs(d_keys, d_values, n, key_bits, d_temp, S(stream));
+    return sort_pairs(d_keys, d_values, n, key_bits, d_temp, S(stream), max_waits);
+}
+
+extern "C" GRTX_API int grtx_sort_pairs(uint64_t *d_keys, uint32_t *d_values, int64_t n, int key_bits, void *d_temp,
+                                        size_t *temp_bytes, void *stream)
+{
+    return grtx_sort_pairs_bounded(d_keys, d_values, n, key_bits, d_temp, temp_bytes, kLookWaits, stream);
 }
 
 extern "C" GRTX_API int grtx_radix_tree(const uint64_t *d_sorted_keys, int64_t n, uint32_t *d_left, uint32_t *d_right,

@@ -176,6 +176,7 @@ _SIGS = {
     "grtx_morton_codes": (C.c_int, [_fp, C.c_int64, _fp, _fp, _fp, _fp]),
     "grtx_morton_codes_sized": (C.c_int, [_fp, C.c_int64, _fp, _fp, _fp, _fp]),
     "grtx_sort_pairs": (C.c_int, [_fp, _fp, C.c_int64, C.c_int, _fp, C.POINTER(C.c_size_t), _fp]),
+    "grtx_sort_pairs_bounded": (C.c_int, [_fp, _fp, C.c_int64, C.c_int, _fp, C.POINTER(C.c_size_t), C.c_int, _fp]),
     "grtx_radix_tree": (C.c_int, [_fp, C.c_int64, _fp, _fp, _fp, _fp]),
     "grtx_ploc_tree": (C.c_int, [_fp, C.c_int64, _fp, _fp, _fp, C.POINTER(C.c_int), _fp]),
     "grtx_refit": (C.c_int, [_fp, _fp, _fp, _fp, C.c_int64, _fp, _fp, _fp]),
@@ -379,6 +380,18 @@ def grtx_sort_pairs(keys, values, key_bits=64, stream=None):
     temp = torch.empty(int(nb.value), dtype=torch.uint8, device=keys.device)
     check(lib().grtx_sort_pairs(ptr(keys), ptr(values), n, key_bits, ptr(temp), C.byref(nb), stream_handle(stream)),
           "grtx_sort_pairs")
+    return temp
+
+
+def grtx_sort_pairs_bounded(keys, values, max_waits: int, key_bits=64, stream=None):
+    import torch
+    n = int(keys.shape[0])
+    nb = C.c_size_t(0)
+    check(lib().grtx_sort_pairs_bounded(None, None, n, key_bits, None, C.byref(nb), int(max_waits), None),
+          "grtx_sort_pairs_bounded(size)")
+    temp = torch.empty(int(nb.value), dtype=torch.uint8, device=keys.device)
+    check(lib().grtx_sort_pairs_bounded(ptr(keys), ptr(values), n, key_bits, ptr(temp), C.byref(nb), int(max_waits),
+                                        stream_handle(stream)), "grtx_sort_pairs_bounded")
     return temp
 
 
