@@ -5,6 +5,7 @@ import pytest
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
+from paper_2601_20429_gb300 import native as N
 from paper_2601_20429_gb300 import render as R
 from paper_2601_20429_gb300 import scenes
 
@@ -92,4 +93,27 @@ def test_depths_of_both_zeros(traversal, k):
     torch.cuda.synchronize()
     assert b["n_blended"].tolist() == [n] * m
     np.testing.assert_array_equal(a[:, 3].cpu().numpy(), ref["rgbT"][:, 3].cpu().numpy())
+    sc.close()
+
+
+@pytest.mark.parametrize("opts", [dict(ckpt_capacity=2, evict_capacity=1), dict(ckpt_capacity=1, evict_capacity=8)])
+@pytest.mark.parametrize("form,width", [("sphere", 2), ("sphere", 4), ("ico20", 2), ("proxy20", 2)])
+def test_a_ray_falls_back_once(form, width, opts):
+    """A ray whose lists are too small for a packet's round leaves them for restarted rounds at once: one fallback
+    a ray, and the image of restarted rounds. (500 faint overlapping Gaussians, dozens of hits a ray.)"""
+    n = 500
+    rng = np.random.default_rng(2)
+    q = rng.standard_normal((n, 4))
+    g = scenes.GaussianParams(rng.uniform(-1, 1, (n, 3)).astype(np.float32), np.log(rng.uniform(0.1, 0.4, (n, 3))).astype(np.float32),
+                              (q / np.linalg.norm(q, axis=1, keepdims=True)).astype(np.float32),
+                              np.full(n, np.log(0.05 / 0.95), np.float32), rng.normal(0, 0.3, (n, 1, 3)).astype(np.float32), 0)
+    sc = R.Scene.from_params(g, form=form, bvh_width=width)
+    cam = scenes.pinhole_camera(40, 24, (0.1, 0.2, -3.0))
+    wide = dict(bvh_width=4) if width == 4 else {}
+    r = R.render(sc, cam, k=4, want_stats=True, **opts, **wide)
+    st = N.stats_dict(r["stats"])
+    assert 0 < st["fallbacks"] <= st["rays"] == 40 * 24
+    ref = R.render(sc, cam, k=4, traversal="restart", **wide)["rgbT"]
+    torch.cuda.synchronize()
+    np.testing.assert_allclose(r["rgbT"].cpu().numpy(), ref.cpu().numpy(), rtol=0, atol=1e-5)
     sc.close()
