@@ -33,7 +33,7 @@ using grtx_serve::Arena;
 #define GRTX_EXTERN_SERVE(K)                                                                                 \
     extern template int serve_launch<K>(const TraceArgs &, const ServeSeg *, const unsigned *, int, int,            \
                                         cudaStream_t, ServeLive);                                                    \
-    extern template int serve_occupancy<K>(int *);
+    extern template int serve_occupancy<K>(int, int *);
 GRTX_EXTERN_SERVE(1)
 GRTX_EXTERN_SERVE(2)
 GRTX_EXTERN_SERVE(4)
@@ -73,15 +73,15 @@ int serve_launch_k(int k, const TraceArgs &a, const ServeSeg *segs, const unsign
     }
 }
 
-int serve_occupancy_k(int k, int *bps)
+int serve_occupancy_k(int k, int traversal, int *bps)
 {
     switch (k) {
-    case 1: return serve_occupancy<1>(bps);
-    case 2: return serve_occupancy<2>(bps);
-    case 4: return serve_occupancy<4>(bps);
-    case 8: return serve_occupancy<8>(bps);
-    case 16: return serve_occupancy<16>(bps);
-    default: return serve_occupancy<32>(bps);
+    case 1: return serve_occupancy<1>(traversal, bps);
+    case 2: return serve_occupancy<2>(traversal, bps);
+    case 4: return serve_occupancy<4>(traversal, bps);
+    case 8: return serve_occupancy<8>(traversal, bps);
+    case 16: return serve_occupancy<16>(traversal, bps);
+    default: return serve_occupancy<32>(traversal, bps);
     }
 }
 
@@ -410,7 +410,7 @@ extern "C" GRTX_API int grtx_server_create(grtx_scene *const *scenes, int n_scen
     int bps = 0, dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (serve_occupancy_k(p->k, &bps) != GRTX_OK || bps <= 0 || sms <= 0)
+    if (serve_occupancy_k(p->k, p->traversal, &bps) != GRTX_OK || bps <= 0 || sms <= 0)
         return grtx_fail(GRTX_ERR_CUDA, "occupancy query failed");
     // sizes: the lists of n_steps step slots of `blocks` 128-ray blocks each, the segment
     // tables and queue counters, and (under a budget) the output arena

@@ -10,7 +10,7 @@
 
 #define GRTX_EXTERN_TRACE(K)                                                                     \
     extern template int trace_launch<K>(const TraceArgs &, int, bool, int, int, cudaStream_t); \
-    extern template int trace_occupancy<K>(int, bool, int, int *);                             \
+    extern template int trace_occupancy<K>(int, bool, int, int, int *);                             \
     extern template int trace_rays_launch<K>(const TraceArgs &, const ServeSeg *, int, cudaStream_t);
 GRTX_EXTERN_TRACE(1)
 GRTX_EXTERN_TRACE(2)
@@ -22,7 +22,7 @@ GRTX_EXTERN_TRACE(32)
 #define GRTX_EXTERN_SEGMENTS(K)                                                                          \
     extern template int serve_launch<K>(const TraceArgs &, const ServeSeg *, const unsigned *, int, int, cudaStream_t, \
                                         ServeLive);                                                                  \
-    extern template int serve_occupancy<K>(int *);
+    extern template int serve_occupancy<K>(int, int *);
 GRTX_EXTERN_SEGMENTS(1)
 GRTX_EXTERN_SEGMENTS(2)
 GRTX_EXTERN_SEGMENTS(4)
@@ -63,15 +63,15 @@ int rays_launch_k(int k, const TraceArgs &a, const ServeSeg *segs, int blocks, c
     }
 }
 
-int occupancy_k(int k, int form, bool instr, int pass, int *bps)
+int occupancy_k(int k, int form, bool instr, int pass, int traversal, int *bps)
 {
     switch (k) {
-    case 1: return trace_occupancy<1>(form, instr, pass, bps);
-    case 2: return trace_occupancy<2>(form, instr, pass, bps);
-    case 4: return trace_occupancy<4>(form, instr, pass, bps);
-    case 8: return trace_occupancy<8>(form, instr, pass, bps);
-    case 16: return trace_occupancy<16>(form, instr, pass, bps);
-    default: return trace_occupancy<32>(form, instr, pass, bps);
+    case 1: return trace_occupancy<1>(form, instr, pass, traversal, bps);
+    case 2: return trace_occupancy<2>(form, instr, pass, traversal, bps);
+    case 4: return trace_occupancy<4>(form, instr, pass, traversal, bps);
+    case 8: return trace_occupancy<8>(form, instr, pass, traversal, bps);
+    case 16: return trace_occupancy<16>(form, instr, pass, traversal, bps);
+    default: return trace_occupancy<32>(form, instr, pass, traversal, bps);
     }
 }
 
@@ -237,7 +237,7 @@ int run(grtx_scene *sc, TraceArgs &a, int k, bool instr, int pass, unsigned *que
     bool single = a.traversal == GRTX_TRAVERSAL_SINGLE && pass == PASS_FWD;
     set_codes(a, pass == PASS_BWD ? (int)FORM_SPHERE : form, instr, sc->n_valid);
     int bps = 0;
-    int occ = single ? trace_single_occupancy(form, instr, &bps) : occupancy_k(k, form, instr, pass, &bps);
+    int occ = single ? trace_single_occupancy(form, instr, &bps) : occupancy_k(k, form, instr, pass, a.traversal, &bps);
     if (occ != GRTX_OK || bps <= 0) return grtx_fail(GRTX_ERR_CUDA, "occupancy query failed");
     int blocks = sm_count() * bps;
     int n_slots = blocks * 128;
@@ -398,15 +398,15 @@ int segments_launch_k(int k, const TraceArgs &a, const ServeSeg *segs, const uns
     }
 }
 
-int segments_occupancy_k(int k, int *bps)
+int segments_occupancy_k(int k, int traversal, int *bps)
 {
     switch (k) {
-    case 1: return serve_occupancy<1>(bps);
-    case 2: return serve_occupancy<2>(bps);
-    case 4: return serve_occupancy<4>(bps);
-    case 8: return serve_occupancy<8>(bps);
-    case 16: return serve_occupancy<16>(bps);
-    default: return serve_occupancy<32>(bps);
+    case 1: return serve_occupancy<1>(traversal, bps);
+    case 2: return serve_occupancy<2>(traversal, bps);
+    case 4: return serve_occupancy<4>(traversal, bps);
+    case 8: return serve_occupancy<8>(traversal, bps);
+    case 16: return serve_occupancy<16>(traversal, bps);
+    default: return serve_occupancy<32>(traversal, bps);
     }
 }
 
@@ -440,7 +440,7 @@ extern "C" GRTX_API int grtx_trace_forward_batch(grtx_scene *sc, const grtx_came
         v[i].split = 0;
     }
     int bps = 0;
-    if (segments_occupancy_k(p->k, &bps) != GRTX_OK || bps <= 0) return grtx_fail(GRTX_ERR_CUDA, "occupancy query failed");
+    if (segments_occupancy_k(p->k, a.traversal, &bps) != GRTX_OK || bps <= 0) return grtx_fail(GRTX_ERR_CUDA, "occupancy query failed");
     int blocks = sm_count() * bps;
     bool ckpt = a.traversal == GRTX_TRAVERSAL_CHECKPOINT;
     // Short ray lists go in bundles of 16 or 8 rays: bounce rays share little, and a wide bundle of 32

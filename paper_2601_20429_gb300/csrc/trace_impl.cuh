@@ -2622,8 +2622,11 @@ int trace_rays_launch(const TraceArgs &a, const ServeSeg *segs, int blocks, cuda
     return cudaGetLastError() == cudaSuccess ? GRTX_OK : GRTX_ERR_CUDA;
 }
 
+// Blocks per multiprocessor of the kernel that trace_launch takes for the same arguments. (The restart
+// kernel keeps no walk and fits 6 blocks at k = 32, the checkpointed one 5: sized by the latter, a
+// restarted 1M 1080p frame took 9.0 instead of 8.1 ms.)
 template <int K>
-int trace_occupancy(int form, bool instr, int pass, int *blocks_per_sm)
+int trace_occupancy(int form, bool instr, int pass, int traversal, int *blocks_per_sm)
 {
     cudaError_t e;
     if (pass == PASS_BWD) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_trace<K, FORM_SPHERE, false, PASS_BWD>, 128, 0);
@@ -2637,6 +2640,7 @@ int trace_occupancy(int form, bool instr, int pass, int *blocks_per_sm)
     else if (form == FORM_SPHERE4Q && instr) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_trace<K, FORM_SPHERE4Q, true, PASS_FWD>, 128, 0);
     else if (form == FORM_SPHERE4Q) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_trace<K, FORM_SPHERE4Q, false, PASS_FWD>, 128, 0);
     else if (instr) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_trace<K, FORM_SPHERE, true, PASS_FWD>, 128, 0);
+    else if (traversal == GRTX_TRAVERSAL_RESTART) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_trace<K, FORM_SPHERE, false, PASS_FWD, TRAV_RESTART>, 128, 0);
     else e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_trace<K, FORM_SPHERE, false, PASS_FWD, TRAV_CKPT>, 128, 0);
     return e == cudaSuccess ? GRTX_OK : GRTX_ERR_CUDA;
 }
@@ -2661,15 +2665,17 @@ int serve_launch(const TraceArgs &a, const ServeSeg *segs, const unsigned *begin
 }
 
 template <int K>
-int serve_occupancy(int *blocks_per_sm)
+int serve_occupancy(int traversal, int *blocks_per_sm)
 {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_serve<K, TRAV_CKPT>, 128, 0) == cudaSuccess
-               ? GRTX_OK : GRTX_ERR_CUDA;
+    const cudaError_t e = traversal == GRTX_TRAVERSAL_RESTART
+                              ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_serve<K, TRAV_RESTART>, 128, 0)
+                              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_serve<K, TRAV_CKPT>, 128, 0);
+    return e == cudaSuccess ? GRTX_OK : GRTX_ERR_CUDA;
 }
 
 #define GRTX_INSTANTIATE_TRACE(K)                                                                  \
     template int trace_launch<K>(const TraceArgs &, int, bool, int, int, cudaStream_t);           \
-    template int trace_occupancy<K>(int, bool, int, int *);                                         \
+    template int trace_occupancy<K>(int, bool, int, int, int *);                                         \
     template int trace_rays_launch<K>(const TraceArgs &, const ServeSeg *, int, cudaStream_t);                        \
     template int serve_launch<K>(const TraceArgs &, const ServeSeg *, const unsigned *, int, int, cudaStream_t, ServeLive);   \
-    template int serve_occupancy<K>(int *);
+    template int serve_occupancy<K>(int, int *);

@@ -17,7 +17,7 @@
 
 #define GRTX_EXTERN_NOALLOC(K)                                                                   \
     extern template int trace_launch<K>(const TraceArgs &, int, bool, int, int, cudaStream_t); \
-    extern template int trace_occupancy<K>(int, bool, int, int *);
+    extern template int trace_occupancy<K>(int, bool, int, int, int *);
 GRTX_EXTERN_NOALLOC(1)
 GRTX_EXTERN_NOALLOC(2)
 GRTX_EXTERN_NOALLOC(4)
@@ -82,15 +82,15 @@ int launch_noalloc(int k, const TraceArgs &a, int form, int blocks, cudaStream_t
     }
 }
 
-int occupancy_noalloc(int k, int form, int *bps)
+int occupancy_noalloc(int k, int form, int traversal, int *bps)
 {
     switch (k) {
-    case 1: return trace_occupancy<1>(form, false, PASS_FWD, bps);
-    case 2: return trace_occupancy<2>(form, false, PASS_FWD, bps);
-    case 4: return trace_occupancy<4>(form, false, PASS_FWD, bps);
-    case 8: return trace_occupancy<8>(form, false, PASS_FWD, bps);
-    case 16: return trace_occupancy<16>(form, false, PASS_FWD, bps);
-    default: return trace_occupancy<32>(form, false, PASS_FWD, bps);
+    case 1: return trace_occupancy<1>(form, false, PASS_FWD, traversal, bps);
+    case 2: return trace_occupancy<2>(form, false, PASS_FWD, traversal, bps);
+    case 4: return trace_occupancy<4>(form, false, PASS_FWD, traversal, bps);
+    case 8: return trace_occupancy<8>(form, false, PASS_FWD, traversal, bps);
+    case 16: return trace_occupancy<16>(form, false, PASS_FWD, traversal, bps);
+    default: return trace_occupancy<32>(form, false, PASS_FWD, traversal, bps);
     }
 }
 
@@ -137,7 +137,7 @@ extern "C" GRTX_API int grtx_trace_forward_noalloc(grtx_scene *sc, const grtx_ca
     st = scratch_for_current_device(&base, &sms);
     if (st) return st;
     int bps = 0;
-    if (occupancy_noalloc(p->k, form, &bps) != GRTX_OK || bps <= 0)
+    if (occupancy_noalloc(p->k, form, a.traversal, &bps) != GRTX_OK || bps <= 0)
         return grtx_fail(GRTX_ERR_CUDA, "occupancy query failed");
     int blocks = (int)std::min<size_t>((size_t)sms * bps, room / per_block);
     int n_slots = blocks * 128;

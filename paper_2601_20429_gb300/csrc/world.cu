@@ -39,7 +39,6 @@ struct WorldArgs {
     const InstRec *inst;      // non-empty instances
     const uint32_t *leaf_base;// inst[i].leaf_base, ascending
     int n_inst, n_tl_nodes;
-    int walk;                 // uninstrumented checkpointed traces: round 1 as world_walk (a.ck0 = a.ev)
     uint4 *wck0, *wck1;       // checkpoint lists of (ref, t bits, instance, 0), [entry][slot]
 };
 
@@ -433,7 +432,7 @@ __device__ __forceinline__ bool world_walk(const WorldArgs &W, bool valid, uint2
 
 // One ray through the world: the round loop of trace_ray with world_round and blending in
 // the frame of each Gaussian's object.
-template <int K, bool INSTR>
+template <int K, bool INSTR, bool WALKED>
 __device__ __forceinline__ void world_ray(const WorldArgs &W, int slot, int64_t pix, float3 o, float3 d, float tn,
                                           float tf, KBuf<K> &kb, Counters &cnt, bool r1_ok, int r1_n_dst, int r1_n_ev,
                                           float lim = INFINITY)
@@ -471,7 +470,7 @@ __device__ __forceinline__ void world_ray(const WorldArgs &W, int slot, int64_t 
         }
         int n_dst = 0;
         bool round_ok;
-        if (first_round && (INSTR || r1_ok)) {         // round 1 was traced for the warp
+        if (first_round && (r1_ok || !WALKED)) {         // round 1 was traced for the warp
             round_ok = r1_ok;
             n_dst = r1_n_dst;
             n_ev = r1_n_ev;
@@ -533,13 +532,13 @@ __device__ __forceinline__ void world_ray(const WorldArgs &W, int slot, int64_t 
     if (INSTR && a.n_blended) a.n_blended[pix] = nb;
 }
 
-template <int K, bool INSTR>
+// WALKS: uninstrumented checkpointed traces, round 1 as world_walk (a.ck0 = a.ev).
+template <int K, bool INSTR, bool WALKS>
 __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, false)) k_trace_world(WorldArgs W)
 {
     __shared__ uint64_t s_k[K * kBlock];
-    constexpr bool walks = !INSTR;
-    __shared__ uint4 s_pst[kBlock / 32][walks ? kWarpShared : kPacketStack];       // the walk's or the packet's
-    __shared__ uint2 s_tst[walks ? kBlock / 32 : 1][kWorldWalkStack];
+    __shared__ uint4 s_pst[kBlock / 32][WALKS ? kWarpShared : kPacketStack];       // the walk's or the packet's
+    __shared__ uint2 s_tst[WALKS ? kBlock / 32 : 1][WALKS ? kWorldWalkStack : 1];
     const int slot = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     KBuf<K> kb;
@@ -566,19 +565,20 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, false)) k_trace_wo
         int n_dst = 0, n_ev = 0;
         bool lane_ok = true;
         float lim = GRTX_INF;
-        if (walks && W.walk) {
+        if constexpr (WALKS) {
             Cut cut;
             cut.clear();
             if (!world_walk<K>(W, valid, s_tst[threadIdx.x >> 5], *reinterpret_cast<WalkShared *>(s_pst[threadIdx.x >> 5]), o, d,
                                inv, tn, tf, (uint32_t)slot, n_ev, kb, cut, lim, lane_ok))
                 lane_ok = false;
-        } else
-        world_packet_round<K, INSTR>(W, valid, s_pst[threadIdx.x >> 5], o, d, inv, tn, tf,
-                                     W.a.traversal == GRTX_TRAVERSAL_CHECKPOINT, W.wck1 + slot, n_dst, W.a.ev + slot,
-                                     n_ev, kb, cnt, lane_ok);
+        } else {
+            world_packet_round<K, INSTR>(W, valid, s_pst[threadIdx.x >> 5], o, d, inv, tn, tf,
+                                         W.a.traversal == GRTX_TRAVERSAL_CHECKPOINT, W.wck1 + slot, n_dst, W.a.ev + slot,
+                                         n_ev, kb, cnt, lane_ok);
+        }
         if (valid) {
             ++rays;
-            world_ray<K, INSTR>(W, slot, pix, o, d, tn, tf, kb, cnt, lane_ok, n_dst, n_ev, lim);
+            world_ray<K, INSTR, WALKS>(W, slot, pix, o, d, tn, tf, kb, cnt, lane_ok, n_dst, n_ev, lim);
         }
         __syncwarp();
     }
@@ -595,18 +595,20 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, false)) k_trace_wo
 }
 
 template <int K>
-int world_launch(const WorldArgs &W, bool instr, int blocks, cudaStream_t s)
+int world_launch(const WorldArgs &W, bool instr, bool walk, int blocks, cudaStream_t s)
 {
-    if (instr) k_trace_world<K, true><<<blocks, kBlock, 0, s>>>(W);
-    else k_trace_world<K, false><<<blocks, kBlock, 0, s>>>(W);
+    if (instr) k_trace_world<K, true, false><<<blocks, kBlock, 0, s>>>(W);
+    else if (walk) k_trace_world<K, false, true><<<blocks, kBlock, 0, s>>>(W);
+    else k_trace_world<K, false, false><<<blocks, kBlock, 0, s>>>(W);
     return cudaGetLastError() == cudaSuccess ? GRTX_OK : GRTX_ERR_CUDA;
 }
 
 template <int K>
-int world_occupancy(bool instr, int *bps)
+int world_occupancy(bool instr, bool walk, int *bps)
 {
-    cudaError_t e = instr ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, k_trace_world<K, true>, kBlock, 0)
-                          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, k_trace_world<K, false>, kBlock, 0);
+    cudaError_t e = instr  ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, k_trace_world<K, true, false>, kBlock, 0)
+                    : walk ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, k_trace_world<K, false, true>, kBlock, 0)
+                           : cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, k_trace_world<K, false, false>, kBlock, 0);
     return e == cudaSuccess ? GRTX_OK : GRTX_ERR_CUDA;
 }
 
@@ -809,14 +811,21 @@ extern "C" GRTX_API int grtx_world_trace_forward(grtx_world *w, const grtx_camer
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if (out->blended_ids)
         GRTX_CUDA(cudaMemsetAsync(out->blended_ids, 0xff, (size_t)cam->width * cam->height * out->ids_cap * 4, s));
-    int bps = 0;
-    int occ = p->k == 8 ? world_occupancy<8>(instr, &bps)
-              : p->k == 16 ? world_occupancy<16>(instr, &bps) : world_occupancy<32>(instr, &bps);
-    if (occ != GRTX_OK || bps <= 0) return grtx_fail(GRTX_ERR_CUDA, "occupancy query failed");
-    int blocks = sm_count_here() * bps;
-    size_t n_slots = (size_t)blocks * kBlock;
     bool ckpt = a.traversal == GRTX_TRAVERSAL_CHECKPOINT;
     size_t C = ckpt ? (size_t)a.ckpt_cap : 1, E = ckpt ? (size_t)a.evict_cap : 1;
+    bool walk = ckpt && !instr;
+    int blocks = 0;
+    for (;;) {
+        int bps = 0;
+        int occ = p->k == 8 ? world_occupancy<8>(instr, walk, &bps)
+                  : p->k == 16 ? world_occupancy<16>(instr, walk, &bps) : world_occupancy<32>(instr, walk, &bps);
+        if (occ != GRTX_OK || bps <= 0) return grtx_fail(GRTX_ERR_CUDA, "occupancy query failed");
+        blocks = sm_count_here() * bps;
+        // the walk addresses the eviction lists with 32 bits
+        if (!walk || (size_t)blocks * kBlock * E < ((size_t)1 << 31)) break;
+        walk = false;
+    }
+    size_t n_slots = (size_t)blocks * kBlock;
     size_t need = n_slots * (2 * C * sizeof(uint4) + E * sizeof(uint2));
     if (need > w->ws_bytes) {
         if (w->ws) {
@@ -840,15 +849,13 @@ extern "C" GRTX_API int grtx_world_trace_forward(grtx_world *w, const grtx_camer
     W.n_inst = w->n_inst;
     W.n_tl_nodes = w->n_tl_nodes;
     set_window(a);
-    // the walk addresses the eviction lists with 32 bits, and keeps opacity codes below the leaf
-    // indices where these leave room
-    W.walk = ckpt && !instr && n_slots * E < ((size_t)1 << 31);
+    // the walk keeps opacity codes below the leaf indices where these leave room
     a.ck0 = a.ev;
-    if (W.walk) set_codes(a, FORM_SPHERE, false, w->n_leaves);
+    if (walk) set_codes(a, FORM_SPHERE, false, w->n_leaves);
     w->stream = s;
     GRTX_CUDA(cudaMemsetAsync(a.queue, 0, sizeof(unsigned), s));
-    int launched = p->k == 8 ? world_launch<8>(W, instr, blocks, s)
-                   : p->k == 16 ? world_launch<16>(W, instr, blocks, s) : world_launch<32>(W, instr, blocks, s);
+    int launched = p->k == 8 ? world_launch<8>(W, instr, walk, blocks, s)
+                   : p->k == 16 ? world_launch<16>(W, instr, walk, blocks, s) : world_launch<32>(W, instr, walk, blocks, s);
     if (launched != GRTX_OK) {
         cudaError_t e = cudaGetLastError();
         return grtx_cuda_fail(e == cudaSuccess ? cudaErrorLaunchFailure : e, "world trace launch");

@@ -117,3 +117,19 @@ def test_a_ray_falls_back_once(form, width, opts):
     torch.cuda.synchronize()
     np.testing.assert_allclose(r["rgbT"].cpu().numpy(), ref.cpu().numpy(), rtol=0, atol=1e-5)
     sc.close()
+
+
+@pytest.mark.parametrize("entry", ["frame", "batch"])
+def test_restart_fills_the_multiprocessors(entry):
+    """A restarted launch keeps no walk: at k = 32 six of its blocks fit a multiprocessor (32 KB of k-buffers and
+    3 KB of packet stacks each, of 228 KB), and the launch takes slots for as many (three 8-byte words each)."""
+    g = scenes.tiny_scene(seed=1, n=200)
+    sc = R.Scene.from_params(g)
+    cam = scenes.pinhole_camera(32, 32, (0.0, 0.0, -3.0))
+    if entry == "frame":
+        R.render(sc, cam, k=32, traversal="restart")
+    else:
+        R.render_batch(sc, [(cam, None), (cam, None)], k=32, traversal="restart")
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert sc.info()["bytes_workspace"] >= 6 * sms * 128 * 3 * 8
+    sc.close()
