@@ -1826,7 +1826,7 @@ template <int K, int FORM, bool INSTR, int PASS>
 __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc, float4 *__restrict__ out, int slot,
                                           int64_t pix, float3 o, float3 d, float tn, float tf, KBuf<K> &kb,
                                           Counters &cnt, Cut cut, bool r1_done = false, bool r1_ok = true,
-                                          int r1_n_dst = 0, int r1_n_ev = 0, float lim = INFINITY, bool walked = false)
+                                          int r1_n_dst = 0, int r1_n_ev = 0, float lim = INFINITY)
 {
     constexpr bool BWD = PASS == PASS_BWD;
     const uint32_t S = (uint32_t)a.n_slots;
@@ -1874,20 +1874,11 @@ __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc
         }
         int n_dst = 0;
         bool round_ok;
-        if (r1_done && first_round && (r1_ok || !walked)) {      // round 1 was traced for the warp
+        if (r1_done && first_round) {                  // round 1 was traced for the warp
             round_ok = r1_ok;
             n_dst = r1_n_dst;
             n_ev = r1_n_ev;
         } else {
-            // a walk that could not finish: this ray traces the round on its own. (A packet that could not
-            // has overflown the lists that this would fill again, or the stack: it restarts below. Tried
-            // with the lists first, 1920x1080 of 6M 4-wide nodes took 27.1 instead of 17.1 ms.)
-            if (r1_done && first_round) {
-                if (INSTR) cnt.fallbacks++;
-                kb.clear();
-                cut.clear();
-                lim = GRTX_INF;
-            }
             round_ok = trace_round<K, FORM, INSTR>(a, sc, o, d, inv, inv_len, tn, tf, Lt, Li, ckpt, from_root, src, n_src,
                                                    dst, n_dst, ev, n_ev, kb, cut, from_root ? a.window : 0, cnt);
         }
@@ -2059,7 +2050,8 @@ __device__ __forceinline__ void trace_warp(const TraceArgs &a, const SceneRef &s
     int n_dst = 0, n_ev = 0;
     bool lane_ok = true;
     float lim = GRTX_INF;
-    const bool walked = FORM == FORM_SPHERE && !INSTR && a.traversal == GRTX_TRAVERSAL_CHECKPOINT;
+    constexpr bool WALKS = FORM == FORM_SPHERE && !INSTR;        // (where the lists are used)
+    const bool walked = WALKS && a.traversal == GRTX_TRAVERSAL_CHECKPOINT;
     static_assert(sizeof(WalkShared) <= kWarpShared * sizeof(uint4), "the walk's shared memory");
     if (walked) {
         if (sc.has_tree && !tile_walk<K>(a, sc, valid, *reinterpret_cast<WalkShared *>(pst), o, d, tn, tf,
@@ -2087,10 +2079,16 @@ __device__ __forceinline__ void trace_warp(const TraceArgs &a, const SceneRef &s
                                      a.ev_off + (uint32_t)slot, n_ev, kb, cut, cnt, lane_ok);
     }
     // a lane whose packet could not finish (lists or the warp's stack overflowed) redoes round 1
-    // from the root on its own, as after any capacity overflow
+    // from the root on its own, as after any capacity overflow. (Tried with its lists again first,
+    // 1920x1080 of 6M 4-wide nodes took 27.1 instead of 17.1 ms.) One whose walk could not finish
+    // begins anew: its bundle may only have shared too little.
+    if (walked && !lane_ok) {
+        cut.clear();
+        lim = GRTX_INF;
+    }
     if (valid)
-        trace_ray<K, FORM, INSTR, PASS>(a, sc, out, slot, pix, o, d, tn, tf, kb, cnt, cut, true, lane_ok, n_dst, n_ev, lim,
-                                        walked);
+        trace_ray<K, FORM, INSTR, PASS>(a, sc, out, slot, pix, o, d, tn, tf, kb, cnt, cut, !WALKS || lane_ok, WALKS || lane_ok,
+                                        n_dst, n_ev, lim);
 }
 
 // After a tile, every checkpoint and eviction list entry of the warp's 32 ray slots is dead:
@@ -2387,9 +2385,13 @@ __global__ void __launch_bounds__(kBlock, 5) k_trace_rays(const __grid_constant_
         int n_ev;
         const bool ok = ray_walk<K>(a, sc, s_w[threadIdx.x >> 5], o, d, tn, tf, ev, n_ev, kb, cut, lim);
         if (!ok || __shfl_sync(full, lim, 0) < GRTX_INF) {
+            if (!ok) {                                           // it begins anew
+                cut.clear();
+                lim = GRTX_INF;
+            }
             if (lane == 0)
-                trace_ray<K, FORM_SPHERE, false, PASS_FWD>(a, sc, out, slot, pix, o, d, tn, tf, kb, cnt, cut, true, ok, 0,
-                                                           n_ev, lim, true);
+                trace_ray<K, FORM_SPHERE, false, PASS_FWD>(a, sc, out, slot, pix, o, d, tn, tf, kb, cnt, cut, ok, true, 0,
+                                                           n_ev, lim);
             __syncwarp();
             continue;
         }
