@@ -264,15 +264,13 @@ __device__ __forceinline__ float safe_rcp(float x)
 // file; t_max, the farthest kept depth once full, stays in a register. A key is one 64-bit number,
 // the depth's bits mapped so that they order as the depths do, then the index: an insertion moves
 // and compares whole keys (1M 1080p frame 3.51 -> 3.23 ms against separate depths and indices).
-// Depths that compare equal have equal keys: -0 is taken as +0 (a ray that starts at the mean of
-// several Gaussians has both among its depths, and a round goes on behind the last key's depth and
-// index, see key_after).
+// Depths that compare equal have to have equal keys, so no depth may be -0 (see sphere_test).
 // ------------------------------------------------------------------------------------------
 constexpr int kBlock = 128;
 
 __device__ __forceinline__ uint64_t make_key(float t, uint32_t i)
 {
-    const uint32_t b = __float_as_uint(__fadd_rn(t, 0.0f));
+    const uint32_t b = __float_as_uint(t);
     return ((uint64_t)(b ^ ((uint32_t)((int)b >> 31) | 0x80000000u)) << 32) | i;
 }
 __device__ __forceinline__ float depth_of_key(uint64_t k)
@@ -483,13 +481,17 @@ __device__ __forceinline__ void sphere_refine(float4 r0, float4 r1, float4 r2, f
     for (int c = 0; c < 3; ++c) w[c] = fmaf(-delta, dc[c], wh[c] + wl[c]);
 }
 
-// Full test of one Gaussian record: returns true for a hit candidate and then (t, D2, w).
+// Full test of one Gaussian record: returns true for a hit candidate and then (t, D2, w). A depth of -0
+// becomes +0: a ray that starts at the mean of several Gaussians has zeros of either sign among its
+// depths, and a round goes on behind the last key's depth and index (key_after), which compares them as
+// equal. (The tile walk takes no ray with t_near < 0, hence has no such depth.)
 __device__ __forceinline__ bool sphere_test(const float4 *__restrict__ g, float3 o, float3 d, float &t, float &D2,
                                             float w[3])
 {
     float4 r0 = __ldg(g), r1 = __ldg(g + 1), r2 = __ldg(g + 2);
     if (!sphere_candidate(r0, r1, r2, o, d, t)) return false;
     sphere_refine(r0, r1, r2, o, d, t, D2, w);
+    t = __fadd_rn(t, 0.0f);
     return true;
 }
 
@@ -2304,6 +2306,7 @@ __device__ __forceinline__ bool ray_walk(const TraceArgs &a, const SceneRef &sc,
             bool hit = lane < m && sphere_candidate(r0, r1, r2, o, d, t, aa) && in_range(t, aa, tn, bound);
             if (hit) {
                 sphere_refine(r0, r1, r2, o, d, t, D2, u);
+                t = __fadd_rn(t, 0.0f);                              // (see sphere_test)
                 hit = D2 <= 1.0f && t > tn && t <= tf && !(t > bound);
                 q = 1.0f - fminf(r3.x * exp2f(r3.y * D2), a.alpha_max);
             }
