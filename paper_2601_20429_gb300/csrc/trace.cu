@@ -248,9 +248,17 @@ int run(grtx_scene *sc, TraceArgs &a, int k, bool instr, int pass, unsigned *que
     // bundles of a ray list may be left to k_trace_rays: their list lies behind the others (room for it
     // whether this call leaves any or not, so that the workspace does not grow from call to call)
     const bool walk = form == FORM_SPHERE && !instr && ckpt;
-    a.split = walk ? split_for(a.n_items / 32, (unsigned)blocks * (kBlock / 32)) : 0;
-    a.middle = walk && a.n_items / 32 > (unsigned)blocks * (kBlock / 32);
+    const unsigned warps = (unsigned)blocks * (kBlock / 32);
     const bool leaves = walk && pass == PASS_FWD && a.cam.cam_type == GRTX_CAMERA_RAYS;
+    a.split = walk ? split_for(a.n_items / 32, warps) : 0;
+    // a list without an image's order (bounce rays) goes in smaller bundles, as in a batch: its rays share
+    // less, and a wide bundle of them is the launch's last (70,354 bounce rays over 6M Gaussians in bundles
+    // of 32 / 16 / 8 / 4: 7.9-9.6 / 5.7-6.6 / 4.7-5.1 / 3.8-4.7 ms; 8 with kListWork: 3.36)
+    if (leaves && a.cam.tiles_x == 0) {
+        a.split = std::max(a.split, split_for(a.n_items / 32, 2 * warps, 2));
+        a.leave_at = kListWork;
+    }
+    a.middle = walk && a.n_items / 32 > warps;
     uint2 *base = nullptr;
     int st = ensure_workspace(sc, n_slots, per_slot, ckpt ? kLeftCap * sizeof(uint2) : 0, s, &base);
     if (st) return st;

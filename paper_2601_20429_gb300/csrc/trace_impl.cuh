@@ -61,6 +61,7 @@ struct TraceArgs {
     int n_slots;
     int split;                   // k_trace: a warp takes 32 >> split rays at a time (see split_for)
     int middle;                  // tiles are handed out from the middle row outwards (see middle_out)
+    int leave_at;                // work after which a bundle of several origins is left (see kWalkTrial)
     uint2 *left;                 // bundles left for k_trace_rays (counted in queue[4]), or NULL: the queue place, or
                                  // (batched views) the first item and the view
     int discard;                 // drop dead list lines from L2 after each tile (lists 256-byte aligned)
@@ -1428,7 +1429,13 @@ constexpr int kSqueeze = 64;
 // four is given up: its rays share almost nothing, and each traces the round on its own. Given up
 // after 128 / 256 / 512 / 1024, the 256x256 preview took 860 / 725 / 604 / 604 us (its wide tiles are
 // still far cheaper than rays on their own) and the 1080p frame 4.24 / 3.47 / 3.47 / 3.47 ms.
-constexpr int kWalkTrial = 512;
+// The work of rays of several origins that can be left to k_trace_rays (ray lists) counts double, since
+// the one-ray kernel costs them less, and a lone list leaves a bundle after kListWork of it whatever it
+// shares: the few bundles deep in fog are the launch's last, and go faster a ray to a warp. 70,354 bounce
+// rays over 6M Gaussians in bundles of 8, k = 16 / 32: neither 4.8 / 4.9 ms, counted double 4.4 / 3.5, left
+// after 1024 / 2048 / 3072 / 4096 / 6144 of it 3.6 / 3.36 / 3.4 / 3.9 / 4.1 ms (k = 16). In a batch the
+// one-ray kernel would begin only behind the images: 11.4 ms without kListWork, 11.6 with it.
+constexpr int kWalkTrial = 512, kListWork = 2048;
 
 // Which rays of one origin o may hit a Gaussian, as one quadratic in the ray's direction. A ray
 // d = mid + x meets the Gaussian where |o_l x d_l|^2 <= |d_l|^2 (o_l = A (o - mu), d_l = A d): with
@@ -1536,11 +1543,12 @@ __device__ __forceinline__ bool tile_walk(const TraceArgs &a, const SceneRef &sc
     }
     const int cap = a.packet_stack < kPacketStack ? a.packet_stack : kWalkStack;
     const int wide = cap - kWalkReserve;
+    const int unit = a.left && !one_origin ? 2 : 1, most = unit == 2 ? a.leave_at : 0x7fffffff;      // (see kWalkTrial)
     int sp = 1, nl = 0, work = 0, cands = 0;
     int squeeze_at = min(kSqueeze, max(a.evict_cap - 31, 1));
     for (;;) {
         // expand up to 32 pending nodes, nearest first (lane 0 takes the top of the stack)
-        if (sp >= cap || (work >= kWalkTrial && 4 * cands < work)) return false;   // no room, or nothing shared
+        if (sp >= cap || (work >= kWalkTrial && (4 * cands < work || work >= most))) return false;   // no room, or too little shared
         const int p = min(min(32, sp), max(1, wide - sp));
         uint32_t cn = GRTX_NONE, cf = GRTX_NONE;                     // near and far child to visit
         if (lane < p) {
@@ -1568,7 +1576,7 @@ __device__ __forceinline__ bool tile_walk(const TraceArgs &a, const SceneRef &sc
         const unsigned gn = __ballot_sync(full, ln), gf = __ballot_sync(full, lf);
         const unsigned below = (1u << lane) - 1u, above = ~(below | (1u << lane));
         sp -= p;
-        work += 4;
+        work += 4 * unit;
         int at = sp + __popc(bn & above) + __popc(bf & above);
         if (cf != GRTX_NONE && !lf) w.stack[at++] = cf;
         if (cn != GRTX_NONE && !ln) w.stack[at] = cn;
@@ -1612,7 +1620,7 @@ __device__ __forceinline__ bool tile_walk(const TraceArgs &a, const SceneRef &sc
                 }
             }
             if (!(valid && lane_ok)) mask = 0;
-            work += m;
+            work += m * unit;
             cands += __reduce_add_sync(full, __popc(mask));
             // ... then the candidates of each ray one after another
             while (mask) {
@@ -2583,6 +2591,7 @@ inline void set_window(TraceArgs &a)
     a.window = a.traversal == GRTX_TRAVERSAL_CHECKPOINT ? cap / 4 : 0;
     a.p_stop = a.T_min >= 1e-30f ? 0.98f * a.T_min : 0.0f;
     a.id_shift = 0;
+    a.leave_at = 0x7fffffff;
 }
 
 // Opacity codes in the list entries: for the walk (uninstrumented sphere-form kernels), where the
