@@ -1836,7 +1836,7 @@ __device__ __forceinline__ void save_blended(const TraceArgs &a, int64_t pix, in
 template <int K, int FORM, bool INSTR, int PASS>
 __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc, float4 *__restrict__ out, int slot,
                                           int64_t pix, float3 o, float3 d, float tn, float tf, KBuf<K> &kb,
-                                          Counters &cnt, Cut cut, bool r1_done = false, bool r1_ok = true,
+                                          Counters &cnt, Cut cut, unsigned live, bool r1_done = false, bool r1_ok = true,
                                           int r1_n_dst = 0, int r1_n_ev = 0, float lim = INFINITY)
 {
     constexpr bool BWD = PASS == PASS_BWD;
@@ -1864,7 +1864,13 @@ __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc
     const uint32_t ev = a.ev_off + (uint32_t)slot;
     bool done = !sc.has_tree;
     bool first_round = true;
-    while (!done) {
+    // The lanes of `live` (the caller's mask of this call) meet at each round, and a lane that restarts runs
+    // the same code as the others: each lane's round is a loop of its own, and lanes that are not made to meet
+    // run the rounds one lane after another (640x360 of 1M Gaussians with eviction lists of 16: 3.5 ms, 5.4
+    // with the restarted round in a copy of its code, 12.6 with neither).
+    for (;;) {
+        live = __ballot_sync(live, !done);
+        if (done) break;
         if (INSTR) cnt.rounds++;
         if (!(r1_done && first_round)) kb.clear();
         if (ckpt && n_ev > 0) {            // raygen: closest evicted hits -> k-buffer
@@ -1895,14 +1901,14 @@ __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc
         }
         if (!round_ok) {
             // a capacity was exceeded: redo this round from the root and stay in restart mode
-            if (INSTR) cnt.fallbacks++;
+            if (INSTR) {
+                cnt.fallbacks++;
+                cnt.rounds--;
+            }
             ckpt = false;
             from_root = true;
-            n_src = 0;
-            n_ev = 0;
-            kb.clear();
-            trace_round<K, FORM, INSTR>(a, sc, o, d, inv, inv_len, tn, tf, Lt, Li, false, true, src, 0, dst, n_dst, ev, n_ev,
-                                         kb, cut, 0, cnt);
+            first_round = false;
+            continue;
         }
         for (int j = 0; j < kb.n; ++j) {
             uint32_t idx = kb.I(j) >> a.id_shift;
@@ -1916,9 +1922,12 @@ __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc
             if (st.T < a.T_min) { done = true; break; }
         }
         first_round = false;
-        if (done) break;
+        if (done) continue;
         if (kb.n < K) {
-            if (!(lim < GRTX_INF)) break;
+            if (!(lim < GRTX_INF)) {
+                done = true;
+                continue;
+            }
             // every hit up to the limit of the first round is blended: go on behind it, from the root
             Lt = lim;
             Li = GRTX_NONE;
@@ -2036,7 +2045,7 @@ __device__ __forceinline__ void trace_warp_restart(const TraceArgs &a, const Sce
 // own. Every lane of the warp calls this together; lanes without a ray pass valid = false. In
 // the backward, a ray whose forward saved its whole blend list takes it from there and leaves
 // the traversal to the others.
-template <int K, int FORM, bool INSTR, int PASS>
+template <int K, int FORM, bool INSTR, int PASS, bool WALK_ONLY = false>
 __device__ __forceinline__ void trace_warp(const TraceArgs &a, const SceneRef &sc, float4 *__restrict__ out, int slot,
                                            bool valid, int64_t pix, float3 o, float3 d, float tn, float tf, KBuf<K> &kb,
                                            Counters &cnt, uint4 *pst)
@@ -2062,7 +2071,7 @@ __device__ __forceinline__ void trace_warp(const TraceArgs &a, const SceneRef &s
     bool lane_ok = true;
     float lim = GRTX_INF;
     constexpr bool WALKS = FORM == FORM_SPHERE && !INSTR;        // (where the lists are used)
-    const bool walked = WALKS && a.traversal == GRTX_TRAVERSAL_CHECKPOINT;
+    const bool walked = WALK_ONLY || (WALKS && a.traversal == GRTX_TRAVERSAL_CHECKPOINT);
     static_assert(sizeof(WalkShared) <= kWarpShared * sizeof(uint4), "the walk's shared memory");
     if (walked) {
         if (sc.has_tree && !tile_walk<K>(a, sc, valid, *reinterpret_cast<WalkShared *>(pst), o, d, tn, tf,
@@ -2097,8 +2106,9 @@ __device__ __forceinline__ void trace_warp(const TraceArgs &a, const SceneRef &s
         cut.clear();
         lim = GRTX_INF;
     }
+    const unsigned rays = __ballot_sync(0xffffffffu, valid);
     if (valid)
-        trace_ray<K, FORM, INSTR, PASS>(a, sc, out, slot, pix, o, d, tn, tf, kb, cnt, cut, !WALKS || lane_ok, WALKS || lane_ok,
+        trace_ray<K, FORM, INSTR, PASS>(a, sc, out, slot, pix, o, d, tn, tf, kb, cnt, cut, rays, !WALKS || lane_ok, WALKS || lane_ok,
                                         n_dst, n_ev, lim);
 }
 
@@ -2185,10 +2195,10 @@ inline int split_for(unsigned tiles, unsigned warps, int most = 3)
 }
 
 // Traversal a frame kernel is compiled for: either (chosen per launch by a.traversal), or one
-// of them only. The forward sphere-form kernel has one instantiation per traversal (TRAV_CKPT
-// also serves any traversal but restart): without the other traversal's code, the register
-// allocation of the one that runs is better (the checkpointed frame kernel spills 100 B
-// instead of 112 B and runs 0.5 % faster).
+// of them only. The forward sphere-form kernel has one instantiation per traversal, and the
+// checkpointed one none of the packet's code: without what does not run, the register allocation of
+// what does is better (1M 1080p frame 3.591 -> 3.587 ms without the packet, a burst of 16 server requests
+// 7.22 -> 7.16 ms).
 constexpr int TRAV_ANY = 0, TRAV_CKPT = 1, TRAV_RESTART = 2;
 
 template <int K, int FORM, bool INSTR, int PASS, int TRAV = TRAV_ANY>
@@ -2224,7 +2234,7 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, PASS == PASS_BWD))
             trace_warp_restart<K, FORM, INSTR, PASS == PASS_SAVE>(a, a.sc, a.rgbT, slot, valid, pix, o, d, tn, tf,
                                                                   kb, cnt, s_pst[threadIdx.x >> 5]);
         else if constexpr (TRAV == TRAV_CKPT)
-            trace_warp<K, FORM, INSTR, PASS>(a, a.sc, a.rgbT, slot, valid, pix, o, d, tn, tf, kb, cnt,
+            trace_warp<K, FORM, INSTR, PASS, true>(a, a.sc, a.rgbT, slot, valid, pix, o, d, tn, tf, kb, cnt,
                                              s_pst[threadIdx.x >> 5]);
         else if (PASS != PASS_BWD && a.traversal == GRTX_TRAVERSAL_RESTART)
             trace_warp_restart<K, FORM, INSTR, PASS == PASS_SAVE>(a, a.sc, a.rgbT, slot, valid, pix, o, d, tn, tf,
@@ -2402,7 +2412,7 @@ __global__ void __launch_bounds__(kBlock, 5) k_trace_rays(const __grid_constant_
                 lim = GRTX_INF;
             }
             if (lane == 0)
-                trace_ray<K, FORM_SPHERE, false, PASS_FWD>(a, sc, out, slot, pix, o, d, tn, tf, kb, cnt, cut, ok, true, 0,
+                trace_ray<K, FORM_SPHERE, false, PASS_FWD>(a, sc, out, slot, pix, o, d, tn, tf, kb, cnt, cut, 1u, ok, true, 0,
                                                            n_ev, lim);
             __syncwarp();
             continue;
@@ -2552,7 +2562,7 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, false))
             trace_warp_restart<K, FORM_SPHERE, false, false>(a, sc, sg.out, slot, valid, pix, o, d, tn, tf, kb, cnt,
                                                       s_pst[threadIdx.x >> 5]);
         else
-            trace_warp<K, FORM_SPHERE, false, PASS_FWD>(a, sc, sg.out, slot, valid, pix, o, d, tn, tf, kb, cnt,
+            trace_warp<K, FORM_SPHERE, false, PASS_FWD, true>(a, sc, sg.out, slot, valid, pix, o, d, tn, tf, kb, cnt,
                                                      s_pst[threadIdx.x >> 5]);
         if (live.seg_done) {
             // the tile's pixels are written; the warp that completes the segment raises its

@@ -168,7 +168,8 @@ __device__ __forceinline__ void single_ray(const TraceArgs &a, const SceneRef &s
             if (INSTR) cnt.fallbacks++;
             Cut cut;
             cut.clear();
-            trace_ray<kFallbackK, FORM, INSTR, false>(a, sc, a.rgbT, slot, pix, o, d, tn, tf, kb, cnt, cut);
+            trace_ray<kFallbackK, FORM, INSTR, false>(a, sc, a.rgbT, slot, pix, o, d, tn, tf, kb, cnt, cut,
+                                                       1u << (threadIdx.x & 31));
             return;
         }
     }
