@@ -464,6 +464,17 @@ GRTX_API int grtx_generate_rays(const grtx_camera *cam, float *d_origins, float 
 GRTX_API int grtx_trace_forward(grtx_scene *scene, const grtx_camera *cam, const grtx_params *p,
                                 const grtx_trace_outputs *out, void *stream);
 
+/* The trace of grtx_trace_forward without optional outputs, by kernels whose walks compare every
+ * node, leaf slot, stack, leaf-list, eviction-list and left-list index with the size of its array
+ * before they use it; an index outside is left out and added to *d_errors (device, uint64, not
+ * cleared by the call). For tests: the counters of grtx_stats come from kernels that take the first
+ * round as a packet, so bounds_errors does not cover the walks. rgbT as in grtx_trace_forward, the
+ * same image. max_nodes > 0: nodes from that index on count as outside (a test of the check itself;
+ * the image lacks what lies below them). Sphere form over binary nodes, checkpoint traversal, k = 16
+ * (GRTX_ERR_INVALID_ARG otherwise). */
+GRTX_API int grtx_trace_self_check(grtx_scene *scene, const grtx_camera *cam, const grtx_params *p,
+                                   float *d_rgbT, int64_t max_nodes, uint64_t *d_errors, void *stream);
+
 #define GRTX_MAX_BATCH 64
 
 /* Trace several cameras or ray lists of one scene in one persistent launch (the segments of
@@ -643,6 +654,11 @@ GRTX_API int grtx_world_update(grtx_world *world, const grtx_instance *inst, int
  * scenes'. The world's trace workspace is grown on demand (stream-ordered allocation). */
 GRTX_API int grtx_world_trace_forward(grtx_world *world, const grtx_camera *cam, const grtx_params *p,
                                       const grtx_trace_outputs *out, void *stream);
+
+/* grtx_trace_self_check for a world: the walk over the scene level and the walks of its objects.
+ * Checkpoint traversal, k = 16. */
+GRTX_API int grtx_world_self_check(grtx_world *world, const grtx_camera *cam, const grtx_params *p, float *d_rgbT,
+                                   uint64_t *d_errors, void *stream);
 
 /* Release a world (waits for its work on the last stream it used; NULL is a no-op). */
 GRTX_API void grtx_world_destroy(grtx_world *world);

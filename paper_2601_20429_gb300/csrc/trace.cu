@@ -420,6 +420,22 @@ int segments_occupancy_k(int k, int traversal, int *bps)
 
 }  // namespace
 
+extern "C" GRTX_API int grtx_trace_self_check(grtx_scene *sc, const grtx_camera *cam, const grtx_params *p, float *d_rgbT,
+                                              int64_t max_nodes, uint64_t *d_errors, void *stream)
+{
+    TraceArgs a = {};
+    int st = setup(sc, cam, p, a);
+    if (st) return st;
+    if (sc->form != GRTX_FORM_SPHERE || p->bvh_width == 4 || p->traversal != GRTX_TRAVERSAL_CHECKPOINT || p->k != kCheckK)
+        return grtx_fail(GRTX_ERR_INVALID_ARG, "checked walks: sphere form over binary nodes, checkpoint traversal, k = 16");
+    if (!d_rgbT || ((uintptr_t)d_rgbT & 15)) return grtx_fail(GRTX_ERR_INVALID_ARG, "rgbT must be a 16-byte aligned pointer");
+    if (!d_errors) return grtx_fail(GRTX_ERR_INVALID_ARG, "d_errors is NULL");
+    a.rgbT = (float4 *)d_rgbT;
+    a.check = reinterpret_cast<unsigned long long *>(d_errors);
+    if (max_nodes > 0) a.sc.n_nodes = (uint32_t)std::min<int64_t>(a.sc.n_nodes, max_nodes);
+    return run(sc, a, p->k, false, PASS_FWD, sc->d_counter, S(stream));
+}
+
 extern "C" GRTX_API int grtx_trace_forward_batch(grtx_scene *sc, const grtx_camera *cams, int n_cams,
                                                  const grtx_params *p, float *const *rgbT, void *stream)
 {

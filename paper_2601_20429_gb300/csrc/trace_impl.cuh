@@ -66,6 +66,7 @@ struct TraceArgs {
                                  // (batched views) the first item and the view
     int discard;                 // drop dead list lines from L2 after each tile (lists 256-byte aligned)
     unsigned *queue;
+    unsigned long long *check;   // failed checks of the checked kernels (see in_bounds), or NULL
     // outputs
     float4 *rgbT;
     int32_t *n_blended;
@@ -154,7 +155,9 @@ __device__ __forceinline__ void log_visit(Counters &c, uint32_t ref)
 // leaf record is fetched its index is compared with the size of its array, and so is the
 // Gaussian index a proxy triangle names. An index outside is counted (grtx_stats.bounds_errors)
 // and not fetched; the traversal treats it as a miss. Every parity render runs these kernels,
-// so every parity case is also a check that the traversal never leaves the scene's arrays.
+// so every parity case is also a check that their traversal never leaves the scene's arrays. They
+// take the first round as a packet: the walks, which the uninstrumented kernels take it by, have
+// checked instantiations of their own (in_bounds, grtx_trace_self_check).
 __device__ __forceinline__ bool ref_ok(const SceneRef &sc, uint32_t ref, Counters &c, bool count = true)
 {
     bool ok = (ref & GRTX_LEAF) ? (ref & ~GRTX_LEAF) < sc.n_leaves : ref < sc.n_nodes;
@@ -173,6 +176,16 @@ __device__ __forceinline__ bool gauss_ok(const SceneRef &sc, uint32_t gi, Counte
 {
     if (gi < sc.n_geom) return true;
     ++c.oob;
+    return false;
+}
+
+// Check of the walks' checked instantiations (CHK): an index outside its array is counted in *a.check,
+// and the caller leaves the access out.
+template <bool CHK>
+__device__ __forceinline__ bool in_bounds(const TraceArgs &a, uint32_t i, uint32_t n)
+{
+    if (!CHK || i < n) return true;
+    atomicAdd(a.check, 1ull);
     return false;
 }
 
@@ -1376,6 +1389,19 @@ __device__ __forceinline__ float warp_max(float v)
     return v;
 }
 
+// Checks of a checked walk: the pending node at entry e of the stack; the leaf slots among a node's
+// children.
+template <bool CHK>
+__device__ __forceinline__ bool next_node(const TraceArgs &a, const SceneRef &sc, const WalkShared &w, int e)
+{
+    return !CHK || (in_bounds<CHK>(a, (uint32_t)e, kWalkStack) && in_bounds<CHK>(a, w.stack[e], sc.n_nodes));
+}
+__device__ __forceinline__ void drop_bad_leaves(const TraceArgs &a, const SceneRef &sc, uint32_t &c0, uint32_t &c1)
+{
+    if (c0 != GRTX_NONE && (c0 & GRTX_LEAF) && !in_bounds<true>(a, c0 & ~GRTX_LEAF, sc.n_geom)) c0 = GRTX_NONE;
+    if (c1 != GRTX_NONE && (c1 & GRTX_LEAF) && !in_bounds<true>(a, c1 & ~GRTX_LEAF, sc.n_geom)) c1 = GRTX_NONE;
+}
+
 // One axis of the bundle test. A ray of the bundle is inside [lo, hi] on this axis at depth t only
 // if lo <= o_max + t d_max and hi >= o_min + t d_min; each condition bounds t from below or from
 // above, by the sign of its direction bound (c[1], c[3] hold the reciprocals).
@@ -1493,7 +1519,7 @@ struct ConeTest {
 // lane_ok becomes false for a ray whose eviction list was too small. Returns false if the bundle was
 // left: no stack, a ray that cannot be bounded, or too little shared. base: added to the leaf slots
 // (a world's objects; the state of the rays goes on from call to call).
-template <int K>
+template <int K, bool CHK = false>
 __device__ __forceinline__ bool tile_walk(const TraceArgs &a, const SceneRef &sc, bool valid, WalkShared &w,
                                           float3 o, float3 d, float tn, float tf, uint32_t ev, int &n_ev, KBuf<K> &kb,
                                           Cut &cut, float &lim, bool &lane_ok, uint32_t base = 0u)
@@ -1552,7 +1578,7 @@ __device__ __forceinline__ bool tile_walk(const TraceArgs &a, const SceneRef &sc
         if (sp >= cap || (work >= kWalkTrial && (4 * cands < work || work >= most))) return false;   // no room, or too little shared
         const int p = min(min(32, sp), max(1, wide - sp));
         uint32_t cn = GRTX_NONE, cf = GRTX_NONE;                     // near and far child to visit
-        if (lane < p) {
+        if (lane < p && next_node<CHK>(a, sc, w, sp - 1 - lane)) {
             const float4 *nd = sc.nodes + 4 * (size_t)w.stack[sp - 1 - lane];
             float4 n0, n1, n2, n3;
             ldg2(nd, n0, n1);
@@ -1570,6 +1596,7 @@ __device__ __forceinline__ bool tile_walk(const TraceArgs &a, const SceneRef &sc
             if (e1 < e0) {
                 const uint32_t t = cn; cn = cf; cf = t;
             }
+            if (CHK) drop_bad_leaves(a, sc, cn, cf);
         }
         __syncwarp();
         const bool ln = cn != GRTX_NONE && (cn & GRTX_LEAF), lf = cf != GRTX_NONE && (cf & GRTX_LEAF);
@@ -1579,12 +1606,12 @@ __device__ __forceinline__ bool tile_walk(const TraceArgs &a, const SceneRef &sc
         sp -= p;
         work += 4 * unit;
         int at = sp + __popc(bn & above) + __popc(bf & above);
-        if (cf != GRTX_NONE && !lf) w.stack[at++] = cf;
-        if (cn != GRTX_NONE && !ln) w.stack[at] = cn;
+        if (cf != GRTX_NONE && !lf && in_bounds<CHK>(a, at, kWalkStack)) w.stack[at++] = cf;
+        if (cn != GRTX_NONE && !ln && in_bounds<CHK>(a, at, kWalkStack)) w.stack[at] = cn;
         sp += __popc(bn) + __popc(bf);
         at = nl + __popc(gn & below) + __popc(gf & below);
-        if (ln) w.leaf[at++] = cn & ~GRTX_LEAF;
-        if (lf) w.leaf[at] = cf & ~GRTX_LEAF;
+        if (ln && in_bounds<CHK>(a, at, kWalkLeaves)) w.leaf[at++] = cn & ~GRTX_LEAF;
+        if (lf && in_bounds<CHK>(a, at, kWalkLeaves)) w.leaf[at] = cf & ~GRTX_LEAF;
         nl += __popc(gn) + __popc(gf);
         __syncwarp();
         if (sp > 0 && nl <= kWalkLeaves - 64) continue;
@@ -1643,7 +1670,7 @@ __device__ __forceinline__ bool tile_walk(const TraceArgs &a, const SceneRef &sc
                             lane_ok = false;
                             break;
                         }
-                        L[ev + (uint32_t)n_ev * S] = make_uint2(__float_as_uint(ct), ci);
+                        if (in_bounds<CHK>(a, n_ev, a.evict_cap)) L[ev + (uint32_t)n_ev * S] = make_uint2(__float_as_uint(ct), ci);
                         ++n_ev;
                     }
                 }
@@ -2045,7 +2072,7 @@ __device__ __forceinline__ void trace_warp_restart(const TraceArgs &a, const Sce
 // own. Every lane of the warp calls this together; lanes without a ray pass valid = false. In
 // the backward, a ray whose forward saved its whole blend list takes it from there and leaves
 // the traversal to the others.
-template <int K, int FORM, bool INSTR, int PASS, bool WALK_ONLY = false>
+template <int K, int FORM, bool INSTR, int PASS, bool WALK_ONLY = false, bool CHK = false>
 __device__ __forceinline__ void trace_warp(const TraceArgs &a, const SceneRef &sc, float4 *__restrict__ out, int slot,
                                            bool valid, int64_t pix, float3 o, float3 d, float tn, float tf, KBuf<K> &kb,
                                            Counters &cnt, uint4 *pst)
@@ -2074,7 +2101,7 @@ __device__ __forceinline__ void trace_warp(const TraceArgs &a, const SceneRef &s
     const bool walked = WALK_ONLY || (WALKS && a.traversal == GRTX_TRAVERSAL_CHECKPOINT);
     static_assert(sizeof(WalkShared) <= kWarpShared * sizeof(uint4), "the walk's shared memory");
     if (walked) {
-        if (sc.has_tree && !tile_walk<K>(a, sc, valid, *reinterpret_cast<WalkShared *>(pst), o, d, tn, tf,
+        if (sc.has_tree && !tile_walk<K, CHK>(a, sc, valid, *reinterpret_cast<WalkShared *>(pst), o, d, tn, tf,
                                          a.ev_off + (uint32_t)slot, n_ev, kb, cut, lim, lane_ok)) {
             // a bundle that cannot be walked: its rays trace the round on their own, one to a warp where
             // the left list has room, or here
@@ -2083,7 +2110,8 @@ __device__ __forceinline__ void trace_warp(const TraceArgs &a, const SceneRef &s
                 __all_sync(0xffffffffu, *reinterpret_cast<volatile unsigned *>(a.queue + 4) < kLeftCap - kLeftRoom)) {
                 if ((threadIdx.x & 31) == 0) {
                     reinterpret_cast<WalkShared *>(pst)->rows = -1;
-                    a.left[atomicAdd(a.queue + 4, 1u)] = reinterpret_cast<WalkShared *>(pst)->place;
+                    const unsigned to = atomicAdd(a.queue + 4, 1u);
+                    if (in_bounds<CHK>(a, to, kLeftCap)) a.left[to] = reinterpret_cast<WalkShared *>(pst)->place;
                 }
                 return;
             }
@@ -2199,7 +2227,8 @@ inline int split_for(unsigned tiles, unsigned warps, int most = 3)
 // checkpointed one none of the packet's code: without what does not run, the register allocation of
 // what does is better (1M 1080p frame 3.591 -> 3.587 ms without the packet, a burst of 16 server requests
 // 7.22 -> 7.16 ms).
-constexpr int TRAV_ANY = 0, TRAV_CKPT = 1, TRAV_RESTART = 2;
+// TRAV_CHECK: TRAV_CKPT with checked walks.
+constexpr int TRAV_ANY = 0, TRAV_CKPT = 1, TRAV_RESTART = 2, TRAV_CHECK = 3;
 
 template <int K, int FORM, bool INSTR, int PASS, int TRAV = TRAV_ANY>
 __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, PASS == PASS_BWD)) k_trace(TraceArgs a)
@@ -2233,8 +2262,8 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, PASS == PASS_BWD))
         if constexpr (TRAV == TRAV_RESTART && PASS != PASS_BWD)
             trace_warp_restart<K, FORM, INSTR, PASS == PASS_SAVE>(a, a.sc, a.rgbT, slot, valid, pix, o, d, tn, tf,
                                                                   kb, cnt, s_pst[threadIdx.x >> 5]);
-        else if constexpr (TRAV == TRAV_CKPT)
-            trace_warp<K, FORM, INSTR, PASS, true>(a, a.sc, a.rgbT, slot, valid, pix, o, d, tn, tf, kb, cnt,
+        else if constexpr (TRAV == TRAV_CKPT || TRAV == TRAV_CHECK)
+            trace_warp<K, FORM, INSTR, PASS, true, TRAV == TRAV_CHECK>(a, a.sc, a.rgbT, slot, valid, pix, o, d, tn, tf, kb, cnt,
                                              s_pst[threadIdx.x >> 5]);
         else if (PASS != PASS_BWD && a.traversal == GRTX_TRAVERSAL_RESTART)
             trace_warp_restart<K, FORM, INSTR, PASS == PASS_SAVE>(a, a.sc, a.rgbT, slot, valid, pix, o, d, tn, tf,
@@ -2263,7 +2292,7 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, PASS == PASS_BWD))
 // The walk of one ray: every lane holds it, the lanes expand its pending nodes and take its leaves
 // through the exact test side by side, and lane 0 collects the hits (its k-buffer and eviction list).
 // False if the stack or the eviction list is too small.
-template <int K>
+template <int K, bool CHK = false>
 __device__ __forceinline__ bool ray_walk(const TraceArgs &a, const SceneRef &sc, WalkShared &w, float3 o, float3 d, float tn,
                                          float tf, uint32_t ev, int &n_ev, KBuf<K> &kb, Cut &cut, float &lim)
 {
@@ -2288,7 +2317,7 @@ __device__ __forceinline__ bool ray_walk(const TraceArgs &a, const SceneRef &sc,
         if (sp >= cap || !__all_sync(full, ok)) return false;        // no room for children or hits
         const int p = min(min(32, sp), max(1, wide - sp));
         uint32_t cn = GRTX_NONE, cf = GRTX_NONE;
-        if (lane < p) {
+        if (lane < p && next_node<CHK>(a, sc, w, sp - 1 - lane)) {
             const float4 *nd = sc.nodes + 4 * (size_t)w.stack[sp - 1 - lane];
             const float4 n0 = __ldg(nd), n1 = __ldg(nd + 1), n2 = __ldg(nd + 2), n3 = __ldg(nd + 3);
             float e0, x0, e1, x1;
@@ -2299,6 +2328,7 @@ __device__ __forceinline__ bool ray_walk(const TraceArgs &a, const SceneRef &sc,
             if (e1 < e0) {
                 const uint32_t t = cn; cn = cf; cf = t;
             }
+            if (CHK) drop_bad_leaves(a, sc, cn, cf);
         }
         __syncwarp();
         const bool ln = cn != GRTX_NONE && (cn & GRTX_LEAF), lf = cf != GRTX_NONE && (cf & GRTX_LEAF);
@@ -2307,12 +2337,12 @@ __device__ __forceinline__ bool ray_walk(const TraceArgs &a, const SceneRef &sc,
         const unsigned below = (1u << lane) - 1u, above = ~(below | (1u << lane));
         sp -= p;
         int at = sp + __popc(bn & above) + __popc(bf & above);
-        if (cf != GRTX_NONE && !lf) w.stack[at++] = cf;
-        if (cn != GRTX_NONE && !ln) w.stack[at] = cn;
+        if (cf != GRTX_NONE && !lf && in_bounds<CHK>(a, at, kWalkStack)) w.stack[at++] = cf;
+        if (cn != GRTX_NONE && !ln && in_bounds<CHK>(a, at, kWalkStack)) w.stack[at] = cn;
         sp += __popc(bn) + __popc(bf);
         at = nl + __popc(gn & below) + __popc(gf & below);
-        if (ln) w.leaf[at++] = cn & ~GRTX_LEAF;
-        if (lf) w.leaf[at] = cf & ~GRTX_LEAF;
+        if (ln && in_bounds<CHK>(a, at, kWalkLeaves)) w.leaf[at++] = cn & ~GRTX_LEAF;
+        if (lf && in_bounds<CHK>(a, at, kWalkLeaves)) w.leaf[at] = cf & ~GRTX_LEAF;
         nl += __popc(gn) + __popc(gf);
         __syncwarp();
         if (sp > 0 && nl < 32) continue;
@@ -2340,7 +2370,7 @@ __device__ __forceinline__ bool ray_walk(const TraceArgs &a, const SceneRef &sc,
                         if (n_ev >= a.evict_cap) {
                             ok = false;
                         } else {
-                            L[ev + (uint32_t)n_ev * S] = make_uint2(__float_as_uint(ct), ci);
+                            if (in_bounds<CHK>(a, n_ev, a.evict_cap)) L[ev + (uint32_t)n_ev * S] = make_uint2(__float_as_uint(ct), ci);
                             ++n_ev;
                         }
                     }
@@ -2373,7 +2403,7 @@ __device__ __forceinline__ bool ray_walk(const TraceArgs &a, const SceneRef &sc,
 // about 30 steps of up to 32 nodes, and every resident warp has one: 20,011 scattered rays over 1M
 // Gaussians, k = 32, 1.90 -> 0.53 ms. The blend spreads over the lanes too: lane j takes entry j of the
 // sorted k-buffer to its alpha and colour, then every lane composites them in order.
-template <int K>
+template <int K, bool CHK>
 __global__ void __launch_bounds__(kBlock, 5) k_trace_rays(const __grid_constant__ TraceArgs a, const ServeSeg *segs)
 {
     const unsigned full = 0xffffffffu;
@@ -2396,6 +2426,7 @@ __global__ void __launch_bounds__(kBlock, 5) k_trace_rays(const __grid_constant_
         float3 o, d;
         float tn, tf;
         const uint2 at = a.left[i / (unsigned)take];
+        if (!segs && !in_bounds<CHK>(a, at.x, a.n_items)) continue;
         const int r = (int)(i % (unsigned)take);
         if (!(segs ? r < (32 >> segs[at.y].split) && make_ray(segs[at.y].cam, at.x + (unsigned)r, pix, o, d, tn, tf)
                    : make_ray(a.cam, split_item(a, at.x, r), pix, o, d, tn, tf)))
@@ -2405,7 +2436,7 @@ __global__ void __launch_bounds__(kBlock, 5) k_trace_rays(const __grid_constant_
         Cut cut;
         float lim;
         int n_ev;
-        const bool ok = ray_walk<K>(a, sc, s_w[threadIdx.x >> 5], o, d, tn, tf, ev, n_ev, kb, cut, lim);
+        const bool ok = ray_walk<K, CHK>(a, sc, s_w[threadIdx.x >> 5], o, d, tn, tf, ev, n_ev, kb, cut, lim);
         if (!ok || __shfl_sync(full, lim, 0) < GRTX_INF) {
             if (!ok) {                                           // it begins anew
                 cut.clear();
@@ -2622,6 +2653,9 @@ inline int lists_discardable(const TraceArgs &a)
     return (m & 255u) == 0 && (a.n_slots % 32) == 0 && ((size_t)a.n_slots * sizeof(uint2)) % 256 == 0;
 }
 
+// k of the checked kernels (the walks are the same for every k).
+constexpr int kCheckK = 16;
+
 // Launch helpers, instantiated per k in the trace_k*.cu units.
 // form: FORM_* of the scene. The backward always runs the sphere leaf test: the icosphere
 // forms hit exactly the Gaussians the sphere form hits, and the proxy form has no backward.
@@ -2642,6 +2676,7 @@ int trace_launch(const TraceArgs &a, int form, bool instr, int pass, int blocks,
     else if (form == FORM_SPHERE4Q) k_trace<K, FORM_SPHERE4Q, false, PASS_FWD><<<g, b, 0, s>>>(a);
     else if (instr) k_trace<K, FORM_SPHERE, true, PASS_FWD><<<g, b, 0, s>>>(a);
     else if (a.traversal == GRTX_TRAVERSAL_RESTART) k_trace<K, FORM_SPHERE, false, PASS_FWD, TRAV_RESTART><<<g, b, 0, s>>>(a);
+    else if (K == kCheckK && a.check) k_trace<K, FORM_SPHERE, false, PASS_FWD, K == kCheckK ? TRAV_CHECK : TRAV_CKPT><<<g, b, 0, s>>>(a);
     else k_trace<K, FORM_SPHERE, false, PASS_FWD, TRAV_CKPT><<<g, b, 0, s>>>(a);
     return cudaGetLastError() == cudaSuccess ? GRTX_OK : GRTX_ERR_CUDA;
 }
@@ -2649,7 +2684,8 @@ int trace_launch(const TraceArgs &a, int form, bool instr, int pass, int blocks,
 template <int K>
 int trace_rays_launch(const TraceArgs &a, const ServeSeg *segs, int blocks, cudaStream_t s)
 {
-    k_trace_rays<K><<<blocks, kBlock, 0, s>>>(a, segs);
+    if (K == kCheckK && a.check) k_trace_rays<K, K == kCheckK><<<blocks, kBlock, 0, s>>>(a, segs);
+    else k_trace_rays<K, false><<<blocks, kBlock, 0, s>>>(a, segs);
     return cudaGetLastError() == cudaSuccess ? GRTX_OK : GRTX_ERR_CUDA;
 }
 

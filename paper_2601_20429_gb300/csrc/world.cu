@@ -374,7 +374,7 @@ __device__ __forceinline__ void world_packet_round(const WorldArgs &W, bool vali
 // 1280x720, k = 16: 5.84 ms with world_packet_round and per-ray later rounds, 3.06 ms with the walk.
 constexpr int kWorldWalkStack = kMaxTlasDepth + 1;
 
-template <int K>
+template <int K, bool CHK>
 __device__ __forceinline__ bool world_walk(const WorldArgs &W, bool valid, uint2 *tst, WalkShared &w, float3 o, float3 d,
                                            float3 inv, float tn, float tf, uint32_t ev, int &n_ev, KBuf<K> &kb, Cut &cut,
                                            float &lim, bool &lane_ok)
@@ -392,11 +392,13 @@ __device__ __forceinline__ bool world_walk(const WorldArgs &W, bool valid, uint2
         const bool in = ((m >> lane) & 1u) && lane_ok;
         const float bound = fminf(fminf(tf, lim), cut.top(W.a));
         if (ref & GRTX_LEAF) {
+            if (!in_bounds<CHK>(W.a, ref & ~GRTX_LEAF, (uint32_t)W.n_inst)) return false;
             const InstRec &I = W.inst[ref & ~GRTX_LEAF];
             float3 oo, od;
             to_object(I, o, d, oo, od);
-            if (!tile_walk<K>(W.a, I.sc, in, w, oo, od, tn, tf, ev, n_ev, kb, cut, lim, lane_ok, I.leaf_base)) return false;
+            if (!tile_walk<K, CHK>(W.a, I.sc, in, w, oo, od, tn, tf, ev, n_ev, kb, cut, lim, lane_ok, I.leaf_base)) return false;
         } else {
+            if (!in_bounds<CHK>(W.a, ref, (uint32_t)W.n_tl_nodes)) return false;
             const float4 *nd = W.tl_nodes + 4 * (size_t)ref;
             const float4 n0 = __ldg(nd), n1 = __ldg(nd + 1), n2 = __ldg(nd + 2), n3 = __ldg(nd + 3);
             const uint32_t c0 = __float_as_uint(n3.x), c1 = __float_as_uint(n3.y);
@@ -409,6 +411,7 @@ __device__ __forceinline__ bool world_walk(const WorldArgs &W, bool valid, uint2
                 const unsigned both = m0 & m1, vote = __ballot_sync(full, h0 && h1 && e0 <= e1);
                 const bool first0 = both ? 2 * __popc(vote) >= __popc(both) : __popc(m0) >= __popc(m1);
                 __syncwarp();
+                if (!in_bounds<CHK>(W.a, sp, kWorldWalkStack)) return false;
                 if (lane == 0) tst[sp] = make_uint2(first0 ? c1 : c0, first0 ? m1 : m0);
                 ++sp;
                 ref = first0 ? c0 : c1;
@@ -532,8 +535,8 @@ __device__ __forceinline__ void world_ray(const WorldArgs &W, int slot, int64_t 
     if (INSTR && a.n_blended) a.n_blended[pix] = nb;
 }
 
-// WALKS: uninstrumented checkpointed traces, round 1 as world_walk (a.ck0 = a.ev).
-template <int K, bool INSTR, bool WALKS>
+// WALKS: uninstrumented checkpointed traces, round 1 as world_walk (a.ck0 = a.ev). CHK: with checked walks.
+template <int K, bool INSTR, bool WALKS, bool CHK = false>
 __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, false)) k_trace_world(WorldArgs W)
 {
     __shared__ uint64_t s_k[K * kBlock];
@@ -568,7 +571,7 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, false)) k_trace_wo
         if constexpr (WALKS) {
             Cut cut;
             cut.clear();
-            if (!world_walk<K>(W, valid, s_tst[threadIdx.x >> 5], *reinterpret_cast<WalkShared *>(s_pst[threadIdx.x >> 5]), o, d,
+            if (!world_walk<K, CHK>(W, valid, s_tst[threadIdx.x >> 5], *reinterpret_cast<WalkShared *>(s_pst[threadIdx.x >> 5]), o, d,
                                inv, tn, tf, (uint32_t)slot, n_ev, kb, cut, lim, lane_ok))
                 lane_ok = false;
         } else {
@@ -598,6 +601,7 @@ template <int K>
 int world_launch(const WorldArgs &W, bool instr, bool walk, int blocks, cudaStream_t s)
 {
     if (instr) k_trace_world<K, true, false><<<blocks, kBlock, 0, s>>>(W);
+    else if (walk && K == kCheckK && W.a.check) k_trace_world<K, false, true, K == kCheckK><<<blocks, kBlock, 0, s>>>(W);
     else if (walk) k_trace_world<K, false, true><<<blocks, kBlock, 0, s>>>(W);
     else k_trace_world<K, false, false><<<blocks, kBlock, 0, s>>>(W);
     return cudaGetLastError() == cudaSuccess ? GRTX_OK : GRTX_ERR_CUDA;
@@ -773,8 +777,8 @@ extern "C" GRTX_API int grtx_world_update(grtx_world *w, const grtx_instance *in
     return world_set(w, inst, n, reinterpret_cast<cudaStream_t>(stream));
 }
 
-extern "C" GRTX_API int grtx_world_trace_forward(grtx_world *w, const grtx_camera *cam, const grtx_params *p,
-                                                 const grtx_trace_outputs *out, void *stream)
+static int world_trace(grtx_world *w, const grtx_camera *cam, const grtx_params *p, const grtx_trace_outputs *out,
+                       uint64_t *d_errors, void *stream)
 {
     if (!w) return grtx_fail(GRTX_ERR_INVALID_ARG, "world is NULL");
     int st = grtx_check_params(p);
@@ -791,6 +795,7 @@ extern "C" GRTX_API int grtx_world_trace_forward(grtx_world *w, const grtx_camer
         return grtx_fail(GRTX_ERR_INVALID_ARG, "visit logs are not available for worlds (node indices of the levels collide)");
     WorldArgs W = {};
     TraceArgs &a = W.a;
+    a.check = reinterpret_cast<unsigned long long *>(d_errors);
     st = grtx_fill_camera(a.cam, a.n_items, cam);
     if (st) return st;
     a.traversal = p->traversal;
@@ -861,6 +866,23 @@ extern "C" GRTX_API int grtx_world_trace_forward(grtx_world *w, const grtx_camer
         return grtx_cuda_fail(e == cudaSuccess ? cudaErrorLaunchFailure : e, "world trace launch");
     }
     return GRTX_OK;
+}
+
+extern "C" GRTX_API int grtx_world_trace_forward(grtx_world *w, const grtx_camera *cam, const grtx_params *p,
+                                                 const grtx_trace_outputs *out, void *stream)
+{
+    return world_trace(w, cam, p, out, nullptr, stream);
+}
+
+extern "C" GRTX_API int grtx_world_self_check(grtx_world *w, const grtx_camera *cam, const grtx_params *p, float *d_rgbT,
+                                              uint64_t *d_errors, void *stream)
+{
+    if (!p || p->traversal != GRTX_TRAVERSAL_CHECKPOINT || p->k != kCheckK)
+        return grtx_fail(GRTX_ERR_INVALID_ARG, "checked walks: checkpoint traversal, k = 16");
+    if (!d_errors) return grtx_fail(GRTX_ERR_INVALID_ARG, "d_errors is NULL");
+    grtx_trace_outputs out = {};
+    out.rgbT = d_rgbT;
+    return world_trace(w, cam, p, &out, d_errors, stream);
 }
 
 extern "C" GRTX_API void grtx_world_destroy(grtx_world *w)

@@ -199,6 +199,8 @@ _SIGS = {
     "grtx_template_mesh": (C.c_int, [C.c_int, _fp, C.POINTER(C.c_int)]),
     "grtx_world_create": (C.c_int, [C.POINTER(grtx_instance), C.c_int, _fp, C.POINTER(_fp)]),
     "grtx_world_update": (C.c_int, [_fp, C.POINTER(grtx_instance), C.c_int, _fp]),
+    "grtx_trace_self_check": (C.c_int, [_fp, C.POINTER(grtx_camera), C.POINTER(grtx_params), _fp, C.c_int64, _fp, _fp]),
+    "grtx_world_self_check": (C.c_int, [_fp, C.POINTER(grtx_camera), C.POINTER(grtx_params), _fp, _fp, _fp]),
     "grtx_world_trace_forward": (C.c_int, [_fp, C.POINTER(grtx_camera), C.POINTER(grtx_params),
                                            C.POINTER(grtx_trace_outputs), _fp]),
     "grtx_world_destroy": (None, [_fp]),
@@ -511,6 +513,16 @@ def grtx_world_update(world: int, placements, stream=None):
     arr = make_instances(placements)
     check(lib().grtx_world_update(C.c_void_p(world), arr, len(list(placements)), stream_handle(stream)),
           "grtx_world_update")
+
+
+def grtx_trace_self_check(scene: int, cam: grtx_camera, p: grtx_params, rgbT, errors, max_nodes: int = 0, stream=None):
+    check(lib().grtx_trace_self_check(C.c_void_p(scene), C.byref(cam), C.byref(p), ptr(rgbT), int(max_nodes), ptr(errors),
+                                      stream_handle(stream)), "grtx_trace_self_check")
+
+
+def grtx_world_self_check(world: int, cam: grtx_camera, p: grtx_params, rgbT, errors, stream=None):
+    check(lib().grtx_world_self_check(C.c_void_p(world), C.byref(cam), C.byref(p), ptr(rgbT), ptr(errors),
+                                      stream_handle(stream)), "grtx_world_self_check")
 
 
 def grtx_world_trace_forward(world: int, cam: grtx_camera, p: grtx_params, rgbT, n_blended=None, blended_ids=None,
