@@ -133,3 +133,48 @@ def test_restart_fills_the_multiprocessors(entry):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     assert sc.info()["bytes_workspace"] >= 6 * sms * 128 * 3 * 8
     sc.close()
+
+
+@pytest.fixture(scope="module")
+def big():
+    """2^24 + 77 faint Gaussians in a box, about 150 hits a ray: too many leaf slots for a list entry that holds a
+    slot and an opacity code."""
+    n = (1 << 24) + 77
+    gen = torch.Generator("cuda").manual_seed(9)
+    means = torch.rand((n, 3), generator=gen, device="cuda") * 2 - 1
+    scales = torch.log(torch.rand((n, 3), generator=gen, device="cuda") * 0.002 + 0.0015)
+    q = torch.randn((n, 4), generator=gen, device="cuda")
+    sh = torch.randn((n, 1, 3), generator=gen, device="cuda") * 0.3
+    sc = R.Scene(means, scales, q, torch.full((n,), float(np.log(0.03 / 0.97)), device="cuda"), sh, 0)
+    del means, scales, q, sh
+    assert sc.info()["n_valid"] == n
+    yield sc
+    sc.close()
+    torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("k,opts", [(8, {}), (16, {}), (16, dict(evict_capacity=100)), (8, dict(T_min=0.2))])
+def test_scenes_of_more_slots_than_codes_leave_room_for(big, k, opts):
+    cam = scenes.pinhole_camera(40, 24, (0.1, 0.2, -2.5))
+    same = {a: v for a, v in opts.items() if a == "T_min"}
+    a = R.render(big, cam, k=k, **opts)["rgbT"]
+    b = R.render(big, cam, k=k, traversal="restart", **same)["rgbT"]
+    torch.cuda.synchronize()
+    assert 0.0 < float(b[:, 3].min()) < 0.5
+    np.testing.assert_array_equal(a[:, 3].cpu().numpy(), b[:, 3].cpu().numpy())
+    np.testing.assert_allclose(a.cpu().numpy(), b.cpu().numpy(), rtol=0, atol=1e-5)
+
+
+@pytest.mark.parametrize("k", [8, 16])
+def test_worlds_of_more_slots_than_codes_leave_room_for(big, k):
+    small = R.Scene.from_params(scenes.surface_scene(n=3000, seed=5, n_spheres=4, n_patches=4))
+    M = np.eye(4)[:3]
+    world = R.World([(big, M), (small, M + [[0, 0, 0, 0.5]] * 3)])
+    cam = scenes.pinhole_camera(40, 24, (0.1, 0.2, -2.5))
+    a = R.render_world(world, cam, k=k)["rgbT"]
+    b = R.render_world(world, cam, k=k, traversal="restart")["rgbT"]
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(a[:, 3].cpu().numpy(), b[:, 3].cpu().numpy())
+    np.testing.assert_allclose(a.cpu().numpy(), b.cpu().numpy(), rtol=0, atol=1e-5)
+    world.close()
+    small.close()
