@@ -1867,6 +1867,7 @@ __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc
                                           int r1_n_dst = 0, int r1_n_ev = 0, float lim = INFINITY)
 {
     constexpr bool BWD = PASS == PASS_BWD;
+    constexpr bool WIDE = FORM == FORM_SPHERE4 || FORM == FORM_SPHERE4Q;
     const uint32_t S = (uint32_t)a.n_slots;
     float3 inv = make_float3(safe_rcp(d.x), safe_rcp(d.y), safe_rcp(d.z));
     const float inv_len = rsqrtf(d.x * d.x + d.y * d.y + d.z * d.z);
@@ -1894,7 +1895,9 @@ __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc
     // The lanes of `live` (the caller's mask of this call) meet at each round, and a lane that restarts runs
     // the same code as the others: each lane's round is a loop of its own, and lanes that are not made to meet
     // run the rounds one lane after another (640x360 of 1M Gaussians with eviction lists of 16: 3.5 ms, 5.4
-    // with the restarted round in a copy of its code, 12.6 with neither).
+    // with the restarted round in a copy of its code, 12.6 with neither). Over 4-wide nodes the restarted
+    // round is a copy, before which the lanes meet as well (1M / 6M 1080p frame 9.8 / 16.9 ms; 10.7 / 16.0 in
+    // one copy, 9.8 / 19.5 if they do not meet there).
     for (;;) {
         live = __ballot_sync(live, !done);
         if (done) break;
@@ -1926,16 +1929,21 @@ __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc
             round_ok = trace_round<K, FORM, INSTR>(a, sc, o, d, inv, inv_len, tn, tf, Lt, Li, ckpt, from_root, src, n_src,
                                                    dst, n_dst, ev, n_ev, kb, cut, from_root ? a.window : 0, cnt);
         }
+        if (WIDE) __syncwarp(live);
         if (!round_ok) {
             // a capacity was exceeded: redo this round from the root and stay in restart mode
-            if (INSTR) {
-                cnt.fallbacks++;
-                cnt.rounds--;
-            }
+            if (INSTR) cnt.fallbacks++;
             ckpt = false;
             from_root = true;
-            first_round = false;
-            continue;
+            if (!WIDE) {
+                if (INSTR) cnt.rounds--;
+                first_round = false;
+                continue;
+            }
+            n_ev = 0;
+            kb.clear();
+            trace_round<K, FORM, INSTR>(a, sc, o, d, inv, inv_len, tn, tf, Lt, Li, false, true, src, 0, dst, n_dst, ev, n_ev,
+                                         kb, cut, 0, cnt);
         }
         for (int j = 0; j < kb.n; ++j) {
             uint32_t idx = kb.I(j) >> a.id_shift;
