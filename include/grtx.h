@@ -128,9 +128,10 @@ enum { GRTX_TRAVERSAL_CHECKPOINT = 0, /* resume from checkpointed nodes + evicti
  * GRTX_PACKET_STACK); a packet that would need more falls back to tracing its rays one by
  * one, with the same result. Smaller values exist to exercise that fallback. (The stack holds
  * the far children still pending along the warp's path: 48 entries of 16 bytes per warp, so
- * that with the k-buffer a 128-ray block takes 19 KB of shared memory, and 8 blocks leave
- * the SM a 92 KB L1 instead of 60 KB; no packet overflowed it on the 111-level tree of the
- * 6M outdoor scene.)
+ * that with the k-buffer of k = 16 a 128-ray block takes 19 KB of shared memory, and 8 blocks leave
+ * the SM a 92 KB L1; no packet overflowed it on the 111-level tree of the 6M outdoor scene.) A
+ * walk's stack has four 4-byte entries for each of these; its blocks take 24 KB, and 8 of them leave
+ * a 60 KB L1.
  * bvh_width (the paper traverses a 6-wide BVH, Sec. V-A): 0 or 2, binary nodes; 4, the build
  * of a sphere-form scene also collapses the binary tree into 4-wide nodes (each binary node at
  * even depth becomes a node over its grandchildren, 128 bytes: lo x, lo y, lo z, hi x, hi y,
@@ -197,7 +198,8 @@ typedef struct grtx_camera {
  * capacity and restarted from the root; stack_overflow: traversal stack overflows (never
  * expected: the build rejects trees deeper than the stack); collected: hits appended to the
  * single-round lists (GRTX_TRAVERSAL_SINGLE only); bounds_errors: node, leaf-record or
- * Gaussian indices that the traversal met outside the scene's arrays. The kernels that fill
+ * Gaussian indices that the traversal met outside the scene's arrays (the tile walks of calls
+ * without these outputs: grtx_trace_self_check). The kernels that fill
  * these counters compare each such index with its array's size before the fetch, count one
  * outside and skip it (never expected: every index comes from the scene's own build). */
 typedef struct grtx_stats {

@@ -1,7 +1,9 @@
 // BVH build on the GPU: Gaussian activation and instance transform, Morton codes, an LSD
 // radix sort, the binary radix tree (Karras 2012), bottom-up bounds and node compaction.
-// The paper builds an Embree BVH-6 on the host (Sec. V-A); this build is an LBVH so that the
-// whole build stays on the device.
+// The paper builds an Embree BVH-6 on the host (Sec. V-A); here the tree is clustered bottom-up over the
+// sorted leaves (PLOC, the default) or the radix tree of their codes, so that the whole build stays on
+// the device. The sort is one launch a digit, the clustering one launch a round, and its last rounds
+// one block's.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>

@@ -1,7 +1,10 @@
-// Trace kernels: one thread per ray, persistent warps pulling 8x4-pixel tiles from a queue.
-// Per ray: rounds of {pre-fill the k-buffer from the eviction list; traverse from the root
-// (first round / restart) or from the checkpointed nodes (later rounds); blend the k-buffer
-// in depth order with early termination} (Sec. III-A; Sec. IV-B, Listing 1).
+// Trace kernels: one thread per ray, persistent warps pulling 8x4-pixel tiles, or parts of one, from a
+// queue. Per ray: rounds of {pre-fill the k-buffer from the eviction list; traverse; blend the k-buffer
+// in depth order with early termination} (Sec. III-A; Sec. IV-B, Listing 1). The first round, from the
+// root, is traced for the whole warp: walked for the tile (tile_walk: checkpointed sphere-form traces
+// without optional outputs) or as a packet (packet_round: the other forms, instrumented traces, every
+// round of restart traversal). Later rounds go on from the checkpointed nodes, a ray a lane
+// (trace_round). Rays of bundles that share nothing are walked one to a warp (k_trace_rays).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -1352,7 +1355,7 @@ __device__ __forceinline__ bool packet_round(const TraceArgs &a, const SceneRef 
 // 2.6 G instead of 7.8 G warp instructions a frame. 1920x1080, k = 16: 9.8 ms with packets and
 // per-ray later rounds, 6.8 ms with packets bounded by opacity (Cut), 3.9 ms with the walk, 3.5 with
 // the quadratic filter below, 3.2 with 64-bit keys and 256-bit gathers. What bounds it now: the L1
-// pipe (78 %: each lane gathers its own records and SH coefficients) and instruction issue (65 %).
+// pipe (80 %: each lane gathers its own records and SH coefficients) and instruction issue (68 %).
 // Keeping the hits' alphas instead of testing again at the blend, colours by groups of four lanes, and
 // 5 to 7 blocks an SM with the registers for it were measured: none was faster.
 // Groups of 8 or 16 rays with a stack each took 7.9 and 4.7 ms against 4.0 for one of 32.
@@ -2188,8 +2191,9 @@ __device__ __forceinline__ void discard_dead_lists(const TraceArgs &a, int warp_
 
 // Resident blocks per SM the trace kernels are compiled for. The traversal is latency-bound,
 // so occupancy pays even at the cost of a few spilled registers (measured on GB300: 8 blocks of
-// 128 threads is the best forward setting for k <= 16; the k = 32 k-buffer's 32 KB of shared
-// memory per block allows 6; the backward keeps more live state and prefers 7).
+// 128 threads is the best forward setting for k <= 16; at k = 32 the k-buffer's 32 KB of shared memory
+// allow 6 blocks, and 5 with a walk's 7.4 KB beside it; the backward keeps more live state and
+// prefers 7).
 __host__ __device__ constexpr int trace_min_blocks(int k, bool bwd) { return k >= 32 ? 6 : (bwd ? 7 : 8); }
 
 // The item that queue place `place` of an image stands for: rows of tiles are handed out from the

@@ -4,7 +4,9 @@
 // the k-buffer round loop of the single-scene kernel over this two-level structure: at a TLAS
 // leaf the ray is mapped into the object's frame and descends its BVH, and traversal entries
 // (stack and checkpoint lists) carry the instance of object-level nodes, as the paper's
-// checkpoint entry carries a TLAS-leaf address for BLAS nodes.
+// checkpoint entry carries a TLAS-leaf address for BLAS nodes. Checkpointed traces without optional
+// outputs walk the first round for the tile, object by object (world_walk); restarted and
+// instrumented ones take it as a packet (world_packet_round).
 #include <cuda_runtime.h>
 
 #include <algorithm>
