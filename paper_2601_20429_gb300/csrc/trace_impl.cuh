@@ -1870,7 +1870,6 @@ __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc
                                           int r1_n_dst = 0, int r1_n_ev = 0, float lim = INFINITY)
 {
     constexpr bool BWD = PASS == PASS_BWD;
-    constexpr bool WIDE = FORM == FORM_SPHERE4 || FORM == FORM_SPHERE4Q;
     const uint32_t S = (uint32_t)a.n_slots;
     float3 inv = make_float3(safe_rcp(d.x), safe_rcp(d.y), safe_rcp(d.z));
     const float inv_len = rsqrtf(d.x * d.x + d.y * d.y + d.z * d.z);
@@ -1895,12 +1894,11 @@ __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc
     const uint32_t ev = a.ev_off + (uint32_t)slot;
     bool done = !sc.has_tree;
     bool first_round = true;
-    // The lanes of `live` (the caller's mask of this call) meet at each round, and a lane that restarts runs
-    // the same code as the others: each lane's round is a loop of its own, and lanes that are not made to meet
-    // run the rounds one lane after another (640x360 of 1M Gaussians with eviction lists of 16: 3.5 ms, 5.4
-    // with the restarted round in a copy of its code, 12.6 with neither). Over 4-wide nodes the restarted
-    // round is a copy, before which the lanes meet as well (1M / 6M 1080p frame 9.8 / 16.9 ms; 10.7 / 16.0 in
-    // one copy, 9.8 / 19.5 if they do not meet there).
+    // The lanes of `live` (the caller's mask of this call) meet behind each round's traversal. It has several
+    // ways out, and left to the compiler the lanes that restart, which run a copy of it, may do so one after
+    // another: 640x360 of 1M Gaussians with eviction lists of 16 / 40: 3.38 / 2.68 ms, 5.3 / 3.2 without; 1M / 6M
+    // 1080p frame over 4-wide nodes 9.8 / 16.9 ms, 9.8 / 19.5 without. (In one copy, round the loop again: 3.45 /
+    // 2.76 and 10.7 / 16.0 ms, and small frames at k = 32 5 % slower.)
     for (;;) {
         live = __ballot_sync(live, !done);
         if (done) break;
@@ -1932,17 +1930,12 @@ __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc
             round_ok = trace_round<K, FORM, INSTR>(a, sc, o, d, inv, inv_len, tn, tf, Lt, Li, ckpt, from_root, src, n_src,
                                                    dst, n_dst, ev, n_ev, kb, cut, from_root ? a.window : 0, cnt);
         }
-        if (WIDE) __syncwarp(live);
+        __syncwarp(live);
         if (!round_ok) {
             // a capacity was exceeded: redo this round from the root and stay in restart mode
             if (INSTR) cnt.fallbacks++;
             ckpt = false;
             from_root = true;
-            if (!WIDE) {
-                if (INSTR) cnt.rounds--;
-                first_round = false;
-                continue;
-            }
             n_ev = 0;
             kb.clear();
             trace_round<K, FORM, INSTR>(a, sc, o, d, inv, inv_len, tn, tf, Lt, Li, false, true, src, 0, dst, n_dst, ev, n_ev,
