@@ -1863,7 +1863,9 @@ __device__ __forceinline__ void save_blended(const TraceArgs &a, int64_t pix, in
     if (j < a.save_cap) a.save_leaves[(size_t)pix * a.save_cap + j] = idx;
 }
 
-template <int K, int FORM, bool INSTR, int PASS>
+constexpr int kMeetLists = 64;
+
+template <int K, int FORM, bool INSTR, int PASS, bool MEET = true>
 __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc, float4 *__restrict__ out, int slot,
                                           int64_t pix, float3 o, float3 d, float tn, float tf, KBuf<K> &kb,
                                           Counters &cnt, Cut cut, unsigned live, bool r1_done = false, bool r1_ok = true,
@@ -1898,9 +1900,12 @@ __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc
     // ways out, and left to the compiler the lanes that restart, which run a copy of it, may do so one after
     // another: 640x360 of 1M Gaussians with eviction lists of 16 / 40: 3.38 / 2.68 ms, 5.3 / 3.2 without; 1M / 6M
     // 1080p frame over 4-wide nodes 9.8 / 16.9 ms, 9.8 / 19.5 without. (In one copy, round the loop again: 3.45 /
-    // 2.76 and 10.7 / 16.0 ms, and small frames at k = 32 5 % slower.)
+    // 2.76 and 10.7 / 16.0 ms, and small frames at k = 32 5 % slower.) The frame kernel, whose rays hardly
+    // ever restart with lists of 64 entries or more, leaves it out for these (!MEET): 256x256 preview 554
+    // instead of 561 us, 1080p frame 3.60 instead of 3.62 ms; the server's spills more with the choice.
+    const bool meet = MEET || a.evict_cap < kMeetLists;
     for (;;) {
-        live = __ballot_sync(live, !done);
+        if (meet) live = __ballot_sync(live, !done);
         if (done) break;
         if (INSTR) cnt.rounds++;
         if (!(r1_done && first_round)) kb.clear();
@@ -1930,7 +1935,7 @@ __device__ __forceinline__ void trace_ray(const TraceArgs &a, const SceneRef &sc
             round_ok = trace_round<K, FORM, INSTR>(a, sc, o, d, inv, inv_len, tn, tf, Lt, Li, ckpt, from_root, src, n_src,
                                                    dst, n_dst, ev, n_ev, kb, cut, from_root ? a.window : 0, cnt);
         }
-        __syncwarp(live);
+        if (meet) __syncwarp(live);
         if (!round_ok) {
             // a capacity was exceeded: redo this round from the root and stay in restart mode
             if (INSTR) cnt.fallbacks++;
@@ -2076,7 +2081,7 @@ __device__ __forceinline__ void trace_warp_restart(const TraceArgs &a, const Sce
 // own. Every lane of the warp calls this together; lanes without a ray pass valid = false. In
 // the backward, a ray whose forward saved its whole blend list takes it from there and leaves
 // the traversal to the others.
-template <int K, int FORM, bool INSTR, int PASS, bool WALK_ONLY = false, bool CHK = false>
+template <int K, int FORM, bool INSTR, int PASS, bool WALK_ONLY = false, bool CHK = false, bool MEET = true>
 __device__ __forceinline__ void trace_warp(const TraceArgs &a, const SceneRef &sc, float4 *__restrict__ out, int slot,
                                            bool valid, int64_t pix, float3 o, float3 d, float tn, float tf, KBuf<K> &kb,
                                            Counters &cnt, uint4 *pst)
@@ -2140,7 +2145,7 @@ __device__ __forceinline__ void trace_warp(const TraceArgs &a, const SceneRef &s
     }
     const unsigned rays = __ballot_sync(0xffffffffu, valid);
     if (valid)
-        trace_ray<K, FORM, INSTR, PASS>(a, sc, out, slot, pix, o, d, tn, tf, kb, cnt, cut, rays, !WALKS || lane_ok, WALKS || lane_ok,
+        trace_ray<K, FORM, INSTR, PASS, MEET>(a, sc, out, slot, pix, o, d, tn, tf, kb, cnt, cut, rays, !WALKS || lane_ok, WALKS || lane_ok,
                                         n_dst, n_ev, lim);
 }
 
@@ -2268,7 +2273,7 @@ __global__ void __launch_bounds__(kBlock, trace_min_blocks(K, PASS == PASS_BWD))
             trace_warp_restart<K, FORM, INSTR, PASS == PASS_SAVE>(a, a.sc, a.rgbT, slot, valid, pix, o, d, tn, tf,
                                                                   kb, cnt, s_pst[threadIdx.x >> 5]);
         else if constexpr (TRAV == TRAV_CKPT || TRAV == TRAV_CHECK)
-            trace_warp<K, FORM, INSTR, PASS, true, TRAV == TRAV_CHECK>(a, a.sc, a.rgbT, slot, valid, pix, o, d, tn, tf, kb, cnt,
+            trace_warp<K, FORM, INSTR, PASS, true, TRAV == TRAV_CHECK, false>(a, a.sc, a.rgbT, slot, valid, pix, o, d, tn, tf, kb, cnt,
                                              s_pst[threadIdx.x >> 5]);
         else if (PASS != PASS_BWD && a.traversal == GRTX_TRAVERSAL_RESTART)
             trace_warp_restart<K, FORM, INSTR, PASS == PASS_SAVE>(a, a.sc, a.rgbT, slot, valid, pix, o, d, tn, tf,
