@@ -469,7 +469,7 @@ extern "C" GRTX_API int grtx_trace_forward_batch(grtx_scene *sc, const grtx_came
     bool ckpt = a.traversal == GRTX_TRAVERSAL_CHECKPOINT;
     // Short ray lists go in bundles of 16 or 8 rays: bounce rays share little, and a wide bundle of 32
     // holds its warp longer than the rest of the launch takes (6 M Gaussians at 1080p with 70,354 bounce
-    // rays in one launch: 13.6 ms in bundles of 32, 9.5 ms so). Not where the launch has fewer tiles
+    // rays in one launch: 13.6 ms in bundles of 32, 9.5 ms so; scenes differ, and from run to run). Not where the launch has fewer tiles
     // than warps: there the whole tiles of the image take as long, beside more bundles (a small image
     // with its bounce rays: 233 us, 248 us with the split).
     const unsigned warps = (unsigned)blocks * (kBlock / 32);
